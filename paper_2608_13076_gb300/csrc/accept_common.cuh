@@ -51,13 +51,13 @@ struct Call {
   int32_t *status;
   const float *temperature;  // [B] softmax temperature of each sequence, or null (all 1)
   const float *top_p;        // [B] nucleus mass of each sequence, or null (no truncation)
-  unsigned *bar;     // barrier words (kBarBytes), zero between calls but for generations
+  unsigned *bar;     // grid barrier words (kBarBytes)
   float4 *pstat;     // [R][NC]: slice max, slice sum-exp, slice argmax (bits), -
   float *ldraft;     // [R]: logit of the row's draft token
   float4 *gstat;     // [R]: merged row max, sum-exp, argmax (bits), accept bit
   float *logits;     // [R][ldl]: logits of the rows of sampled sequences (before temperature)
-  float2 *zpart;     // [2 attempts][B][kMaxGroup]: share masses of the sampled distribution (float-float)
-  unsigned *nhist;   // [2][kMaxGroup][R][kNucBins]: bin masses of the nucleus search (2^31 = all of p)
+  unsigned long long *zpart;  // [2 attempts][B][kMaxGroup]: share masses of the sampled distribution (float-float)
+  unsigned *nhist;   // [kNucRounds][kMaxGroup][R][kNucBins]: bin masses of the nucleus search (2^31 = all of p)
   // Fused KV commit (null kc: not requested): clear the rejected draft slots of
   // the caches [B, Hkv, cap, Dk] and advance ctx_lens once the decisions exist.
   uint4 *kc, *vc;
@@ -72,6 +72,7 @@ struct Call {
   int NC;    // vocabulary slices (CTAs of the statistics phase)
   int ldl;   // floats per logits row, a multiple of 4
   int qvec;  // draft_probs rows may be read as float4 (16-byte aligned rows)
+  int pool;  // bytes of RowsSmem::pool (nucleus search)
 };
 
 // bar.sync is the aligned form: every lane of a warp must arrive together.
@@ -92,15 +93,32 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
   return v;
 }
 
+__device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long *p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(unsigned *p, unsigned v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed64(unsigned long long *p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 // Barrier words: the grid barrier's arrival count at word 0 and its generation
 // in kReplicas copies, a 128-byte line each (CTA c polls copy c % kReplicas:
-// 152 CTAs polling one line queue on it); then one (count, generation) pair of
-// lines per group of CTAs that draws a token together.
+// 152 CTAs polling one line queue on it).
 constexpr int kReplicas = 8;
 constexpr int kGenWord = 32;
-constexpr int kGroupWord = 512;
-constexpr int kBarBytes = kGroupWord * 4 + kMaxNC * 2 * kGenWord * 4;
-static_assert(kGenWord * (kReplicas + 1) <= kGroupWord, "grid barrier words fit their region");
+constexpr int kBarBytes = 2048;
+static_assert(kGenWord * (kReplicas + 1) * 4 <= kBarBytes, "barrier words fit their region");
+// Words that the CTAs of a group exchange (share masses, nucleus bins) are set to
+// all ones before the statistics end; a reader polls the word itself until its
+// writer has replaced it, so an exchange costs one store and one load through
+// L2 (a barrier beside it: an atomic, a generation bump and a poll as well;
+// 2.8 us against 1.3).
+constexpr unsigned kUnset = 0xffffffffu;
+constexpr unsigned long long kUnset64 = 0xffffffffffffffffull;
 constexpr int kNucBinBits = 5;                 // key bits decided per round of the nucleus search
 constexpr int kNucBins = 1 << kNucBinBits;     // bins per round
 constexpr int kNucRounds = 4;                  // all 20 key bits, see nuc_key
@@ -206,15 +224,10 @@ __device__ __forceinline__ bool ff_gt(ff2 a, ff2 b) {
 __device__ __forceinline__ ff2 ff_shfl(ff2 v, int src) {
   return ff2{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
 }
-__device__ __forceinline__ ff2 warp_sum_ff(ff2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    v = ff_add(v, ff2{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
-  return ff_shfl(v, 0);  // one value for every lane
-}
-// Inclusive prefix sum over the warp's lanes.
-__device__ __forceinline__ ff2 warp_scan_ff(ff2 v, int lane) {
-#pragma unroll
+// Inclusive prefix sum over the warp's lanes.  (Rolled, one copy: the rows phase
+// runs once after a long stream, and its cost is largely instruction fetch.)
+static __device__ __noinline__ ff2 warp_scan_ff(ff2 v, int lane) {
+#pragma unroll 1
   for (int o = 1; o < 32; o <<= 1) {
     const ff2 t{__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
     if (lane >= o) v = ff_add(t, v);
@@ -222,47 +235,35 @@ __device__ __forceinline__ ff2 warp_scan_ff(ff2 v, int lane) {
   return v;
 }
 
-// Arrival at a barrier of n CTAs (one thread, after a CTA barrier that orders
-// the CTA's writes before it): the last arrival resets the count and bumps the
-// generation words.  Returns the generation seen before arriving; *last: this
-// arrival completed the barrier and there is nothing to wait for.
-__device__ __forceinline__ unsigned bar_arrive(unsigned *count, unsigned *gen, int copies, int my_copy, int n,
-                                               bool *last) {
-  const unsigned seen = ld_relaxed(gen + kGenWord * my_copy);  // before arriving (the release orders it first)
-  unsigned arrived;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(count) : "memory");
-  *last = arrived == static_cast<unsigned>(n) - 1;
-  if (*last) {
-    asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(count) : "memory");
-    // One release fence orders everything above before all the copies.
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    for (int r = 0; r < copies; ++r)
-      asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(gen + kGenWord * r) : "memory");
-  }
-  return seen;
-}
-// Bounded poll for a generation newer than `seen` (one thread).
-__device__ __forceinline__ bool bar_poll(const unsigned *gen_p, unsigned seen) {
-  bool ok = true;
-  const uint64_t t0 = globaltimer();
-  while (ld_relaxed(gen_p) == seen) {
-    if (globaltimer() - t0 > kWaitLimitNs) { ok = false; break; }
-    __nanosleep(20);
-  }
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
-  return ok;
-}
-
-// Device-wide barrier among the nctas co-resident CTAs (cooperative launch).
-// Returns false if the wait expired.
+// Device-wide barrier among the nctas co-resident CTAs (cooperative launch).  The
+// last CTA to arrive resets the count and bumps the generation copies; the
+// others poll theirs (relaxed loads with a short back-off, then an acquire
+// fence) with a time limit.  Returns false if the wait expired.
 __device__ __forceinline__ bool grid_barrier(unsigned *bar, int nctas) {
   __shared__ int s_ok;
   block_sync();
   if (threadIdx.x == 0) {
-    bool last;
-    const int copy = blockIdx.x % kReplicas;
-    const unsigned seen = bar_arrive(bar, bar + kGenWord, kReplicas, copy, nctas, &last);
-    s_ok = last || bar_poll(bar + kGenWord * (1 + copy), seen);
+    s_ok = 1;
+    unsigned *gen_p = bar + kGenWord * (1 + blockIdx.x % kReplicas);
+    // Read before arriving (the arrival's release orders this load first).
+    const unsigned gen = ld_relaxed(gen_p);
+    unsigned arrived;
+    // The arrival releases this CTA's writes (ordered before it by bar.sync).
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(bar) : "memory");
+    if (arrived == static_cast<unsigned>(nctas) - 1) {
+      st_relaxed(bar, 0u);
+      // One release fence orders everything above before all the copies.
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      for (int r = 0; r < kReplicas; ++r)
+        asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(bar + kGenWord * (1 + r)) : "memory");
+    } else {
+      const uint64_t t0 = globaltimer();
+      while (ld_relaxed(gen_p) == gen) {
+        if (globaltimer() - t0 > kWaitLimitNs) { s_ok = 0; break; }
+        __nanosleep(20);
+      }
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    }
   }
   block_sync();
   return s_ok != 0;
@@ -285,31 +286,95 @@ __device__ __forceinline__ SeqInfo seq_info(const Call &p, int b) {
   return q;
 }
 
-// Per-row tables of the statistics epilogue (the epilogue warps, thread et of
-// kEpiThreads, while the first stages already stream): draft token (-1: none), 1 / T, and which rows' logits
-// are kept for the draw (bit n % 16 of word n / 16).  Row n = cu_q[b] + i is
-// position i of sequence b; it holds draft i for i < k_b.  nrows: a multiple
-// of 16 that covers the rows.
-__device__ __forceinline__ void setup_rows(const Call &p, int nrows, int32_t *s_draft, float *s_it, unsigned *s_keep,
-                                           int et) {
-  for (int n = et; n < nrows; n += kEpiThreads) { s_draft[n] = -1; s_it[n] = 1.f; }
-  for (int w = et; w < nrows / kBlk; w += kEpiThreads) s_keep[w] = 0u;
-  named_bar(1, kEpiThreads);
-  for (int b = et; b < p.B; b += kEpiThreads) {
-    const SeqInfo q = seq_info(p, b);
-    if (!q.valid) {
-      atomicOr(p.status, SPADE_DEV_BAD_INDEX);
-      continue;
+// Every sequence's rows and kind, in shared memory for the whole call.
+struct SeqTable {
+  int r0[kMaxB], k[kMaxB];
+  unsigned valid[kMaxB / 32], stoch[kMaxB / 32];
+};
+__device__ __forceinline__ SeqInfo table_info(const SeqTable &t, int b) {
+  const unsigned bit = 1u << (b % 32);
+  return SeqInfo{t.r0[b], t.k[b], (t.valid[b / 32] & bit) != 0u, (t.stoch[b / 32] & bit) != 0u};
+}
+// Warp w of nw fills the words w, w + nw, ... (32 sequences each).
+__device__ __forceinline__ void fill_table(const Call &p, SeqTable &t, int w, int nw, int lane, bool report) {
+  for (int b0 = 32 * w; b0 < p.B; b0 += 32 * nw) {
+    const int b = b0 + lane;
+    SeqInfo q{0, 0, false, false};
+    if (b < p.B) {
+      q = seq_info(p, b);
+      t.r0[b] = q.r0;
+      t.k[b] = q.k;
+      if (!q.valid && report) atomicOr(p.status, SPADE_DEV_BAD_INDEX);
     }
-    const float it = inv_temp(p, b);
-    for (int i = 0; i <= q.k; ++i) {
-      const int n = q.r0 + i;
-      s_it[n] = it;
-      if (i < q.k) s_draft[n] = p.draft_tokens[n - b];
-      if (q.stoch) atomicOr(&s_keep[n / kBlk], 1u << (n % kBlk));
+    const unsigned mv = __ballot_sync(0xffffffffu, q.valid), ms = __ballot_sync(0xffffffffu, q.stoch);
+    if (lane == 0) {
+      t.valid[b0 / 32] = mv;
+      t.stoch[b0 / 32] = ms;
+    }
+  }
+}
+
+// Per-row tables of the statistics epilogue, `nrows` entries each (a multiple of
+// 16): row n = cu_q[b] + i is position i of sequence b; it holds draft i for i < k_b.
+struct RowTables {
+  int32_t *draft;   // draft token, -1: none
+  float *it;        // 1 / T
+  unsigned *keep;   // [nrows / 16]: bit n % 16 of word n / 16: the row's logits are kept for the draw
+  float *u, *q;     // uniform and q(draft), or null: read by the rows phase itself
+};
+__host__ __device__ constexpr int row_table_bytes(int nrows, bool uq) {
+  return nrows * (uq ? 16 : 8) + nrows / kBlk * 4;
+}
+__device__ __forceinline__ RowTables row_tables(uint8_t *mem, int nrows, bool uq) {
+  RowTables t;
+  t.draft = reinterpret_cast<int32_t *>(mem);
+  t.it = reinterpret_cast<float *>(t.draft + nrows);
+  t.u = uq ? t.it + nrows : nullptr;
+  t.q = uq ? t.u + nrows : nullptr;
+  t.keep = reinterpret_cast<unsigned *>((uq ? t.q : t.it) + nrows);
+  return t;
+}
+// Filled by the epilogue warps (thread et of kEpiThreads) while the first
+// stages already stream.
+__device__ __forceinline__ void setup_rows(const Call &p, int nrows, SeqTable &seqs, const RowTables &t, int et) {
+  for (int n = et; n < nrows; n += kEpiThreads) { t.draft[n] = -1; t.it[n] = 1.f; }
+  for (int w = et; w < nrows / kBlk; w += kEpiThreads) t.keep[w] = 0u;
+  fill_table(p, seqs, et / 32, kEpiWarps, et % 32, true);
+  named_bar(1, kEpiThreads);
+  // The rows' sequences (one warp per sequence), then one thread per row, so
+  // that the loads of all rows are in flight together.
+  for (int b = et / 32; b < p.B; b += kEpiWarps) {
+    const SeqInfo q = table_info(seqs, b);
+    if (!q.valid) continue;
+    for (int i = et % 32; i <= q.k; i += 32) t.draft[q.r0 + i] = b;
+  }
+  named_bar(1, kEpiThreads);
+  for (int n = et; n < p.R; n += kEpiThreads) {
+    const int b = t.draft[n];
+    if (b < 0) continue;
+    const SeqInfo q = table_info(seqs, b);
+    const int d = n - q.r0 < q.k ? p.draft_tokens[n - b] : -1;
+    t.it[n] = inv_temp(p, b);
+    t.draft[n] = d;
+    if (q.stoch) atomicOr(&t.keep[n / kBlk], 1u << (n % kBlk));
+    if (t.u) {
+      t.u[n] = p.uniforms[n];
+      t.q[n] = q.stoch && d >= 0 && d < p.V ? __ldg(&p.draft_probs[static_cast<size_t>(n - b) * p.V + d]) : 0.f;
     }
   }
   named_bar(1, kEpiThreads);
+}
+
+// Sets the words that the rows phase's groups exchange to unset (thread i of n
+// of the statistics launch; ordered before the rows phase by the grid barrier
+// or the launch's end).
+__device__ __forceinline__ void clear_exchange(const Call &p, int i, int n) {
+  for (int e = i; e < 2 * p.B * kMaxGroup; e += n) p.zpart[e] = kUnset64;
+  if (p.top_p != nullptr) {
+    uint4 *h = reinterpret_cast<uint4 *>(p.nhist);
+    const int words = kNucRounds * kMaxGroup * p.R * (kNucBins / 4);
+    for (int e = i; e < words; e += n) h[e] = make_uint4(kUnset, kUnset, kUnset, kUnset);
+  }
 }
 
 // Running statistics of a block's 16 rows over the entries one warp has seen:
@@ -331,15 +396,16 @@ __device__ __forceinline__ void blk_init(BlkStat &st, int lane) {
 // shared-memory transpose gives lane (row = lane % 16, half = lane / 16) one
 // row over 16 entries, reduced serially; the two halves meet by a shuffle each
 // for the maximum and the sum.  The argmax search runs only when the block
-// raises a row's running maximum.  Rows whose bit is set in `keep` also store
+// raises a row's running maximum.  Rows marked in `rows.keep` also store
 // their logits, 128 contiguous bytes per row and warp.
-__device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0, int v0, int v_hi, unsigned keep,
-                                           const int32_t *s_draft, const float *s_it, float *T, int lane, BlkStat &st) {
+__device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0, int v0, int v_hi, const RowTables &rows,
+                                           float *T, int lane, BlkStat &st) {
   uint32_t raw[kBlk];
   tmem_ld8(taddr, raw);
   tmem_ld8(taddr + 8, raw + 8);
   tmem_wait_ld();
   const bool mine = v0 + lane < v_hi;  // lanes past the slice are masked
+  const unsigned keep = rows.keep[r0 / kBlk];
   if (keep != 0u) {
     float *dst = p.logits + static_cast<size_t>(r0) * p.ldl + v0 + lane;
 #pragma unroll
@@ -353,7 +419,7 @@ __device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0
   __syncwarp();
   const int row = lane % kBlk, vb = (lane / kBlk) * kBlk;  // 16 entries from v0 + vb on
   const int n = r0 + row;
-  const float it = s_it[n];  // logits at the row's temperature, l / T
+  const float it = rows.it[n];  // logits at the row's temperature, l / T
   const float rm = st.m[row];
   float x[kBlk];
   float m = -INFINITY;
@@ -389,7 +455,7 @@ __device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0
       st.i[row] = idx;
     }
   }
-  const int d = s_draft[n] - (v0 + vb);
+  const int d = rows.draft[n] - (v0 + vb);
   if (d >= 0 && d < kBlk && v0 + vb + d < v_hi) p.ldraft[n] = __fmul_rn(T[(vb + d) * kTStride + row], it);
   __syncwarp();
 }
@@ -410,51 +476,78 @@ __device__ __forceinline__ void publish_slice(const Call &p, const BlkStat *stat
 }
 
 // Shared memory of the rows phase.
+constexpr int kPiece = 8192;       // entries of a share that the draw holds in shared memory at once
+constexpr int kMaxPieces = 80;     // 622592 entries, the largest vocabulary
 struct RowsSmem {
-  int n_st, n_gr, first, nl, owner, owner_warp, last, retry;
-  unsigned gen;
-  int abort;
-  ff2 tgt, wtgt;
-  ff2 wm[kWarps];        // masses of the warps' parts of this CTA's share
+  uint64_t bar;          // bulk copies of a piece
+  int n_st, n_gr, first, nl, owner_piece, owner_warp, retry, abort;
+  ff2 tgt, before;
+  ff2 pm[kMaxPieces][kWarps];  // masses of the warps' parts of each piece of this CTA's share
   int st[kMaxB];         // sampled sequences, ascending
   int gr[kMaxB];         // greedy and invalid ones
   float m[kMaxR], z[kMaxR];           // rows of the sequence at hand: maximum, sum of exponentials
   float u[kMaxR], q[kMaxR], l[kMaxR]; // uniform, q(draft), draft logit
   int arg[kMaxR], d[kMaxR], ok[kMaxR];
   int tkey[kMaxR];       // nucleus key threshold (INT_MIN: all of p)
+  union alignas(16) {
+    struct {
+      float l[kPiece], q[kPiece];     // the piece's logits (then its terms) and draft distribution
+    } piece;
+    float bins[kWarps][kNucSubs * kNucBins * 32];  // nucleus search
+  };
   // Nucleus search only (one-launch path, at most 256 rows):
   int npre[kMaxRes];
   unsigned nab[kMaxRes];
-  unsigned hist[kMaxRes][kNucBins];
-  float bins[kWarps][kNucSubs * kNucBins * 32];
+  // Call::pool bytes: unsigned hist[rows][kNucBins], uint16_t cnt[items][32]
+  // (list lengths per item and lane), float list[items][entries][32].
+  uint8_t pool[16];
 };
-constexpr size_t kRowsBytesPlain = offsetof(RowsSmem, npre);
+constexpr size_t kRowsBytesPlain = offsetof(RowsSmem, piece) + 2 * kPiece * sizeof(float);
+static_assert(offsetof(RowsSmem, piece) % 16 == 0, "bulk copies need 16-byte alignment");
+constexpr int kPoolPerRow = kNucBins * 4 + 32 * 2;  // bins and list lengths of one searched row
 
-// Barrier of the gs CTAs of group g, split so that work that needs no other
-// CTA can run between the two halves.
-__device__ __forceinline__ void group_arrive(const Call &p, RowsSmem &s, int g, int gs) {
-  block_sync();
-  if (gs > 1 && threadIdx.x == 0) {
-    unsigned *count = p.bar + kGroupWord + g * 2 * kGenWord;
-    bool last;
-    s.gen = bar_arrive(count, count + kGenWord, 1, 0, gs, &last);
-    s.last = last;
+// Bounded poll of an exchanged word until its writer has set it.  After an
+// expired wait of the CTA every later poll gives up at once.
+__device__ __forceinline__ unsigned poll_word(const Call &p, RowsSmem &s, const unsigned *a) {
+  unsigned v = ld_relaxed(a);
+  if (v != kUnset) return v;
+  const uint64_t t0 = globaltimer();
+  while ((v = ld_relaxed(a)) == kUnset) {
+    if (*const_cast<volatile int *>(&s.abort)) return 0u;
+    if (globaltimer() - t0 > kWaitLimitNs) {
+      *const_cast<volatile int *>(&s.abort) = 1;
+      atomicOr(p.status, SPADE_DEV_TIMEOUT);
+      return 0u;
+    }
   }
+  return v;
 }
-__device__ __forceinline__ void group_wait(const Call &p, RowsSmem &s, int g, int gs) {
-  if (gs > 1 && threadIdx.x == 0 && !s.last && !s.abort &&
-      !bar_poll(p.bar + kGroupWord + g * 2 * kGenWord + kGenWord, s.gen)) {
-    atomicOr(p.status, SPADE_DEV_TIMEOUT);
-    s.abort = 1;
+__device__ __forceinline__ ff2 poll_mass(const Call &p, RowsSmem &s, const unsigned long long *a) {
+  unsigned long long v = ld_relaxed64(a);
+  if (v == kUnset64) {
+    const uint64_t t0 = globaltimer();
+    while ((v = ld_relaxed64(a)) == kUnset64) {
+      if (*const_cast<volatile int *>(&s.abort)) return ff2{0.f, 0.f};
+      if (globaltimer() - t0 > kWaitLimitNs) {
+        *const_cast<volatile int *>(&s.abort) = 1;
+        atomicOr(p.status, SPADE_DEV_TIMEOUT);
+        return ff2{0.f, 0.f};
+      }
+    }
   }
-  block_sync();
+  return ff2{__uint_as_float(static_cast<unsigned>(v)), __uint_as_float(static_cast<unsigned>(v >> 32))};
+}
+__device__ __forceinline__ void post_mass(unsigned long long *a, ff2 z) {
+  // (a NaN mass must not read as unset: lo is then zero)
+  const unsigned lo = z.lo == z.lo ? __float_as_uint(z.lo) : 0u;
+  st_relaxed64(a, static_cast<unsigned long long>(lo) << 32 | __float_as_uint(z.hi));
 }
 
 // Merged statistics and accept bits of the rows of sequence b, one warp per
 // row over the NC slice partials.  Greedy: the draft is the argmax (lowest
 // index on ties); stochastic: u < p(d) / q(d) (Sec. III-C).
-__device__ __forceinline__ void decide_rows(const Call &p, RowsSmem &s, int b, const SeqInfo &q, bool writer, int warp,
-                                            int lane) {
+__device__ __forceinline__ void decide_rows(const Call &p, RowsSmem &s, const RowTables &rows, int b, const SeqInfo &q,
+                                            bool writer, int warp, int lane) {
   constexpr int kLoads = kMaxNC / 32;
 #pragma unroll 1
   for (int i = warp; i <= q.k; i += kWarps) {
@@ -469,23 +562,37 @@ __device__ __forceinline__ void decide_rows(const Call &p, RowsSmem &s, int b, c
     int d = -1;
     float u = 0.f, qd = 0.f, ld = 0.f;
     if (i < q.k) {
-      d = p.draft_tokens[n - b];
-      u = p.uniforms[n];
-      if (d >= 0 && d < p.V) {
+      if (rows.u) {  // read while the vocabulary streamed
         ld = __ldcg(&p.ldraft[n]);
-        if (q.stoch) qd = __ldg(&p.draft_probs[static_cast<size_t>(n - b) * p.V + d]);
+        d = rows.draft[n];
+        u = rows.u[n];
+        qd = rows.q[n];
+      } else {
+        d = p.draft_tokens[n - b];
+        ld = __ldcg(&p.ldraft[n]);
+        u = p.uniforms[n];
+        if (q.stoch && d >= 0 && d < p.V) qd = __ldg(&p.draft_probs[static_cast<size_t>(n - b) * p.V + d]);
       }
     }
-    float m = -INFINITY, z = 0.f;
+    // The maximum first, then its lowest index and the rescaled sum.
+    float m = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < kLoads; ++j) m = fmaxf(m, part[j].x);
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float z = 0.f;
     int idx = INT_MAX;
+    if (m != -INFINITY) {
 #pragma unroll
-    for (int j = 0; j < kLoads; ++j) stat_merge(m, z, idx, part[j].x, part[j].y, __float_as_int(part[j].z));
-#pragma unroll
+      for (int j = 0; j < kLoads; ++j) {
+        z += part[j].y * ex2((part[j].x - m) * kLog2e);
+        if (part[j].x == m) idx = min(idx, __float_as_int(part[j].z));
+      }
+    }
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, m, o);
-      const float oz = __shfl_xor_sync(0xffffffffu, z, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-      stat_merge(m, z, idx, om, oz, oi);
+      z += __shfl_xor_sync(0xffffffffu, z, o);
+      idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, o));
     }
     if (lane == 0) {  // lane 0's values are everyone's
       int ok = 0;
@@ -575,6 +682,32 @@ __device__ __forceinline__ void share_of(int V, int gs, int rank, int *lo, int *
   *hi = min(V, *lo + per);
 }
 
+// Adds four values of a row to a lane's bins.  `v` holds scaled logits; a value
+// counts when `in` says so and its key has the prefix bits.
+struct BinRound {
+  float nb65, mlog;
+  int sh, pre_bits;
+};
+__device__ __forceinline__ void bin4(const BinRound &t, float *bins, const float (&l)[4], const bool (&in)[4]) {
+  float ex[4];
+  int a[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int kbits = nuc_key_bits(l[c], t.nb65);
+    const bool hit = in[c] && (kbits >> (t.sh + kNucBinBits)) == t.pre_bits;
+    ex[c] = hit ? ex2(__fmaf_rn(l[c], kLog2e, t.mlog)) : 0.f;
+    a[c] = ((c % kNucSubs) * kNucBins + ((kbits >> t.sh) & (kNucBins - 1))) * 32;
+  }
+#pragma unroll
+  for (int c = 0; c < 4; c += kNucSubs) {
+    float v[kNucSubs];
+#pragma unroll
+    for (int h = 0; h < kNucSubs; ++h) v[h] = bins[a[c + h]];
+#pragma unroll
+    for (int h = 0; h < kNucSubs; ++h) bins[a[c + h]] = v[h] + ex[c + h];
+  }
+}
+
 // Top-p: the nucleus of the rows of sequence b that can decide anything (see
 // nuc_key), its group together.  A draft row whose u is past p(d) / (top_p q(d))
 // is rejected whatever its nucleus (the nucleus holds at least top_p of p), so
@@ -582,12 +715,14 @@ __device__ __forceinline__ void share_of(int V, int gs, int rank, int *lo, int *
 // its share of each row -- lane-private fp32 bins in kNucSubs copies (lane i's
 // words all in bank i: no conflicts, no shared-memory atomics per value), summed
 // in a fixed order and added to the row's bins in fixed point (2^31 = all of p:
-// integer sums, the same in any order) -- publishes them, and after the group
-// barrier sums every CTA's bins itself, so a round takes one barrier.  Two
-// buffers alternate: a CTA writes a round's bins only after every CTA has read
-// those of two rounds before.
-__device__ __forceinline__ void nucleus(const Call &p, RowsSmem &s, int b, const SeqInfo &q, float top, int g,
-                                        int rank, int gs, int lo, int hi, int tid, int warp, int lane) {
+// integer sums, the same in any order) -- posts them, and sums every CTA's bins
+// itself as they arrive.
+// The first round bins every value and is bound by its ~18 instructions each.
+// The second keeps the values of the chosen bin (one unit of log-probability
+// wide: a few percent of a row) in lane-private lists, and it and the later
+// rounds bin only those; an item whose list overflows reads its values again.
+__device__ __forceinline__ void nucleus(const Call &p, RowsSmem &s, int b, const SeqInfo &q, float top, int rank,
+                                        int gs, int lo, int hi, int tid, int warp, int lane) {
   if (tid == 0) s.nl = q.k + 1;
   block_sync();
   for (int i = tid; i < q.k; i += kThreads) {
@@ -603,54 +738,90 @@ __device__ __forceinline__ void nucleus(const Call &p, RowsSmem &s, int b, const
   }
   const float IT = inv_temp(p, b);
   const int parts = nl < kWarps ? kWarps / nl : 1;  // warps per row
+  const int items = nl * parts;
   const int per = ((hi - lo + parts - 1) / parts + 127) & ~127;
+  unsigned(*hist)[kNucBins] = reinterpret_cast<unsigned(*)[kNucBins]>(s.pool);
+  uint16_t(*cnt)[32] = reinterpret_cast<uint16_t(*)[32]>(s.pool + nl * kNucBins * 4);
+  float *lists = reinterpret_cast<float *>(s.pool + nl * kNucBins * 4 + items * 32 * 2);
+  // List entries per lane and item.
+  const int cap = min(4096, (p.pool - nl * kNucBins * 4 - items * 32 * 2) / (32 * 4 * items));
   float *bins = s.bins[warp] + lane;
 #pragma unroll 1
   for (int r = 0; r < kNucRounds; ++r) {
     const int sh = kNucKeyBits - kNucBinBits * (r + 1);  // this round's bin: key bits [sh, sh + 5)
-    for (int e = tid; e < nl * kNucBins; e += kThreads) s.hist[e / kNucBins][e % kNucBins] = 0u;
+    for (int e = tid; e < nl * kNucBins; e += kThreads) hist[e / kNucBins][e % kNucBins] = 0u;
     block_sync();
 #pragma unroll 1
-    for (int item = warp; item < nl * parts; item += kWarps) {
+    for (int item = warp; item < items; item += kWarps) {
       const int i = item / parts, part = item - i * parts;
       const int pre = s.npre[i];
       if (pre < 0) continue;
       const float M = s.m[i];
-      const float nb65 = -kNucScale * __fsub_rn(M, kNucSpan);
-      const float mlog = -M * kLog2e;
-      const int pre_bits = pre + (kNucKeyBias >> (sh + kNucBinBits));  // the range's key prefix, as bits
+      BinRound t;
+      t.nb65 = -kNucScale * __fsub_rn(M, kNucSpan);
+      t.mlog = -M * kLog2e;
+      t.sh = sh;
+      t.pre_bits = pre + (kNucKeyBias >> (sh + kNucBinBits));  // the range's key prefix, as bits
       const float *lg = p.logits + static_cast<size_t>(q.r0 + i) * p.ldl;
       const int plo = lo + part * per, phi = min(hi, plo + per);
+      float *list = lists + item * cap * 32 + lane;  // entry j of this lane: list[32 j]
+      int n = r == 0 ? cap + 1 : (r == 1 ? 0 : cnt[item][lane]);
 #pragma unroll 8
       for (int k = 0; k < kNucSubs * kNucBins; ++k) bins[k * 32] = 0.f;
+      if (r == 1) {
+        // Values with the first round's prefix, kept (past cap only counted).
 #pragma unroll 1
-      for (int e0 = plo + 4 * lane; e0 < phi; e0 += 4 * 128) {
-        float4 v4[4];
+        for (int e0 = plo + 4 * lane; e0 < phi; e0 += 4 * 128) {
+          float4 v4[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          v4[j] = e0 + 128 * j < phi ? __ldcg(reinterpret_cast<const float4 *>(lg + e0 + 128 * j))
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int j = 0; j < 4; ++j)
+            v4[j] = e0 + 128 * j < phi ? __ldcg(reinterpret_cast<const float4 *>(lg + e0 + 128 * j))
+                                       : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float x[4] = {v4[j].x, v4[j].y, v4[j].z, v4[j].w};
-          float ex[4];
-          int a[4];
+          for (int j = 0; j < 4; ++j) {
+            const float x[4] = {v4[j].x, v4[j].y, v4[j].z, v4[j].w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float l = __fmul_rn(x[c], IT);
+              const bool in = e0 + 128 * j + c < phi &&
+                              (nuc_key_bits(l, t.nb65) >> (sh + kNucBinBits)) == t.pre_bits;
+              if (in) {
+                if (n < cap) list[32 * n] = l;
+                ++n;
+              }
+            }
+          }
+        }
+        cnt[item][lane] = static_cast<uint16_t>(min(n, cap + 1));
+      }
+      if (__any_sync(0xffffffffu, n > cap)) {
+#pragma unroll 1
+        for (int e0 = plo + 4 * lane; e0 < phi; e0 += 4 * 128) {
+          float4 v4[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            v4[j] = e0 + 128 * j < phi ? __ldcg(reinterpret_cast<const float4 *>(lg + e0 + 128 * j))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int e = e0 + 128 * j;
+            const float l[4] = {__fmul_rn(v4[j].x, IT), __fmul_rn(v4[j].y, IT), __fmul_rn(v4[j].z, IT),
+                                __fmul_rn(v4[j].w, IT)};
+            const bool in[4] = {e < phi, e + 1 < phi, e + 2 < phi, e + 3 < phi};
+            bin4(t, bins, l, in);
+          }
+        }
+      } else {
+#pragma unroll 1
+        for (int j = 0; j < n; j += 4) {
+          float l[4];
+          bool in[4];
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const float l = __fmul_rn(x[c], IT);
-            const int kbits = nuc_key_bits(l, nb65);
-            const bool in = e0 + 128 * j + c < phi && (kbits >> (sh + kNucBinBits)) == pre_bits;
-            ex[c] = in ? ex2(__fmaf_rn(l, kLog2e, mlog)) : 0.f;
-            a[c] = ((c % kNucSubs) * kNucBins + ((kbits >> sh) & (kNucBins - 1))) * 32;
+            in[c] = j + c < n;
+            l[c] = in[c] ? list[32 * (j + c)] : 0.f;
           }
-#pragma unroll
-          for (int c = 0; c < 4; c += kNucSubs) {
-            float v[kNucSubs];
-#pragma unroll
-            for (int h = 0; h < kNucSubs; ++h) v[h] = bins[a[c + h]];
-#pragma unroll
-            for (int h = 0; h < kNucSubs; ++h) bins[a[c + h]] = v[h] + ex[c + h];
-          }
+          bin4(t, bins, l, in);
         }
       }
       __syncwarp();
@@ -662,28 +833,42 @@ __device__ __forceinline__ void nucleus(const Call &p, RowsSmem &s, int b, const
 #pragma unroll
         for (int h = 0; h < kNucSubs; ++h) f += all[(h * kNucBins + lane) * 32 + ((j + lane) & 31)];
       const unsigned fixed = __float2uint_rn(f * (0x1p31f / s.z[i]));
-      if (fixed != 0u) atomicAdd(&s.hist[i][lane], fixed);
+      if (fixed != 0u) atomicAdd(&hist[i][lane], fixed);
       __syncwarp();
     }
     block_sync();
-    if (gs > 1) {
-      unsigned *mine = p.nhist + (static_cast<size_t>((r & 1) * kMaxGroup + rank) * p.R + q.r0) * kNucBins;
-      for (int e = tid; e < nl * kNucBins; e += kThreads) __stcg(&mine[e], s.hist[e / kNucBins][e % kNucBins]);
-      group_arrive(p, s, g, gs);
-      group_wait(p, s, g, gs);
-    }
+    unsigned *round = p.nhist + (static_cast<size_t>(r * kMaxGroup) * p.R + q.r0) * kNucBins;
+    const size_t stride = static_cast<size_t>(p.R) * kNucBins;  // words between the CTAs' bins
+    if (gs > 1)
+      for (int e = tid; e < nl * kNucBins; e += kThreads)
+        st_relaxed(round + rank * stride + e, hist[e / kNucBins][e % kNucBins]);
     // C_k = mass of keys at or above bin k plus the mass above the range: keep
     // the highest bin with C_k >= top_p.  Sums stay below 2^33.
 #pragma unroll 1
     for (int i = warp; i < nl; i += kWarps) {
-      unsigned long long own = 0;
+      unsigned long long own = hist[i][lane];
       if (gs > 1) {
-        const unsigned *src =
-            p.nhist + (static_cast<size_t>((r & 1) * kMaxGroup) * p.R + q.r0 + i) * kNucBins + lane;
-#pragma unroll 8
-        for (int c = 0; c < gs; ++c) own += __ldcg(src + static_cast<size_t>(c) * p.R * kNucBins);
-      } else {
-        own = s.hist[i][lane];
+        const unsigned *src = round + i * kNucBins + lane;
+        unsigned v[kMaxGroup];  // every CTA's bins in flight at once
+#pragma unroll
+        for (int c = 0; c < kMaxGroup; ++c) v[c] = c < gs && c != rank ? ld_relaxed(src + c * stride) : 0u;
+#pragma unroll 1
+        for (int again = 1; again;) {  // late ones (all lanes of a warp retry together)
+          again = 0;
+#pragma unroll
+          for (int c = 0; c < kMaxGroup; ++c) again |= v[c] == kUnset;
+          if (again) {
+#pragma unroll 1
+            for (int c = 0; c < gs; ++c)
+              if (c != rank) poll_word(p, s, src + c * stride);
+#pragma unroll
+            for (int c = 0; c < kMaxGroup; ++c) v[c] = c < gs && c != rank ? ld_relaxed(src + c * stride) : 0u;
+            if (*const_cast<volatile int *>(&s.abort)) break;
+          }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < kMaxGroup; ++c) own += v[c] == kUnset ? 0u : v[c];
       }
       unsigned long long C = own;  // suffix sum over lanes >= this one
 #pragma unroll
@@ -732,47 +917,70 @@ struct Dist {
   const float *q;   // draft distribution, or null: p
   float M, invS, IT, base;
   int tkey;
-  bool qvec;
 };
-__device__ __forceinline__ void dist_load4(const Dist &t, int e, int hi, float4 &l4, float4 &q4) {
-  l4 = __ldcg(reinterpret_cast<const float4 *>(t.lg + e));
-  q4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (t.q) {
-    if (t.qvec) {
-      q4 = __ldg(reinterpret_cast<const float4 *>(t.q + e));
-    } else {
-      q4.x = __ldg(t.q + e);
-      if (e + 1 < hi) q4.y = __ldg(t.q + e + 1);
-      if (e + 2 < hi) q4.z = __ldg(t.q + e + 2);
-      if (e + 3 < hi) q4.w = __ldg(t.q + e + 3);
-    }
+// Entries of a lane's block of a piece of `len` entries: the ten warps take
+// contiguous parts, their lanes contiguous blocks of an odd length (lanes then
+// read distinct banks).
+__device__ __forceinline__ int lane_block(int len) { return ((len + kThreads - 1) / kThreads) | 1; }
+
+// Loads entries [e0, e0 + len) of the logits row (and of q) into shared memory,
+// replaces the logits by the terms of the distribution and returns the
+// inclusive prefix of this lane's block sum over the warp.  The piece arrives
+// by bulk copies (q by plain loads when its rows are not 16-byte aligned).
+// The terms are fp32; sums are compensated (the terms are >= 0, so ordering the
+// two addends by size makes the error term exact).
+__device__ __forceinline__ ff2 piece_terms(const Call &p, RowsSmem &s, const Dist &t, int e0, int len, uint32_t parity,
+                                        int tid, int warp, int lane) {
+  float *sl = s.piece.l, *sq = s.piece.q;
+  const bool bulk_q = t.q != nullptr && p.qvec;
+  if (tid == 0) {
+    fence_proxy_async();  // earlier generic accesses, and the logits' stores, come first
+    const uint32_t bytes = static_cast<uint32_t>((len + 3) & ~3) * 4u;
+    mbar_arrive_expect_tx(&s.bar, bulk_q ? 2 * bytes : bytes);
+    bulk_load(sl, t.lg + e0, bytes, &s.bar);
+    if (bulk_q) bulk_load(sq, t.q + e0, bytes, &s.bar);
   }
-}
-__device__ __forceinline__ float dist_term(const Dist &t, float l, float q, bool in_share) {
-  const float lv = __fmul_rn(l, t.IT);
-  const bool in = t.tkey == INT_MIN || nuc_key(lv, t.base) >= t.tkey;
-  const float pv = in ? ex2((lv - t.M) * kLog2e) * t.invS : 0.f;
-  const float rv = t.q ? fmaxf(0.f, pv - q) : pv;
-  return in_share ? rv : 0.f;
-}
-__device__ __forceinline__ void dist_terms(const Dist &t, int e, int hi, const float4 &l4, const float4 &q4,
-                                           float (&x)[4]) {
-  x[0] = dist_term(t, l4.x, q4.x, e < hi);
-  x[1] = dist_term(t, l4.y, q4.y, e + 1 < hi);
-  x[2] = dist_term(t, l4.z, q4.z, e + 2 < hi);
-  x[3] = dist_term(t, l4.w, q4.w, e + 3 < hi);
+  if (t.q != nullptr && !bulk_q) {
+#pragma unroll 4
+    for (int e = tid; e < len; e += kThreads) sq[e] = __ldg(t.q + e0 + e);
+  }
+  // (the copies read valid memory: this wait does not give up on an earlier
+  // expired wait, so that no copy is left in flight at exit)
+  if (!mbar_wait_unabortable(&s.bar, parity)) {
+    atomicOr(p.status, SPADE_DEV_TIMEOUT);
+    s.abort = 1;
+  }
+  block_sync();
+  const int bs = lane_block(len);
+  const int b0 = (warp * 32 + lane) * bs, b1 = min(len, b0 + bs);
+  float sh = 0.f, lo = 0.f;
+#pragma unroll 4
+  for (int e = b0; e < b1; ++e) {
+    const float lv = __fmul_rn(sl[e], t.IT);
+    const bool in = t.tkey == INT_MIN || nuc_key(lv, t.base) >= t.tkey;
+    const float pv = in ? ex2((lv - t.M) * kLog2e) * t.invS : 0.f;
+    const float x = t.q != nullptr ? fmaxf(0.f, pv - sq[e]) : pv;
+    sl[e] = x;
+    const float sm = sh + x;
+    lo += (fmaxf(sh, x) - sm) + fminf(sh, x);
+    sh = sm;
+  }
+  return warp_scan_ff(ff_norm(sh, lo), lane);
 }
 
 // The draw of sequence b by its group: next_token[b] is the first entry whose
 // cumulative mass exceeds u Z.  Terms are fp32, every sum float-float, so the
-// cumulative masses that place u Z are as exact as the terms allow.  Each warp
-// sums a contiguous part of the CTA's share; the shares' masses meet in the
-// workspace, every CTA finds the owner of u Z from the same masses, and the
-// owner's warp that holds it scans its part again.  A residual with no mass is
-// retried on p (every CTA sees the same total, so all retry together).
+// cumulative masses that place u Z are as exact as the terms allow.  The shares'
+// masses meet in the workspace, every CTA finds the owner of u Z from the same
+// masses, and the owner walks down: piece, warp, lane block, entry.  A residual
+// with no mass is retried on p (every CTA sees the same total, so all retry
+// together).  Bound by the latency of its few dependent steps, and by fetching
+// its code: loops are rolled.
 // `commit`: the group's first CTA updates the cache while the masses travel.
-__device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, const SeqInfo &q, int a, int g, int rank,
-                                           int gs, int lo, int hi, bool commit, int tid, int warp, int lane) {
+// `parity`: phase of the copies' mbarrier, advanced by every piece.
+__device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, const SeqInfo &q, int a, int rank, int gs,
+                                           int lo, int hi, bool commit, uint32_t &parity, int tid, int warp,
+                                           int lane) {
   const int n = q.r0 + a;
   Dist t;
   t.lg = p.logits + static_cast<size_t>(n) * p.ldl;
@@ -782,149 +990,130 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
   t.IT = inv_temp(p, b);
   t.base = __fsub_rn(t.M, kNucSpan);
   t.tkey = s.tkey[a];
-  t.qvec = p.qvec != 0;
   const float u = p.uniforms[q.r0 + q.k];
-  const int per = ((hi - lo + kWarps - 1) / kWarps + 127) & ~127;  // entries per warp
-  const int wlo = min(hi, lo + warp * per), whi = min(hi, wlo + per);
+  const int npiece = (hi - lo + kPiece - 1) / kPiece;
+  ff2 incl;
+  int i = 0, attempt = 0;
+  bool again = false;  // the owner takes the piece that holds the target once more
 #pragma unroll 1
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-    for (int e0 = wlo + 4 * lane; e0 < whi; e0 += 4 * 128) {
-      float4 l4[4], q4[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        l4[j] = q4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e0 + 128 * j < whi) dist_load4(t, e0 + 128 * j, whi, l4[j], q4[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float x[4];
-        dist_terms(t, e0 + 128 * j, whi, l4[j], q4[j], x);
-        // Compensated chains: the terms are >= 0, so ordering the two addends
-        // by size makes the error term exact.
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float sm = sh[c] + x[c];
-          sl[c] += (fmaxf(sh[c], x[c]) - sm) + fminf(sh[c], x[c]);
-          sh[c] = sm;
-        }
-      }
-    }
-    const ff2 mass = warp_sum_ff(ff_add(ff_add(ff_norm(sh[0], sl[0]), ff_norm(sh[1], sl[1])),
-                                        ff_add(ff_norm(sh[2], sl[2]), ff_norm(sh[3], sl[3]))));
-    if (lane == 0) s.wm[warp] = mass;
+  for (;;) {  // (one copy of the piece's code)
+    incl = piece_terms(p, s, t, lo + i * kPiece, min(kPiece, hi - lo - i * kPiece), parity, tid, warp, lane);
+    parity ^= 1u;
+    if (again) break;
+    if (lane == 31) s.pm[i][warp] = incl;
     block_sync();
-    float2 *zp = p.zpart + (static_cast<size_t>(attempt) * p.B + b) * kMaxGroup;
-    if (tid == 0) {
-      ff2 z{0.f, 0.f};
-      for (int w = 0; w < kWarps; ++w) z = ff_add(z, s.wm[w]);
-      __stcg(&zp[rank], make_float2(z.hi, z.lo));
-    }
-    group_arrive(p, s, g, gs);
-    if (attempt == 0 && commit && rank == 0) commit_seq(p, b, q.k, a, tid);
-    group_wait(p, s, g, gs);
+    if (++i < npiece) continue;
+    unsigned long long *zp = p.zpart + (static_cast<size_t>(attempt) * p.B + b) * kMaxGroup;
     if (warp == 0) {
-      const float2 zz = lane < gs ? __ldcg(&zp[lane]) : make_float2(0.f, 0.f);
-      const ff2 mine{zz.x, zz.y};
-      const ff2 incl = warp_scan_ff(mine, lane);
-      const ff2 tot = ff_shfl(incl, 31);
+      // This share's mass: lane w sums the pieces of warp w's parts, in order.
+      ff2 z{0.f, 0.f};
+      for (int j = 0; j < npiece && lane < kWarps; ++j) z = ff_add(z, s.pm[j][lane]);
+      z = ff_shfl(warp_scan_ff(z, lane), 31);
+      if (lane == 0) post_mass(&zp[rank], z);
+    }
+    if (attempt == 0 && commit && rank == 0) commit_seq(p, b, q.k, a, tid);
+    if (warp == 0) {
+      const ff2 mine = lane < gs ? poll_mass(p, s, &zp[lane]) : ff2{0.f, 0.f};
+      __syncwarp();
+      const ff2 reach = warp_scan_ff(mine, lane);
+      const ff2 tot = ff_shfl(reach, 31);
       const bool ok = tot.hi > 0.f && isfinite(tot.hi);
       const ff2 target = ff_mul_f(tot, u);
-      const unsigned hit = __ballot_sync(0xffffffffu, ok && mine.hi > 0.f && ff_gt(incl, target));
+      const unsigned hit = __ballot_sync(0xffffffffu, ok && mine.hi > 0.f && ff_gt(reach, target));
       const unsigned pos = __ballot_sync(0xffffffffu, ok && mine.hi > 0.f);
       // Rounding past the total clamps to the last share with mass.
       const int own = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : -1);
-      const ff2 before = ff_shfl(ff_sub(incl, mine), own < 0 ? 0 : own);
+      const ff2 before = ff_shfl(ff_sub(reach, mine), own < 0 ? 0 : own);
+      int own_piece = -1, own_warp = 0;
+      if (own == rank) {
+        // The piece, then the warp part, in vocabulary order; rounding past the
+        // share's mass clamps to the last part with mass.
+        ff2 left = hit ? ff_sub(target, before) : ff2{INFINITY, 0.f};
+        ff2 run{0.f, 0.f}, left_at = left;
+        bool over = false;
+#pragma unroll 1
+        for (int j = 0; j < npiece && !over; ++j) {
+          const ff2 wm = lane < kWarps ? s.pm[j][lane] : ff2{0.f, 0.f};
+          const ff2 wr = ff_add(run, warp_scan_ff(wm, lane));
+          const unsigned wh = __ballot_sync(0xffffffffu, wm.hi > 0.f && ff_gt(wr, left));
+          const unsigned wp = __ballot_sync(0xffffffffu, wm.hi > 0.f);
+          const int w = wh ? __ffs(wh) - 1 : (wp ? 31 - __clz(wp) : -1);
+          over = wh != 0u;
+          if (w >= 0) {
+            own_piece = j;
+            own_warp = w;
+            left_at = over ? ff_sub(left, ff_shfl(ff_sub(wr, wm), w)) : ff2{INFINITY, 0.f};
+          }
+          run = ff_shfl(wr, 31);
+        }
+        if (lane == 0) s.tgt = left_at;  // target left inside the warp's part
+      }
       if (lane == 0) {
         s.retry = !ok;
-        s.owner = own;
-        s.tgt = ff_sub(target, before);  // target left inside the owner's share
+        s.owner_piece = own_piece;
+        s.owner_warp = own_warp;
+        if (!ok && attempt == 1 && rank == 0) p.next_token[b] = -1;  // p has no mass either
+        if (ok && attempt == 1 && rank == 0) atomicOr(p.status, SPADE_DEV_FALLBACK);
       }
     }
     block_sync();
-    if (!s.retry) {
-      if (attempt == 1 && rank == 0 && tid == 0) atomicOr(p.status, SPADE_DEV_FALLBACK);
-      break;
+    if (s.retry) {  // the residual has no mass: sample p
+      if (attempt == 1) return;
+      attempt = 1;
+      t.q = nullptr;
+      i = 0;
+      continue;
     }
-    t.q = nullptr;  // the residual has no mass: sample p
+    if (s.owner_piece < 0) return;
+    if (s.owner_piece == npiece - 1) break;
+    i = s.owner_piece;
+    again = true;
   }
-  if (s.retry || s.owner < 0) {
-    if (rank == 0 && tid == 0) p.next_token[b] = -1;  // p has no mass either
-    return;
-  }
-  if (s.owner != rank) return;
-  // The warp part holding the target, then the entry, in vocabulary order.
-  if (warp == 0) {
-    const ff2 mine = lane < kWarps ? s.wm[lane] : ff2{0.f, 0.f};
-    const ff2 incl = warp_scan_ff(mine, lane);
-    const unsigned hit = __ballot_sync(0xffffffffu, mine.hi > 0.f && ff_gt(incl, s.tgt));
-    const unsigned pos = __ballot_sync(0xffffffffu, mine.hi > 0.f);
-    const int own = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
-    const ff2 before = ff_shfl(ff_sub(incl, mine), own);
-    if (lane == 0) {
-      s.owner_warp = own;
-      s.wtgt = hit ? ff_sub(s.tgt, before) : ff2{INFINITY, 0.f};  // rounding: clamp to the last mass
-    }
-  }
-  block_sync();
-  if (warp == s.owner_warp) {
-    const ff2 target = s.wtgt;
-    ff2 run{0.f, 0.f};
-    int found = -1, last = -1;  // last: the last entry with mass so far
+  const int e0 = lo + s.owner_piece * kPiece, len = min(kPiece, hi - e0);
+  if (warp != s.owner_warp) return;
+  // The lane block, then the entry.
+  const ff2 left = s.tgt;
+  const ff2 prev{__shfl_up_sync(0xffffffffu, incl.hi, 1), __shfl_up_sync(0xffffffffu, incl.lo, 1)};
+  const bool some = lane == 0 ? incl.hi > 0.f : ff_gt(incl, prev);
+  const unsigned hit = __ballot_sync(0xffffffffu, some && ff_gt(incl, left));
+  const unsigned pos = __ballot_sync(0xffffffffu, some);
+  const int blk = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
+  const ff2 before = blk == 0 ? ff2{0.f, 0.f} : ff_shfl(incl, blk - 1);
+  const int bs = lane_block(len), b0 = (warp * 32 + blk) * bs, b1 = min(len, b0 + bs);
+  ff2 run = before;
+  int token = -1;
+  bool over = false;
 #pragma unroll 1
-    for (int e0 = wlo; e0 < whi && found < 0; e0 += 128) {
-      const int e = e0 + 4 * lane;
-      float4 l4 = make_float4(0.f, 0.f, 0.f, 0.f), q4 = l4;
-      if (e < whi) dist_load4(t, e, whi, l4, q4);
-      float x[4];
-      dist_terms(t, e, whi, l4, q4, x);
-      ff2 mine{x[0], 0.f};
-#pragma unroll
-      for (int c = 1; c < 4; ++c) mine = ff_add_f(mine, x[c]);
-      const ff2 incl = ff_add(run, warp_scan_ff(mine, lane));
-      const unsigned hit = __ballot_sync(0xffffffffu, mine.hi > 0.f && ff_gt(incl, target));
-      const unsigned pos = __ballot_sync(0xffffffffu, mine.hi > 0.f);
-      const int src = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : -1);
-      if (src >= 0) {
-        // Lane src's first entry past the target, else its last one with mass.
-        ff2 acc = ff_sub(incl, mine);
-        int at = -1;
-        bool over = false;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          acc = ff_add_f(acc, x[c]);
-          if (x[c] > 0.f && !over) {
-            at = e + c;
-            over = hit != 0u && ff_gt(acc, target);
-          }
-        }
-        at = __shfl_sync(0xffffffffu, at, src);
-        if (hit) found = at;
-        else last = at;
-      }
-      run = ff_shfl(incl, 31);
-    }
-    if (lane == 0) p.next_token[b] = found >= 0 ? found : (last >= 0 ? last : wlo);
+  for (int c = b0; c < b1 && !over; c += 32) {
+    const int e = c + lane;
+    const float x = e < b1 ? s.piece.l[e] : 0.f;
+    const ff2 reach = ff_add(run, warp_scan_ff(ff2{x, 0.f}, lane));
+    const unsigned xh = __ballot_sync(0xffffffffu, hit != 0u && x > 0.f && ff_gt(reach, left));
+    const unsigned xp = __ballot_sync(0xffffffffu, x > 0.f);
+    over = xh != 0u;
+    if (xp) token = e0 + c + (over ? __ffs(xh) - 1 : 31 - __clz(xp));  // else the last entry with mass
+    run = ff_shfl(reach, 31);
   }
+  if (lane == 0) p.next_token[b] = token >= 0 ? token : e0 + b0;
 }
 
 // After the statistics of every slice (a grid barrier, or the previous launch's
 // end): decisions, outputs, commit and the draws.  Sampled sequences are dealt
 // to groups of CTAs from the front of the grid, greedy ones to single CTAs
-// from its end; no group waits for another.
-__device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, int c, int nctas) {
+// from its end; no group waits for another.  The CTAs of a group wait for one
+// another's words (every CTA is resident: cooperative launches).
+__device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const SeqTable &seqs, const RowTables &rows, int c,
+                                           int nctas) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (warp == 0) {
     int ns = 0, ng = 0;
     for (int b0 = 0; b0 < p.B; b0 += 32) {
       const int b = b0 + lane;
-      const bool st = b < p.B && seq_info(p, b).stoch;
-      const unsigned ms = __ballot_sync(0xffffffffu, st);
-      const unsigned mg = __ballot_sync(0xffffffffu, b < p.B && !st);
-      const unsigned below = (1u << lane) - 1u;
-      if (st) s.st[ns + __popc(ms & below)] = b;
-      else if (b < p.B) s.gr[ng + __popc(mg & below)] = b;
+      const unsigned in = p.B - b0 >= 32 ? 0xffffffffu : (1u << (p.B - b0)) - 1u;
+      const unsigned ms = seqs.stoch[b0 / 32] & in, mg = ~seqs.stoch[b0 / 32] & in;
+      const unsigned bit = 1u << lane, below = bit - 1u;
+      if (ms & bit) s.st[ns + __popc(ms & below)] = b;
+      if (mg & bit) s.gr[ng + __popc(mg & below)] = b;
       ns += __popc(ms);
       ng += __popc(mg);
     }
@@ -932,6 +1121,8 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, int c, in
       s.n_st = ns;
       s.n_gr = ng;
       s.abort = 0;
+      mbar_init(&s.bar, 1);
+      fence_mbar_init();
     }
   } else if (c == 0) {
     for (int b = tid - 32; b < p.B; b += kThreads - 32) {
@@ -952,27 +1143,28 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, int c, in
     const int g = c / gs, rank = c - g * gs;
     int lo, hi;
     share_of(p.V, gs, rank, &lo, &hi);
+    uint32_t parity = 0;
 #pragma unroll 1
     for (int i = g; i < ns; i += ngroups) {
       const int b = s.st[i];
-      const SeqInfo q = seq_info(p, b);
-      decide_rows(p, s, b, q, rank == 0, warp, lane);
+      const SeqInfo q = table_info(seqs, b);
+      decide_rows(p, s, rows, b, q, rank == 0, warp, lane);
       const float top = seq_top_p(p, b);
       int upto = q.k;
       if (top < 1.f) {
-        nucleus(p, s, b, q, top, g, rank, gs, lo, hi, tid, warp, lane);
+        nucleus(p, s, b, q, top, rank, gs, lo, hi, tid, warp, lane);
         upto = min(q.k, s.nl);
       }
       const int a = first_reject(s, upto, tid);
       if (rank == 0 && tid == 0) p.accepted_len[b] = a;
-      draw_token(p, s, b, q, a, g, rank, gs, lo, hi, p.kc != nullptr, tid, warp, lane);
+      draw_token(p, s, b, q, a, rank, gs, lo, hi, p.kc != nullptr, parity, tid, warp, lane);
       block_sync();
     }
   }
 #pragma unroll 1
   for (int i = nctas - 1 - c; i < ng; i += nctas) {
     const int b = s.gr[i];
-    const SeqInfo q = seq_info(p, b);
+    const SeqInfo q = table_info(seqs, b);
     if (!q.valid) {
       if (tid == 0) {
         p.accepted_len[b] = 0;
@@ -980,7 +1172,7 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, int c, in
       }
       continue;
     }
-    decide_rows(p, s, b, q, true, warp, lane);
+    decide_rows(p, s, rows, b, q, true, warp, lane);
     const int a = first_reject(s, q.k, tid);
     if (tid == 0) {
       p.accepted_len[b] = a;

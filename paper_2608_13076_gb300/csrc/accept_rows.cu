@@ -11,13 +11,23 @@ namespace spade {
 namespace accept {
 
 __global__ void __launch_bounds__(kThreads, 1) accept_rows_kernel(const __grid_constant__ Call c) {
-  extern __shared__ __align__(16) uint8_t smem_rows[];
+  extern __shared__ __align__(128) uint8_t smem_rows[];
+  __shared__ SeqTable seqs;
   griddep_wait();
   griddep_launch_dependents();
-  rows_phase(c, *reinterpret_cast<RowsSmem *>(smem_rows), blockIdx.x, gridDim.x);
+  fill_table(c, seqs, threadIdx.x / 32, kWarps, threadIdx.x % 32, false);  // (reported by the first launch)
+  block_sync();
+  rows_phase(c, *reinterpret_cast<RowsSmem *>(smem_rows), seqs, RowTables{}, blockIdx.x, gridDim.x);
 }
 
 spade_status launch_accept_rows(const Call &c, int sms, cudaStream_t stream) {
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(accept_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(kRowsBytesPlain));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(accept_rows)");
+    configured = true;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sms < kMaxNC ? sms : kMaxNC);
   cfg.blockDim = dim3(kThreads);

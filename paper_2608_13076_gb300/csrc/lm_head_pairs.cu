@@ -37,15 +37,16 @@ struct PairParams {
 };
 
 struct PairSmem {
-  int stage, off_bar, off_misc, off_rows, off_stat, off_tbuf, total;
+  int stage, off_bar, off_misc, off_seq, off_rows, off_stat, off_tbuf, total;
 };
 __host__ __device__ inline PairSmem pair_layout(int Ncols, int stages) {
   PairSmem s;
   s.stage = kWChunkBytes + Ncols / 2 * 128;  // W rows, then this CTA's half of each N-chunk
   s.off_bar = stages * s.stage;
   s.off_misc = s.off_bar + (2 * kMaxStages + 6) * 8;
-  s.off_rows = (s.off_misc + 16 + 15) & ~15;
-  s.off_stat = s.off_rows + Ncols * 8 + Ncols / kBlk * 4;
+  s.off_seq = (s.off_misc + 16 + 15) & ~15;
+  s.off_rows = s.off_seq + static_cast<int>(sizeof(SeqTable));
+  s.off_stat = s.off_rows + row_table_bytes(Ncols, false);
   // A statistics warp keeps every second block of rows.
   s.off_tbuf = (s.off_stat + kEpiWarps * ((Ncols / kBlk + 1) / 2) * static_cast<int>(sizeof(BlkStat)) + 15) & ~15;
   s.total = s.off_tbuf + kTBufBytes + 1024;
@@ -65,9 +66,7 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
   uint64_t *fin = acc_empty + 2;            // teardown handshake
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.off_misc);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.off_misc + 8);
-  int32_t *s_draft = reinterpret_cast<int32_t *>(smem + L.off_rows);
-  float *s_it = reinterpret_cast<float *>(s_draft + p.Ncols);
-  unsigned *s_keep = reinterpret_cast<unsigned *>(s_it + p.Ncols);
+  const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, false);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x;
@@ -190,7 +189,8 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
     const int et = tid - 64, ew = warp - 2, q4 = warp & 3, part = ew >> 2;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
     float *T = reinterpret_cast<float *>(smem + L.off_tbuf) + ew * (32 * kTStride);
-    setup_rows(p.c, p.Ncols, s_draft, s_it, s_keep, et);
+    clear_exchange(p.c, c * kEpiThreads + et, p.c.NC * kEpiThreads);
+    setup_rows(p.c, p.Ncols, *reinterpret_cast<SeqTable *>(smem + L.off_seq), rows, et);
     const int nblk = p.Ncols / kBlk, per = (nblk + 1) / 2;
     BlkStat *stats = reinterpret_cast<BlkStat *>(smem + L.off_stat) + ew * per;
     for (int j = 0; j < per; ++j) blk_init(stats[j], lane);
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
       if (v0 < hi) {
 #pragma unroll 1
         for (int bk = part; bk < nblk; bk += 2)
-          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, hi, s_keep[bk], s_draft, s_it, T, lane, stats[bk >> 1]);
+          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, hi, rows, T, lane, stats[bk >> 1]);
       }
       // The accumulator is read: the MMA thread counts both CTAs' warps.
       tc_fence_before();

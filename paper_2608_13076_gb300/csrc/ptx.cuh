@@ -41,6 +41,9 @@ SPADE_DEVICE void fence_mbar_init() {
 SPADE_DEVICE void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// Orders this thread's view of generic-proxy accesses (shared and global memory)
+// against the async proxy's.
+SPADE_DEVICE void fence_proxy_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
 SPADE_DEVICE void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                "r"(bytes)

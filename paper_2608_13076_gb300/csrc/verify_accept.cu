@@ -54,7 +54,7 @@ struct Params {
 
 struct Smem {
   int w_slot, h_slot;
-  int off_h, off_bar, off_misc, off_rows, off_stat, off_tbuf, total;
+  int off_h, off_bar, off_misc, off_seq, off_rows, off_stat, off_tbuf, total;
 };
 
 __host__ __device__ inline Smem smem_layout(const Params &p) {
@@ -64,8 +64,9 @@ __host__ __device__ inline Smem smem_layout(const Params &p) {
   s.off_h = p.WS * s.w_slot;
   s.off_bar = s.off_h + p.HS * s.h_slot;  // the rings end here; the rows phase reuses them
   s.off_misc = (s.off_bar + (2 * p.WS + 2 * p.HS + 4) * 8 + 127) & ~127;
-  s.off_rows = s.off_misc + 64;  // int, float [Ncols], unsigned [Ncols / 16]
-  s.off_stat = s.off_rows + p.Ncols * 8 + p.Ncols / kBlk * 4;
+  s.off_seq = s.off_misc + 64;
+  s.off_rows = s.off_seq + static_cast<int>(sizeof(SeqTable));
+  s.off_stat = s.off_rows + row_table_bytes(p.Ncols, true);
   s.off_tbuf = (s.off_stat + kEpiWarps * (p.Ncols / kBlk) * static_cast<int>(sizeof(BlkStat)) + 127) & ~127;
   s.total = s.off_tbuf + kTBufBytes + 1024;
   return s;
@@ -91,9 +92,8 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
   uint64_t *acc_empty = acc_full + 2;   // [2]
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.off_misc);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.off_misc + 8);
-  int32_t *s_draft = reinterpret_cast<int32_t *>(smem + L.off_rows);
-  float *s_it = reinterpret_cast<float *>(s_draft + p.Ncols);
-  unsigned *s_keep = reinterpret_cast<unsigned *>(s_it + p.Ncols);
+  SeqTable &seqs = *reinterpret_cast<SeqTable *>(smem + L.off_seq);
+  const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, true);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x;
@@ -267,7 +267,8 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
     const int part = ew >> 2;            // which of the quarter's two warps
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
     float *T = reinterpret_cast<float *>(smem + L.off_tbuf) + ew * (32 * kTStride);
-    setup_rows(p.c, p.Ncols, s_draft, s_it, s_keep, et);
+    clear_exchange(p.c, c * kEpiThreads + et, p.c.NC * kEpiThreads);
+    setup_rows(p.c, p.Ncols, seqs, rows, et);
     // The quarter's two warps take the (tile, 16-row block) items in turn; each
     // keeps running statistics of every block, in shared memory (one copy of
     // the block's code, whatever the row count).
@@ -289,13 +290,14 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
         const uint32_t col = tmem + lane_base + static_cast<uint32_t>(buf * kHalfCols + j * p.Ncols);
 #pragma unroll 1
         for (int bk = (t * nblk + part) & 1; bk < nblk; bk += 2)
-          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, v_hi, s_keep[bk], s_draft, s_it, T, lane, stats[bk]);
+          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, v_hi, rows, T, lane, stats[bk]);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[buf]);
       tdone += nt;
     }
+    fence_proxy_async();  // the draws read the stored logits by bulk copies
     // Merge the warps' statistics and publish this CTA's slice partials.
     named_bar(1, kEpiThreads);
     publish_slice(p.c, all_stats, nblk, c, et);
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
     if (tid == 0) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
   }
   // (the rings are idle: the last round's accumulators were complete)
-  rows_phase(p.c, *reinterpret_cast<RowsSmem *>(smem), c, p.c.NC);
+  rows_phase(p.c, *reinterpret_cast<RowsSmem *>(smem), seqs, rows, c, p.c.NC);
 
   // ---- teardown: every TMEM access above has completed --------------------
   tc_fence_before();
@@ -326,8 +328,10 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
 
 // Rounds of one CTA's `tiles` vocabulary tiles: as few as let a round's
 // accumulators (Ncols columns each) fit half of the tensor memory -- every round
-// reads the hidden rows once more -- of nearly equal sizes, the larger first, as
-// only the last round's statistics follow the stream.
+// reads the hidden rows once more -- of nearly equal sizes, the larger first.
+// (3, 2, 2 tiles of a 7-tile slice at 72 rows; 3, 3, 1 ends with less statistics
+// to take after the stream, but its one-tile round streams slower: the copies
+// end at 168 us instead of 163.)
 static bool plan_rounds(int tiles, int Ncols, int *round_tiles, int *nrounds) {
   const int fit = kHalfCols / Ncols;
   if (fit <= 0) return false;
@@ -445,7 +449,7 @@ static WsLayout ws_layout(int B, int R, int V, int sms) {
   L.zpart = off;
   off += round_up(static_cast<size_t>(2) * B * kMaxGroup * 8, 256);
   L.nhist = off;
-  if (!L.two_launches) off += round_up(static_cast<size_t>(2) * kMaxGroup * rows * kNucBins * 4, 256);
+  if (!L.two_launches) off += round_up(static_cast<size_t>(kNucRounds) * kMaxGroup * rows * kNucBins * 4, 256);
   L.logits = off;
   off += round_up(rows * L.ldl * 4, 256);
   L.end = off;
@@ -484,8 +488,11 @@ static spade_status prepare(Params &p, const void *hidden, const void *w_lm, int
   if (p.WS < 2) return fail(SPADE_ERR_SHAPE, "shared memory too small for R = %d", R);
   // After the stream the rows phase works in the rings.
   const size_t rings = static_cast<size_t>(smem_layout(p).off_bar);
-  if (rings < (p.c.top_p ? sizeof(RowsSmem) : kRowsBytesPlain))
+  const size_t items = R < kWarps ? kWarps : R;  // rows or parts of rows that the nucleus search lists, at most
+  const size_t pool0 = offsetof(RowsSmem, pool);
+  if (rings < (p.c.top_p ? pool0 + items * kPoolPerRow : kRowsBytesPlain))
     return fail(SPADE_ERR_SHAPE, "shared memory too small for R = %d", R);
+  p.c.pool = static_cast<int>(rings - pool0);
   p.NS = (p.KC + p.KG - 1) / p.KG;
 
   // 2-D views (one k-chunk per box, zero fill past H) serve a ragged last
@@ -641,7 +648,7 @@ static spade_status verify_accept_impl(const void *hidden, const void *w_lm,
   c.pstat = reinterpret_cast<float4 *>(ws + L.pstat);
   c.ldraft = reinterpret_cast<float *>(ws + L.ldraft);
   c.gstat = reinterpret_cast<float4 *>(ws + L.gstat);
-  c.zpart = reinterpret_cast<float2 *>(ws + L.zpart);
+  c.zpart = reinterpret_cast<unsigned long long *>(ws + L.zpart);
   c.nhist = reinterpret_cast<unsigned *>(ws + L.nhist);
   c.logits = reinterpret_cast<float *>(ws + L.logits);
   if (cm) {
