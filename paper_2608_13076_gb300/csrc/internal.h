@@ -17,6 +17,12 @@ spade_status cuda_fail(cudaError_t e, const char *what);
 // Checks that the current device is sm_103 and returns its SM count.
 spade_status device_info(int *num_sms, int *device);
 
+// Encodes a bf16 tensor map of `rank` (2 .. 5) dimensions, innermost first, with
+// the outer dimensions' strides in bytes, 128-byte swizzle, zero fill out of
+// bounds.  Returns false (with a message recorded) on failure.
+bool encode_tmap_bf16_sw128_nd(CUtensorMap *map, const void *base, uint32_t rank, const uint64_t *dims,
+                               const uint64_t *strides_bytes, const uint32_t *box);
+
 // Encodes a 2-D bf16 tensor map [rows, inner] with row stride
 // `row_stride_bytes`, box {box_inner, box_rows}, 128-byte swizzle, zero fill
 // out of bounds.  Returns false (with a message recorded) on failure.

@@ -52,14 +52,19 @@ SPADE_DEVICE void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
 SPADE_DEVICE void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// How long (ns) a try_wait may keep its thread suspended in hardware.  Without
+// this hint it returns at once while the phase is pending, and the waiting warps
+// of a CTA (eight epilogue warps through a whole stream) poll in a loop that takes
+// issue slots and shared-memory cycles from the producer and the MMA thread.
+constexpr uint32_t kSuspendNs = 1000000;
 SPADE_DEVICE bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.b32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
       : "memory");
   return ok != 0;
 }
@@ -83,11 +88,46 @@ SPADE_DEVICE bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort)
 // Bounded wait that ignores the abort flag: used to drain copies already in
 // flight before a CTA exits after an expired wait.
 SPADE_DEVICE bool mbar_wait_unabortable(uint64_t *bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer();
   while (!mbar_try_wait(bar, parity)) {
     if (globaltimer() - t0 > kWaitLimitNs) return false;
   }
   return true;
+}
+
+// ---------------------------------------------------------------- warp-uniform issue
+// The operands of copies, MMAs and commits sit in uniform registers.  A role whose
+// loop runs on one lane keeps its values in per-thread registers and moves every
+// operand over for every instruction (~110 cycles per MMA, ~350 per copy, measured);
+// a role whose whole warp walks the loop, with one elected lane issuing, keeps
+// them uniform.
+SPADE_DEVICE int uniform_warp() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0); }
+// The same value on every lane, in a uniform register (a warp's lanes agree on v).
+SPADE_DEVICE int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+SPADE_DEVICE bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+// Bounded wait of a whole warp (all lanes get the same answer): true once the
+// phase has completed, false if this or an earlier wait of the CTA expired.
+SPADE_DEVICE bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = globaltimer();
+  bool done = false, give_up = false;
+  while (!done && !give_up) {
+    done = mbar_try_wait(bar, parity);
+    if (!done) {
+      if (globaltimer() - t0 > kWaitLimitNs) *abort = 1;
+      give_up = *abort != 0;
+    }
+  }
+  return __all_sync(0xffffffffu, done);
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch
@@ -143,6 +183,25 @@ SPADE_DEVICE void tma_load_3d(void *dst, const CUtensorMap *map, int32_t x, int3
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       ".L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
+
+// Bulk copy from this CTA's shared memory to another CTA's of the cluster (both
+// addresses from cluster_map), completing on that CTA's mbarrier.
+SPADE_DEVICE void bulk_copy_cluster(uint32_t dst_cluster, const void *src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_cluster),
+      "r"(smem_u32(src)), "r"(bytes), "r"(bar_cluster)
+      : "memory");
+}
+
+// 4-D tiled load of box {x, y, z, u}; see tma_load_2d.
+SPADE_DEVICE void tma_load_4d(void *dst, const CUtensorMap *map, int32_t x, int32_t y, int32_t z, int32_t u,
+                              uint64_t *bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      ".L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(u), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
 
@@ -255,10 +314,10 @@ SPADE_DEVICE bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.b32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
       : "memory");
   return ok != 0;
 }

@@ -1,0 +1,381 @@
+// qkv_cluster.cu -- the verify block's QKV projection with rotary embedding
+// (the attention input side of f_l in x_{l+1} = x_l + f_l(x_l), Sec. III-A, for
+// the d+1 positions of the single forward pass, Sec. III-B) for up to 128 verify
+// rows, where streaming W bounds it.
+//
+// Design (GB300):
+//  * Clusters of two CTAs (76 of them cover every SM; clusters of three or more
+//    leave 8 to 16 SMs idle).  A cluster owns a contiguous range of the output's
+//    rotary pairs, cut in quads (4 pairs: 8 rows of W, one swizzle atom), so the
+//    ranges are equal whatever the head count; each of its CTAs takes half of K.
+//    An SM then receives its share of W and half of x, the two partial sums meet
+//    through distributed shared memory, and nothing goes through a workspace:
+//    no partials in L2 (8 MB written and read at 72 rows x 4096), no waiting on
+//    other clusters, so the launch need not be cooperative (that attribute costs
+//    2.7 us between dependent launches).
+//  * tcgen05.mma kind::f16 (bf16 in, fp32 in tensor memory) with the cluster's W
+//    rows on the MMA M side and the verify rows on N.  W is seen as
+//    [head][half][pair][k], so one box brings a head's piece of the range, both
+//    halves of its pairs; a range is one to three pieces, packed back to back.
+//    Each piece is one box of its exact size (a tensor map per size in use):
+//    copies cost ~50 ns each to issue, and pieces cut into boxes of 32, 8 and 4
+//    pairs streamed at 58 GB/s per SM (25.6 us for the Llama-3-8B layer).  The
+//    last 128-row operand of a stage may read past its valid rows (into the
+//    stage's x rows or the next stage: lanes that are never read); the ring is
+//    followed by at least 16 KB of staging so that this stays in plain buffers.
+//  * A ring slot's round trip (MMAs done, slot released, copies issued, data
+//    landed, MMA thread woken) is ~2.2 us whether W comes from HBM or L2, so the
+//    stream's rate is the bytes in flight: one-chunk stages packed without
+//    padding, as many as fit (8 of 21 KB at the Llama-3-8B layer).
+//  * Epilogue: accumulators go to shared memory; the columns of the verify rows
+//    that the peer finishes travel there by one bulk copy (scalar remote stores
+//    took 4.6 us), and each CTA sums, rotates and stores its half of the rows.
+#include "qkv_common.cuh"
+
+namespace spade {
+namespace qkv {
+namespace pair {
+
+constexpr int kThreads = 320;                  // producer warp, MMA warp, eight epilogue warps
+constexpr int kEpiThreads = 256;
+constexpr int kMaxRows = 128;                  // verify rows
+constexpr int kMaxStages = 12;
+constexpr int kMinStages = 4;
+constexpr int kMaxPiece = 16;                  // quads of a piece (a head of dimension 128)
+constexpr int kMaxQuads = 64;                  // quads of a cluster's range (512 rows)
+constexpr int kSmemBudget = 222 * 1024;
+constexpr int kTileBytes = 128 * kKChunk * 2;  // one 128-row operand x one k-chunk
+
+struct Maps {
+  CUtensorMap w[kMaxPiece];  // boxes of 1 .. 16 quads (those in use)
+  CUtensorMap x;
+};
+
+struct Params {
+  Call c;
+  int quads, nclusters;  // quads of the output, clusters
+  int qmax;              // most quads of a cluster
+  int KC;                // k-chunks (ceil(H / 64))
+  int Ncols;             // verify rows rounded up to 16: MMA N
+  int stages;
+  uint32_t tmem_cols;
+};
+
+// Shared-memory plan (offsets from a 1024-byte aligned base): tables first, then
+// the ring, then the staging: this CTA's partial sums, and those received for the
+// verify rows that it finishes.
+struct Layout {
+  int rseq, rpos, freq, qrow, bars, misc, ring, stage_bytes, row_stride, part, recv, total;
+};
+__host__ __device__ inline Layout layout(int R, int Ncols, int qmax, int stages) {
+  Layout L;
+  L.rseq = 0;
+  L.rpos = L.rseq + kMaxRows * 4;
+  L.freq = L.rpos + kMaxRows * 4;
+  L.qrow = L.freq + 64 * 4;  // uint16 [kMaxQuads][2]
+  L.bars = L.qrow + kMaxQuads * 4;
+  L.misc = L.bars + (2 * kMaxStages + 2) * 8;
+  L.ring = (L.misc + 32 + 1023) & ~1023;
+  L.stage_bytes = qmax * 1024 + Ncols * 128;  // 8 W rows per quad, then the x rows
+  L.part = L.ring + stages * L.stage_bytes;
+  L.row_stride = qmax * 8 + 4;                // floats per staged verify row
+  L.recv = L.part + R * L.row_stride * 4;
+  const int staging = (R + (R + 1) / 2) * L.row_stride * 4;
+  L.total = L.part + (staging > kTileBytes ? staging : kTileBytes) + 1024;  // + slack for the 1024-byte alignment
+  return L;
+}
+
+__device__ __forceinline__ void epi_bar() {
+  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    qkv_cluster_kernel(const __grid_constant__ Params p, const __grid_constant__ Maps maps) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const Layout L = layout(p.c.R, p.Ncols, p.qmax, p.stages);
+  int32_t *s_rseq = reinterpret_cast<int32_t *>(smem + L.rseq);
+  int32_t *s_rpos = reinterpret_cast<int32_t *>(smem + L.rpos);
+  float *s_freq = reinterpret_cast<float *>(smem + L.freq);
+  uint16_t *s_qrow = reinterpret_cast<uint16_t *>(smem + L.qrow);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + L.bars);
+  uint64_t *empty = full + kMaxStages;
+  uint64_t *acc_full = empty + kMaxStages;
+  uint64_t *recv_full = acc_full + 1;  // the peer's partial sums have landed
+  uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.misc);
+  volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.misc + 8);
+
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int cl = blockIdx.x >> 1;
+  const int q0 = static_cast<int>(static_cast<int64_t>(p.quads) * cl / p.nclusters);
+  const int nq = static_cast<int>(static_cast<int64_t>(p.quads) * (cl + 1) / p.nclusters) - q0;
+  const int rows = nq * 8;                  // W rows of the cluster
+  const int ntile = (rows + 127) / 128;     // 128-row operands
+  const int qph = p.c.D / 8;                // quads per head
+  // Verify rows [0, h0) are finished by CTA 0, [h0, R) by CTA 1.
+  const int h0 = (p.c.R + 1) / 2;
+  const int n_own = rank ? p.c.R - h0 : h0, n_send = p.c.R - n_own;
+  // This CTA's half of K.  Every cluster reads the same x rows: each starts at
+  // another chunk, so that they do not all load the same lines from L2 at once.
+  const int kc0 = p.KC * static_cast<int>(rank) / 2, nk = p.KC * (static_cast<int>(rank) + 1) / 2 - kc0;
+  const int rot = nk > 0 ? cl % nk : 0;
+
+  // ---- set-up that reads no input -----------------------------------------
+  if (tid == 0) *s_abort = 0;
+  for (int j = tid; j < p.c.D / 2; j += kThreads) s_freq[j] = p.c.inv_freq[j];
+  if (warp == 0 && lane == 0) {
+    tma_prefetch_desc(&maps.x);
+    // Pieces: one box per head.  A box lands as its pairs' rows of the first
+    // half, then of the second; s_qrow: where a quad's four rows of each half start.
+    for (int q = q0; q < q0 + nq;) {
+      const int j = q % qph, take = min(qph - j, q0 + nq - q);
+      tma_prefetch_desc(&maps.w[take - 1]);
+      for (int i = 0; i < take; ++i) {
+        s_qrow[2 * (q - q0 + i)] = static_cast<uint16_t>((q - q0) * 8 + i * 4);
+        s_qrow[2 * (q - q0 + i) + 1] = static_cast<uint16_t>((q - q0) * 8 + (take + i) * 4);
+      }
+      q += take;
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      for (int s = 0; s < p.stages; ++s) {
+        mbar_init(&full[s], 1);
+        mbar_init(&empty[s], 1);
+      }
+      mbar_init(acc_full, 1);
+      mbar_init(recv_full, 1);
+      fence_mbar_init();
+      if (n_own > 0) mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(n_own * L.row_stride * 4));
+    }
+    __syncwarp();
+    tmem_alloc(s_tmem, p.tmem_cols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // the peer runs: its shared memory may be written from here on
+  tc_fence_after();
+  // Inputs written by earlier kernels in the stream are visible from here on.
+  griddep_wait();
+  griddep_launch_dependents();
+  const uint32_t tmem = *s_tmem;
+  const int xoff = p.qmax * 1024;
+
+  if (warp == 0) {
+    // ============================ producer: TMA ============================
+    const bool leader = elect_one();
+    const uint64_t pol_w = l2_policy_evict_first();  // W streams once
+    const uint64_t pol_x = l2_policy_evict_last();   // x is re-read by every cluster
+    const uint32_t bytes = static_cast<uint32_t>(rows * 128 + p.Ncols * 128);
+    const int h_first = q0 / qph, j_first = q0 - h_first * qph;
+    int s = 0, issued = 0, kc = kc0 + rot;
+    uint32_t ph = 1;
+    bool ok = true;
+    for (; issued < nk; ++issued) {
+      ok = warp_wait(&empty[s], ph, s_abort);
+      if (!ok) break;
+      uint8_t *stage = smem + L.ring + s * L.stage_bytes;
+      const int kx = kc * kKChunk;
+      if (leader) mbar_arrive_expect_tx(&full[s], bytes);
+      // The range's pieces, one box per head.
+      for (int q = 0, h = h_first, j = j_first; q < nq; ++h, j = 0) {
+        const int take = min(qph - j, nq - q);
+        if (leader) tma_load_4d(stage + q * 1024, &maps.w[take - 1], kx, j * 4, 0, h, &full[s], pol_w);
+        q += take;
+      }
+      if (leader) tma_load_2d(stage + xoff, &maps.x, kx, 0, &full[s], pol_x);
+      if (++kc == kc0 + nk) kc = kc0;
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
+    }
+    if (!ok && leader) {
+      atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+      // Drain: every copy issued must land before shared memory goes away.
+      for (int i = (issued > p.stages ? issued - p.stages : 0); i < issued; ++i)
+        mbar_wait_unabortable(&full[i % p.stages], (i / p.stages) & 1);
+    }
+  } else if (warp == 1) {
+    // ============================ MMA issuer ===============================
+    const bool leader = elect_one();
+    const uint32_t idesc = idesc_bf16_f32(128, p.Ncols);
+    int s = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int it = 0; it < nk; ++it) {
+      ok &= warp_wait(&full[s], ph, s_abort);  // (after an expired wait the results are void, the waits no-ops)
+      tc_fence_after();
+      const uint32_t base = smem_u32(smem + L.ring + s * L.stage_bytes);
+      // Descriptors built once per operand; a K step of 16 adds 32 bytes, 2 in
+      // the descriptor's address field.
+      const uint64_t db = smem_desc_sw128(base + xoff);
+      for (int t = 0; t < ntile; ++t) {
+        const uint64_t da = smem_desc_sw128(base + t * kTileBytes);
+        const uint32_t d = tmem + static_cast<uint32_t>(t * p.Ncols);
+#pragma unroll
+        for (int kk = 0; kk < kKChunk / 16; ++kk)
+          if (leader) tc_mma_f16(d, da + 2u * kk, db + 2u * kk, idesc, (it > 0 || kk > 0) ? 1u : 0u);
+      }
+      if (leader) tc_commit(&empty[s]);
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
+    }
+    if (nk > 0 && leader) {
+      tc_commit(acc_full);
+      if (!ok) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+    }
+  } else {
+    // ===================== epilogue warps: stage the partial sums ==========
+    const int et = tid - 64, q4 = warp & 3, part = (warp - 2) >> 2;
+    build_rows(p.c, s_rseq, s_rpos, et, kEpiThreads, [] { epi_bar(); });
+    if (nk > 0) {
+      if (!mbar_wait(acc_full, 0, s_abort)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+      tc_fence_after();
+    }
+    // Two warps per lane quarter, each every second 16 columns.
+    const int R = p.c.R;
+    for (int t = 0; t < ntile; ++t) {
+      if (t * 128 + q4 * 32 >= rows) break;  // (whole warps: rows is a multiple of 8)
+      const int row = t * 128 + q4 * 32 + lane;
+      const uint32_t a = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(t * p.Ncols);
+      for (int c = 16 * part; c < p.Ncols; c += 32) {
+        uint32_t v[16];
+        if (nk > 0) {
+          tmem_ld8(a + c, v);
+          tmem_ld8(a + c + 8, v + 8);
+          tmem_wait_ld();
+        } else {  // (one k-chunk in all: this CTA has none)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) v[e] = 0u;
+        }
+        if (row < rows) {
+          float *to = reinterpret_cast<float *>(smem + L.part) + c * L.row_stride + row;
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            if (c + e < R) to[e * L.row_stride] = __uint_as_float(v[e]);
+        }
+      }
+    }
+    tc_fence_before();
+    // The peer's rows travel in one copy.
+    fence_proxy_async_smem();
+    epi_bar();
+    const uint8_t *send = smem + L.part + (rank ? 0 : h0) * L.row_stride * 4;
+    if (et == 0 && n_send > 0)
+      bulk_copy_cluster(cluster_map(smem + L.recv, rank ^ 1u), send, static_cast<uint32_t>(n_send * L.row_stride * 4),
+                        cluster_map(recv_full, rank ^ 1u));
+  }
+  __syncwarp();
+  __syncthreads();
+  {
+    const int n0 = rank ? h0 : 0;
+    const float *own = reinterpret_cast<const float *>(smem + L.part) + n0 * L.row_stride;
+    const float *recv = reinterpret_cast<const float *>(smem + L.recv);
+    if (n_own > 0 && !mbar_wait_unabortable(recv_full, 0)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+    const OutMap om = out_map(p.c);
+    for (int it = tid; it < n_own * nq; it += kThreads) {
+      const int n = it / nq, q = it - n * nq;
+      const int b = s_rseq[n0 + n];
+      if (b < 0) continue;
+      const int at1 = n * L.row_stride + s_qrow[2 * q], at2 = n * L.row_stride + s_qrow[2 * q + 1];
+      float y1[4], y2[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        y1[e] = own[at1 + e] + recv[at1 + e];
+        y2[e] = own[at2 + e] + recv[at2 + e];
+      }
+      const int Q = q0 + q, hg = Q / qph;
+      store_quad(om, s_freq, b, n0 + n, s_rpos[n0 + n], hg, (Q - hg * qph) * 4, y1, y2);
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, p.tmem_cols);
+  }
+  cluster_sync();  // the copy to the peer has left this CTA's shared memory
+}
+
+// W [(Hq + 2 Hkv) D, H] as {H, D / 2 pairs, 2 halves, heads}, box {64, pairs, 2, 1},
+// 128-byte swizzle.
+static bool encode_w(CUtensorMap *map, const void *w, const Call &c, uint32_t pairs) {
+  const uint64_t H = c.H, row = H * 2;
+  const uint64_t dims[4] = {H, static_cast<uint64_t>(c.D / 2), 2, static_cast<uint64_t>(c.Hq + 2 * c.Hkv)};
+  const uint64_t strides[3] = {row, row * (c.D / 2), row * c.D};
+  const uint32_t box[4] = {kKChunk, pairs, 2, 1};
+  return encode_tmap_bf16_sw128_nd(map, w, 4, dims, strides, box);
+}
+
+// Plan for these sizes; stages = 0 when the form does not take them.
+static Params plan(const Call &c, int sms) {
+  Params p{};
+  p.c = c;
+  p.quads = (c.Hq + 2 * c.Hkv) * c.D / 8;
+  p.nclusters = sms / 2 < p.quads ? sms / 2 : p.quads;
+  if (c.R > kMaxRows || p.nclusters < 1) return p;
+  p.qmax = (p.quads + p.nclusters - 1) / p.nclusters;
+  p.KC = (c.H + kKChunk - 1) / kKChunk;
+  p.Ncols = (c.R + 15) / 16 * 16;
+  const int cols = (p.qmax * 8 + 127) / 128 * p.Ncols;  // accumulator columns
+  if (cols > 512 || p.qmax > kMaxQuads) return p;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < static_cast<uint32_t>(cols)) p.tmem_cols *= 2;
+  const Layout L = layout(c.R, p.Ncols, p.qmax, 0);
+  const int n = (kSmemBudget - L.total) / L.stage_bytes;
+  p.stages = n > kMaxStages ? kMaxStages : n;
+  return p;
+}
+
+}  // namespace pair
+
+// The cluster form streams W at the rate its ring allows: it takes the call when
+// at least kMinStages fit (fewer rows, or ranges of fewer quads); larger calls
+// spend their time in the MMAs and the rows' traffic, and the stream-K form
+// gives an SM 128 rows of W per x row it loads.
+bool cluster_fits(const Call &c, int sms) { return pair::plan(c, sms).stages >= pair::kMinStages; }
+
+spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int sms, cudaStream_t stream) {
+  using namespace pair;
+  const Params p = plan(c, sms);
+  Maps m;
+  if (!encode_tmap_bf16_sw128(&m.x, x, c.H, c.R, static_cast<uint64_t>(c.H) * 2, kKChunk, p.Ncols)) return SPADE_ERR_CUDA;
+  // The piece sizes that some cluster's range has.
+  const int qph = c.D / 8;
+  uint32_t used = 0;
+  for (int cl = 0, q = 0; cl < p.nclusters; ++cl) {
+    const int end = static_cast<int>(static_cast<int64_t>(p.quads) * (cl + 1) / p.nclusters);
+    while (q < end) {
+      const int left = qph - q % qph, take = left < end - q ? left : end - q;
+      if (!(used >> (take - 1) & 1u) && !encode_w(&m.w[take - 1], w_qkv, c, 4 * take)) return SPADE_ERR_CUDA;
+      used |= 1u << (take - 1);
+      q += take;
+    }
+  }
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(qkv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(qkv_cluster)");
+    configured = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * p.nclusters);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = layout(c.R, p.Ncols, p.qmax, p.stages).total;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, qkv_cluster_kernel, p, m);
+  if (e != cudaSuccess) return cuda_fail(e, "qkv_cluster launch");
+  return SPADE_OK;
+}
+
+}  // namespace qkv
+}  // namespace spade

@@ -37,18 +37,12 @@
 //  * Programmatic dependent launch: barriers, tensor memory and tensor-map
 //    prefetch come before the wait on the previous kernel; the attention that
 //    follows may be scheduled while this kernel finishes.
-#include <cuda_bf16.h>
-
-#include <cstdint>
-
-#include "internal.h"
-#include "ptx.cuh"
+#include "qkv_common.cuh"
 
 namespace spade {
 namespace qkv {
 
 constexpr int kTileM = 128;                     // W rows per tile (MMA M)
-constexpr int kKChunk = 64;                     // k elements per 128-byte swizzled row
 constexpr int kWBytes = kTileM * kKChunk * 2;   // 16 KB: one W tile x one k-chunk
 constexpr int kMaxR = 512;                      // verify rows per call
 constexpr int kEpiWarps = 4;
@@ -59,16 +53,9 @@ constexpr int kMaxStages = 8;
 
 
 struct Params {
-  const int32_t *ctx_lens;
-  const int32_t *n_draft;
-  const int32_t *cu_q;
-  __nv_bfloat16 *q_out;    // [R, Hq, D]
-  __nv_bfloat16 *k_cache;  // [B, Hkv, cap, D] (or a pool, see block_table)
-  __nv_bfloat16 *v_cache;
-  int32_t *status;
+  Call c;
   float *partials;         // [num_ctas + tiles slots][Ncols][128] fp32 (workspace)
   int32_t *counters;       // [2][tiles]: parts published, slabs done; zero between calls (workspace)
-  int B, R, H, Hq, Hkv, D, cap, max_k;
   int tiles;    // (Hq + 2 Hkv) D / 128
   int KC;       // k-chunks (ceil(H / 64))
   int KG;       // k-chunks per ring stage at most (1 or 2; 2 only when H is a multiple of 64)
@@ -79,11 +66,6 @@ struct Params {
   int nbuf;     // accumulator buffers (2 when two fit in tensor memory)
   int slabs;    // row slabs per split tile in the final reduction
   uint32_t buf_cols, tmem_cols;
-  float inv_freq[64];  // theta^(-2j/D), j < D/2, rounded from double on the host
-  // Paged caches (block_table null: dense [B, Hkv, cap, D]): pools
-  // [num_pages, Hkv, page_size, D], block_table [B, max_pages].
-  const int32_t *block_table;
-  int page_size, max_pages, num_pages;
 };
 
 // Shared-memory plan (offsets from a 1024-byte aligned base).
@@ -131,19 +113,6 @@ __device__ __forceinline__ int add_acq_rel(int32_t *a, int v) {
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory"); }
 
 
-// Sine and cosine of pos * f: the product as an exact pair (a + e == pos * f),
-// reduced to [-pi, pi] with 2 pi split in two parts (Cody and Waite's method),
-// then the SFU's sine and cosine (accurate to a few 1e-7 on that interval).
-__device__ __forceinline__ void rope_angle(int pos, float f, float *sn, float *cs) {
-  const float x = static_cast<float>(pos);  // exact: positions are below 2^24
-  const float a = x * f;
-  const float e = fmaf(x, f, -a);
-  const float k = rintf(a * 0.15915494309189535f);           // 1 / (2 pi)
-  float r = fmaf(-k, 6.28318548202514648f, a);               // 2 pi rounded to float
-  r = fmaf(-k, -1.7484555314695172e-07f, r);                 // 2 pi minus that
-  __sincosf(r + e, sn, cs);
-}
-
 // The reduction of verify rows [r0, r1) of tile t once every part has been
 // published: for each row and each 4 consecutive dimension pairs of a head
 // (thread th of nth takes items th, th + nth, ...), the sum of the partials
@@ -156,12 +125,8 @@ template <int kIB, int kPB>
 __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq, const int32_t *s_rpos,
                                          const float *s_freq, int t, int c_first, int nparts, int r0,
                                          int r1, int th, int nth) {
-  // Every field used below in a local: the stores through dst could alias
-  // the parameter block as far as the compiler knows, and it would reload them.
-  const int D = p.D, Hq = p.Hq, Hkv = p.Hkv, cap = p.cap, Ncols = p.Ncols;
-  const int max_pages = p.max_pages, page_size = p.page_size;
-  const int32_t *block_table = p.block_table;
-  __nv_bfloat16 *q_out = p.q_out, *k_cache = p.k_cache, *v_cache = p.v_cache;
+  const OutMap om = out_map(p.c);
+  const int D = om.D, Ncols = p.Ncols;
   const float *partials = p.partials;
   const int half = D / 2;
   const int hpt = kTileM / D;  // heads per tile
@@ -210,37 +175,8 @@ __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq,
     for (int i = 0; i < kIB; ++i) {
       const int b = bb[i];
       if (b < 0) continue;
-      const int r = rr[i], j0 = jj[i];
-      const int hg = t * hpt + hl[i];  // head among the Hq + 2 Hkv of the projection
-      const int pos = s_rpos[r];
-      if (hg < Hq + Hkv) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float sn, cs;
-          rope_angle(pos, s_freq[j0 + e], &sn, &cs);
-          const float o1 = y1[i][e] * cs - y2[i][e] * sn, o2 = y2[i][e] * cs + y1[i][e] * sn;
-          y1[i][e] = o1;
-          y2[i][e] = o2;
-        }
-      }
-      __nv_bfloat16 *dst;
-      if (hg < Hq) {
-        dst = q_out + (static_cast<size_t>(r) * Hq + hg) * D;
-      } else {
-        const int hk = hg < Hq + Hkv ? hg - Hq : hg - Hq - Hkv;
-        __nv_bfloat16 *cache = hg < Hq + Hkv ? k_cache : v_cache;
-        if (block_table) {
-          const int pg = block_table[static_cast<int64_t>(b) * max_pages + pos / page_size];
-          dst = cache + ((static_cast<size_t>(pg) * Hkv + hk) * page_size + pos % page_size) * D;
-        } else {
-          dst = cache + ((static_cast<size_t>(b) * Hkv + hk) * cap + pos) * D;
-        }
-      }
-      // 4 bf16 = 8 bytes at each half (j0 a multiple of 4, rows 16-byte aligned).
-      *reinterpret_cast<uint2 *>(dst + j0) =
-          make_uint2(pack_bf16(y1[i][0], y1[i][1]), pack_bf16(y1[i][2], y1[i][3]));
-      *reinterpret_cast<uint2 *>(dst + j0 + half) =
-          make_uint2(pack_bf16(y2[i][0], y2[i][1]), pack_bf16(y2[i][2], y2[i][3]));
+      // (head among the Hq + 2 Hkv of the projection)
+      store_quad(om, s_freq, b, rr[i], s_rpos[rr[i]], t * hpt + hl[i], jj[i], y1[i], y2[i]);
     }
   }
 }
@@ -265,14 +201,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int *s_fin = reinterpret_cast<volatile int *>(smem + L.misc + 32);  // last tile, c_first, nparts; slab flag
 
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = uniform_warp();
   const int lane = tid & 31;
   const int u0 = range_lo(p.units, p.num_ctas, blockIdx.x);
   const int u1 = range_lo(p.units, p.num_ctas, blockIdx.x + 1);
 
   // ---- set-up that reads no input -----------------------------------------
   if (tid == 0) { *s_abort = 0; s_fin[0] = -1; }
-  for (int j = tid; j < 64; j += kThreads) s_freq[j] = p.inv_freq[j];
+  for (int j = tid; j < 64; j += kThreads) s_freq[j] = p.c.inv_freq[j];
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(p.KG > 1 ? &tm_w3 : &tm_w);
     tma_prefetch_desc(&tm_x0);
@@ -306,83 +242,86 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ============================ producer: TMA ============================
-    if (lane == 0) {
-      const uint64_t pol_w = l2_policy_evict_first();  // W streams once
-      const uint64_t pol_x = l2_policy_evict_last();   // x is re-read for every unit
-      const uint32_t xbytes = p.Ncols * 128;  // x rows of one k-chunk
-      bool expired = false;
-      int issued = 0;
-      for (int u = u0, i = 0; u < u1; ++i) {
-        const int st = i % p.stages;
-        const uint32_t ph = (i / p.stages) & 1;
-        if (!mbar_wait(&bar_empty[st], ph ^ 1, s_abort)) expired = true;
-        if (*s_abort) break;
-        issued = i + 1;
-        uint8_t *stage = smem + L.ring + st * L.stage_bytes;
-        const int t = u / p.KC, c0 = u - t * p.KC;
-        const int nch = min(p.KG, min(u1, (t + 1) * p.KC) - u);  // chunks of one tile and this range
-        mbar_arrive_expect_tx(&bar_full[st], nch * (kWBytes + xbytes));
-        if (nch > 1)
-          tma_load_3d(stage, &tm_w3, 0, t * kTileM, c0, &bar_full[st], pol_w);  // nch chunks, 16 KB apart
-        else
-          tma_load_2d(stage, &tm_w, c0 * kKChunk, t * kTileM, &bar_full[st], pol_w);
-        uint8_t *xs = stage + p.KG * kWBytes;
-        for (int j = 0; j < nch; ++j) {
-          tma_load_2d(xs + j * xbytes, &tm_x0, (c0 + j) * kKChunk, 0, &bar_full[st], pol_x);
-          if (n1) tma_load_2d(xs + j * xbytes + n0 * 128, &tm_x1, (c0 + j) * kKChunk, n0, &bar_full[st], pol_x);
+    const bool leader = elect_one();
+    const uint64_t pol_w = l2_policy_evict_first();  // W streams once
+    const uint64_t pol_x = l2_policy_evict_last();   // x is re-read for every unit
+    const uint32_t xbytes = p.Ncols * 128;  // x rows of one k-chunk
+    bool ok = true;
+    int issued = 0, st = 0, t = u0 / p.KC, c0 = u0 - t * p.KC;
+    uint32_t ph = 1;
+    for (int u = u0; u < u1; ++issued) {
+      ok = warp_wait(&bar_empty[st], ph, s_abort);
+      if (!ok) break;
+      uint8_t *stage = smem + L.ring + st * L.stage_bytes;
+      const int nch = min(p.KG, min(u1 - u, p.KC - c0));  // chunks of one tile and this range
+      if (leader) mbar_arrive_expect_tx(&bar_full[st], nch * (kWBytes + xbytes));
+      if (nch > 1) {
+        if (leader) tma_load_3d(stage, &tm_w3, 0, t * kTileM, c0, &bar_full[st], pol_w);  // nch chunks, 16 KB apart
+      } else {
+        if (leader) tma_load_2d(stage, &tm_w, c0 * kKChunk, t * kTileM, &bar_full[st], pol_w);
+      }
+      uint8_t *xs = stage + p.KG * kWBytes;
+      for (int j = 0; j < nch; ++j) {
+        if (leader) tma_load_2d(xs + j * xbytes, &tm_x0, (c0 + j) * kKChunk, 0, &bar_full[st], pol_x);
+        if (n1) {
+          if (leader) tma_load_2d(xs + j * xbytes + n0 * 128, &tm_x1, (c0 + j) * kKChunk, n0, &bar_full[st], pol_x);
         }
-        u += nch;
       }
-      if (expired || *s_abort) {
-        atomicOr(p.status, SPADE_DEV_TIMEOUT);
-        // Drain: every copy issued must land before shared memory goes away.
-        for (int i = (issued > p.stages ? issued - p.stages : 0); i < issued; ++i)
-          mbar_wait_unabortable(&bar_full[i % p.stages], (i / p.stages) & 1);
-      }
+      u += nch;
+      c0 += nch;
+      if (c0 == p.KC) { c0 = 0; ++t; }
+      if (++st == p.stages) { st = 0; ph ^= 1u; }
+    }
+    if (!ok && leader) {
+      atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+      // Drain: every copy issued must land before shared memory goes away.
+      for (int i = (issued > p.stages ? issued - p.stages : 0); i < issued; ++i)
+        mbar_wait_unabortable(&bar_full[i % p.stages], (i / p.stages) & 1);
     }
   } else if (warp == 1) {
     // ============================ MMA issuer ===============================
-    if (lane == 0) {
-      const uint32_t idesc0 = idesc_bf16_f32(kTileM, n0);
-      const uint32_t idesc1 = idesc_bf16_f32(kTileM, n1 ? n1 : 16);
-      bool expired = false;
-      int i = 0, seg = 0;
-      for (int u = u0; u < u1; ++seg) {
-        const int t = u / p.KC;
-        const int se = min(u1, (t + 1) * p.KC);
-        const int buf = seg % p.nbuf, use = seg / p.nbuf;
-        // The buffer's previous segment has been drained by the epilogue warps.
-        if (use > 0 && !mbar_wait(&acc_empty[buf], (use - 1) & 1, s_abort)) expired = true;
+    const bool leader = elect_one();
+    const uint32_t idesc0 = idesc_bf16_f32(kTileM, n0);
+    const uint32_t idesc1 = idesc_bf16_f32(kTileM, n1 ? n1 : 16);
+    bool ok = true;  // (after an expired wait the results are void and the waits no-ops)
+    int st = 0, buf = 0, use = 0, c0 = u0 % p.KC;
+    uint32_t ph = 0;
+    for (int u = u0; u < u1;) {
+      const int len = min(u1 - u, p.KC - c0);  // this segment's chunks
+      // The buffer's previous segment has been drained by the epilogue warps.
+      if (use > 0) ok &= warp_wait(&acc_empty[buf], (use - 1) & 1, s_abort);
+      tc_fence_after();
+      const uint32_t acc_addr = tmem + static_cast<uint32_t>(buf) * p.buf_cols;
+      for (int done = 0; done < len;) {
+        const int nch = min(p.KG, len - done);  // as the producer cut the stage
+        ok &= warp_wait(&bar_full[st], ph, s_abort);
         tc_fence_after();
-        const uint32_t acc_addr = tmem + static_cast<uint32_t>(buf) * p.buf_cols;
-        for (const int us = u; u < se; ++i) {
-          const int st = i % p.stages;
-          const uint32_t ph = (i / p.stages) & 1;
-          const int nch = min(p.KG, se - u);  // as the producer cut the stage
-          if (!mbar_wait(&bar_full[st], ph, s_abort)) expired = true;
-          tc_fence_after();
-          if (!*s_abort) {
-            const uint32_t a0 = smem_base + L.ring + st * L.stage_bytes;
-            for (int j = 0; j < nch; ++j) {
-              const uint32_t a = a0 + j * kWBytes;
-              const uint32_t b = a0 + p.KG * kWBytes + j * p.Ncols * 128;
+        const uint32_t a0 = smem_base + L.ring + st * L.stage_bytes;
+        for (int j = 0; j < nch; ++j) {
+          const uint32_t a = a0 + j * kWBytes;
+          const uint32_t b = a0 + p.KG * kWBytes + j * p.Ncols * 128;
+          // Descriptors built once per chunk; a K step of 16 adds 32 bytes,
+          // 2 in the descriptor's address field.
+          const uint64_t da = smem_desc_sw128(a), db = smem_desc_sw128(b), db1 = smem_desc_sw128(b + n0 * 128);
 #pragma unroll
-              for (int kk = 0; kk < kKChunk / 16; ++kk) {
-                const uint32_t acc = (u > us || j > 0 || kk > 0) ? 1u : 0u;
-                tc_mma_f16(acc_addr, smem_desc_sw128(a + kk * 32), smem_desc_sw128(b + kk * 32), idesc0, acc);
-                if (n1)
-                  tc_mma_f16(acc_addr + 256, smem_desc_sw128(a + kk * 32),
-                             smem_desc_sw128(b + n0 * 128 + kk * 32), idesc1, acc);
-              }
+          for (int kk = 0; kk < kKChunk / 16; ++kk) {
+            const uint32_t acc = (done > 0 || j > 0 || kk > 0) ? 1u : 0u;
+            if (leader) tc_mma_f16(acc_addr, da + 2u * kk, db + 2u * kk, idesc0, acc);
+            if (n1) {
+              if (leader) tc_mma_f16(acc_addr + 256, da + 2u * kk, db1 + 2u * kk, idesc1, acc);
             }
           }
-          tc_commit(&bar_empty[st]);
-          u += nch;
         }
-        tc_commit(&acc_full[buf]);
+        if (leader) tc_commit(&bar_empty[st]);
+        done += nch;
+        if (++st == p.stages) { st = 0; ph ^= 1u; }
       }
-      if (expired) atomicOr(p.status, SPADE_DEV_TIMEOUT);
+      if (leader) tc_commit(&acc_full[buf]);
+      u += len;
+      c0 = 0;
+      if (++buf == p.nbuf) { buf = 0; ++use; }
     }
+    if (!ok && leader) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
   } else {
     // ===================== epilogue warps: drain, publish, reduce ==========
     const int et = tid - 64;         // 0..127
@@ -390,31 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Row table: sequence and position of every verify row.  Only the tile
     // reductions read it, so it is built here while the producer and the MMA
     // warp already stream the first units.
-    for (int r = et; r < p.R; r += kEpiThreads) s_rseq[r] = -1;
-    epi_bar();
-    for (int b = et; b < p.B; b += kEpiThreads) {
-      const int c = p.ctx_lens[b], k = p.n_draft[b];
-      const int q0 = p.cu_q[b], q1 = p.cu_q[b + 1];
-      int bad = 0;
-      if (c < 0 || k < 0 || k > p.max_k || q0 < 0 || q1 > p.R || q1 - q0 != k + 1) bad = SPADE_DEV_BAD_INDEX;
-      else if (static_cast<int64_t>(c) + k + 1 > p.cap) bad = SPADE_DEV_CAPACITY;
-      if (!bad && p.block_table) {
-        // Every page the block writes must exist.
-        for (int i = 0; i <= k; ++i) {
-          const int pg = p.block_table[static_cast<int64_t>(b) * p.max_pages + (c + i) / p.page_size];
-          if (pg < 0 || pg >= p.num_pages) bad = SPADE_DEV_BAD_INDEX;
-        }
-      }
-      if (bad) {
-        if (blockIdx.x == 0) atomicOr(p.status, bad);
-        continue;
-      }
-      for (int i = 0; i <= k; ++i) {
-        s_rseq[q0 + i] = b;
-        s_rpos[q0 + i] = c + i;
-      }
-    }
-    epi_bar();
+    build_rows(p.c, s_rseq, s_rpos, et, kEpiThreads, [] { __syncwarp(); epi_bar(); });
     bool expired = false;
     int seg = 0;
     for (int u = u0; u < u1; ++seg) {
@@ -426,12 +341,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       // Accumulator -> this CTA's slot [Ncols][128] of the tile's partials.
       float *part = p.partials + static_cast<size_t>(blockIdx.x + t) * p.Ncols * kTileM;
       const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(buf) * p.buf_cols;
-      for (int c = 0; c < p.Ncols; c += 8) {
-        uint32_t v[8];
-        tmem_ld8(tl + c, v);
+      float *out = part + q4 * 32 + lane;
+      int c = 0;
+#pragma unroll 1
+      for (; c + 32 <= p.Ncols; c += 32) {  // four loads behind one wait
+        uint32_t v[32];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) tmem_ld8(tl + c + 8 * j, v + 8 * j);
         tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) __stcg(part + (c + e) * kTileM + q4 * 32 + lane, __uint_as_float(v[e]));
+        for (int e = 0; e < 32; ++e) __stcg(out + (c + e) * kTileM, __uint_as_float(v[e]));
+      }
+      if (c < p.Ncols) {  // the last 16 columns
+        uint32_t v[16];
+        tmem_ld8(tl + c, v);
+        tmem_ld8(tl + c + 8, v + 8);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) __stcg(out + (c + e) * kTileM, __uint_as_float(v[e]));
       }
       tc_fence_before();
       __syncwarp();
@@ -454,16 +381,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (et == 0) { s_fin[0] = t; s_fin[1] = c_first; s_fin[2] = nparts; }
           } else {
             if (nparts == 1)
-              reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.R, et, kEpiThreads);
+              reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, et, kEpiThreads);
             else
-              reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.R, et, kEpiThreads);
+              reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, et, kEpiThreads);
             if (et == 0 && nparts > 1) p.counters[t] = 0;  // every part has arrived: reset for the next call
           }
         }
       }
       u = se;
     }
-    if (expired) atomicOr(p.status, SPADE_DEV_TIMEOUT);
+    if (expired) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
   }
   // The CTA's last tile, if this CTA finishes it, with every thread.
   __syncwarp();
@@ -471,9 +398,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (s_fin[0] >= 0) {
     const int t = s_fin[0], c_first = s_fin[1], nparts = s_fin[2];
     if (nparts == 1)
-      reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.R, tid, kThreads);
+      reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, tid, kThreads);
     else
-      reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.R, tid, kThreads);
+      reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, tid, kThreads);
     if (tid == 0 && nparts > 1) p.counters[t] = 0;  // every part has arrived: reset for the next call
   }
   // Row slabs of the split tiles (slabs > 1): item i = t * slabs + s goes to
@@ -492,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t t0 = globaltimer();
         while (load_acquire(&published[t]) != nparts) {
           if (globaltimer() - t0 > kWaitLimitNs) {
-            atomicOr(p.status, SPADE_DEV_TIMEOUT);
+            atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
             s_fin[3] = 0;
             break;
           }
@@ -502,8 +429,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     const int ok = s_fin[3];
     if (ok) {
-      const int r0 = static_cast<int>(static_cast<int64_t>(p.R) * sl / p.slabs);
-      const int r1 = static_cast<int>(static_cast<int64_t>(p.R) * (sl + 1) / p.slabs);
+      const int r0 = static_cast<int>(static_cast<int64_t>(p.c.R) * sl / p.slabs);
+      const int r1 = static_cast<int>(static_cast<int64_t>(p.c.R) * (sl + 1) / p.slabs);
       reduce_tile<2, 6>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, r0, r1, tid, kThreads);
     }
     __syncthreads();  // every load of the parts is done
@@ -580,20 +507,23 @@ static spade_status qkv_rope_impl(const void *x, const void *w_qkv, const int32_
                 workspace_bytes);
 
   Params p{};
-  p.ctx_lens = ctx_lens;
-  p.n_draft = n_draft;
-  p.cu_q = cu_q;
-  p.q_out = static_cast<__nv_bfloat16 *>(q_out);
-  p.k_cache = static_cast<__nv_bfloat16 *>(k_cache);
-  p.v_cache = static_cast<__nv_bfloat16 *>(v_cache);
-  p.status = status;
+  Call &c = p.c;
+  c.ctx_lens = ctx_lens;
+  c.n_draft = n_draft;
+  c.cu_q = cu_q;
+  c.q_out = static_cast<__nv_bfloat16 *>(q_out);
+  c.k_cache = static_cast<__nv_bfloat16 *>(k_cache);
+  c.v_cache = static_cast<__nv_bfloat16 *>(v_cache);
+  c.status = status;
+  c.B = B; c.R = R; c.H = H; c.Hq = Hq; c.Hkv = Hkv; c.D = D; c.cap = cap; c.max_k = max_k;
+  c.block_table = pg ? pg->block_table : nullptr;
+  c.page_size = pg ? pg->page_size : 0;
+  c.max_pages = pg ? pg->max_pages : 0;
+  c.num_pages = pg ? pg->num_pages : 0;
+  for (int j = 0; j < D / 2; ++j) c.inv_freq[j] = static_cast<float>(pow(static_cast<double>(rope_theta), -2.0 * j / D));
+  if (cluster_fits(c, sms)) return launch_cluster(c, x, w_qkv, sms, reinterpret_cast<cudaStream_t>(stream));
   p.counters = static_cast<int32_t *>(workspace);
   p.partials = reinterpret_cast<float *>(static_cast<uint8_t *>(workspace) + counter_bytes(tiles));
-  p.B = B; p.R = R; p.H = H; p.Hq = Hq; p.Hkv = Hkv; p.D = D; p.cap = cap; p.max_k = max_k;
-  p.block_table = pg ? pg->block_table : nullptr;
-  p.page_size = pg ? pg->page_size : 0;
-  p.max_pages = pg ? pg->max_pages : 0;
-  p.num_pages = pg ? pg->num_pages : 0;
   p.tiles = tiles;
   p.KC = (H + kKChunk - 1) / kKChunk;
   p.Ncols = (R + 15) / 16 * 16;
@@ -601,7 +531,6 @@ static spade_status qkv_rope_impl(const void *x, const void *w_qkv, const int32_
   while (p.buf_cols < static_cast<uint32_t>(p.Ncols)) p.buf_cols *= 2;
   p.nbuf = p.buf_cols * 2 <= 512 ? 2 : 1;
   p.tmem_cols = p.buf_cols * p.nbuf;
-  for (int j = 0; j < D / 2; ++j) p.inv_freq[j] = static_cast<float>(pow(static_cast<double>(rope_theta), -2.0 * j / D));
   // Stages of up to two k-chunks when H allows the 3-D view and the ring
   // still holds three of them; otherwise one chunk per stage.
   p.KG = 1;

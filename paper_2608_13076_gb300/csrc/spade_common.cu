@@ -67,8 +67,8 @@ EncodeFn g_encode = nullptr;
 std::once_flag g_encode_once;
 }  // namespace
 
-bool encode_tmap_bf16_sw128(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
-                            uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_rows) {
+bool encode_tmap_bf16_sw128_nd(CUtensorMap *map, const void *base, uint32_t rank, const uint64_t *dims,
+                               const uint64_t *strides_bytes, const uint32_t *box) {
   std::call_once(g_encode_once, [] {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -81,51 +81,37 @@ bool encode_tmap_bf16_sw128(CUtensorMap *map, const void *base, uint64_t inner, 
     fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     return false;
   }
-  cuuint64_t dims[2] = {inner, rows};
-  cuuint64_t strides[1] = {row_stride_bytes};
-  cuuint32_t box[2] = {box_inner, box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  cuuint64_t d[5], s[4];
+  cuuint32_t b[5], es[5];
+  for (uint32_t i = 0; i < rank; ++i) {
+    d[i] = dims[i];
+    b[i] = box[i];
+    es[i] = 1;
+    if (i + 1 < rank) s[i] = strides_bytes[i];
+  }
+  const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), d, s, b, es,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
-    fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d) for [%llu x %llu] box %u x %u",
-         static_cast<int>(r), (unsigned long long)rows, (unsigned long long)inner, box_rows,
-         box_inner);
+    fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d): %u-D, inner %llu, rows %llu, box %u x %u",
+         static_cast<int>(r), rank, (unsigned long long)dims[0], (unsigned long long)dims[1], box[0], box[1]);
     return false;
   }
   return true;
 }
 
+bool encode_tmap_bf16_sw128(CUtensorMap *map, const void *base, uint64_t inner, uint64_t rows,
+                            uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_rows) {
+  const uint64_t dims[2] = {inner, rows}, strides[1] = {row_stride_bytes};
+  const uint32_t box[2] = {box_inner, box_rows};
+  return encode_tmap_bf16_sw128_nd(map, base, 2, dims, strides, box);
+}
+
 bool encode_tmap_rows_by_slab(CUtensorMap *map, const void *base, uint64_t rows, uint32_t cols,
                               uint32_t box_rows, uint32_t box_slabs) {
-  std::call_once(g_encode_once, [] {
-    void *fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      g_encode = reinterpret_cast<EncodeFn>(fn);
-  });
-  if (!g_encode) {
-    fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    return false;
-  }
-  cuuint64_t dims[3] = {64, rows, cols / 64};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 2, 128};
-  cuuint32_t box[3] = {64, box_rows, box_slabs ? box_slabs : cols / 64};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
-                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled (row slabs) failed (%d) for [%llu x %u]",
-         static_cast<int>(r), (unsigned long long)rows, cols);
-    return false;
-  }
-  return true;
+  const uint64_t dims[3] = {64, rows, cols / 64}, strides[2] = {static_cast<uint64_t>(cols) * 2, 128};
+  const uint32_t box[3] = {64, box_rows, box_slabs ? box_slabs : cols / 64};
+  return encode_tmap_bf16_sw128_nd(map, base, 3, dims, strides, box);
 }
 
 // One thread waits on an mbarrier that nothing completes, bounded as every
