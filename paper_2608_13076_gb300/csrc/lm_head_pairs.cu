@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.off_misc + 8);
   const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, false);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int c = blockIdx.x;
   const uint32_t rank = cluster_ctarank();
   const int v_lo = static_cast<int>(static_cast<int64_t>(c) * p.c.V / p.c.NC);
@@ -109,79 +109,88 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
   const int k_rot = (c >> 1) % p.KC;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // Both CTAs' copies of a stage complete on the even CTA's full barrier,
-      // armed with the bytes of both before either CTA may issue them (at
-      // set-up, then by the MMA thread as it takes the previous use).
-      const uint64_t pol_w = l2_policy_evict_first(), pol_h = l2_policy_evict_last();
-      const uint32_t full0 = cluster_map(full, 0);
-      const int hrow0 = static_cast<int>(rank) * (p.n0w / 2);
-      const int hrow1 = p.n0w + static_cast<int>(rank) * (p.n1w / 2);
-      uint32_t i = 0, issued = 0, eph = 1;
-      int s = 0;
-      for (int t = 0; t < p.ntiles; ++t) {
-        const int row0 = v_lo + t * p.th;
-        for (int it = 0; it < p.KC; ++it, ++i) {
-          const int kc = it + k_rot < p.KC ? it + k_rot : it + k_rot - p.KC;
-          mbar_wait(&empty[s], eph, s_abort);
-          if (!*s_abort) {
-            uint8_t *dst = smem + s * L.stage;
-            const uint32_t bar = full0 + 8u * s;
-            tma_load_2d_pair(dst, &tm_w, kc * kKChunk, row0, bar, pol_w);
-            tma_load_2d_pair(dst + kWChunkBytes, &tm_h0, kc * kKChunk, hrow0, bar, pol_h);
-            if (p.n1w) tma_load_2d_pair(dst + h1_off, &tm_h1, kc * kKChunk, hrow1, bar, pol_h);
-            issued = i + 1;
-          }
-          if (++s == p.stages) { s = 0; eph ^= 1u; }
+    // Both CTAs' copies of a stage complete on the even CTA's full barrier,
+    // armed with the bytes of both before either CTA may issue them (at
+    // set-up, then by the MMA warp as it takes the previous use).
+    const bool leader = elect_one();
+    const uint64_t pol_w = l2_policy_evict_first(), pol_h = l2_policy_evict_last();
+    const uint32_t full0 = cluster_map(full, 0);
+    const int hrow0 = static_cast<int>(rank) * (p.n0w / 2);
+    const int hrow1 = p.n0w + static_cast<int>(rank) * (p.n1w / 2);
+    uint32_t issued = 0, eph = 1;
+    int s = 0;
+    bool ok = true;
+    for (int t = 0; ok && t < p.ntiles; ++t) {
+      const int row0 = v_lo + t * p.th;
+      int kc = k_rot;
+      for (int it = 0; it < p.KC; ++it) {
+        ok = warp_wait(&empty[s], eph, s_abort);
+        if (!ok) break;
+        uint8_t *dst = smem + s * L.stage;
+        const uint32_t bar = full0 + 8u * s;
+        const int kx = kc * kKChunk;
+        if (leader) {
+          tma_load_2d_pair(dst, &tm_w, kx, row0, bar, pol_w);
+          tma_load_2d_pair(dst + kWChunkBytes, &tm_h0, kx, hrow0, bar, pol_h);
         }
-      }
-      // After an expired wait the even CTA drains the copies of both (its full
-      // barriers count them); the odd CTA's shared memory stays alive until the
-      // teardown handshake with the even CTA.
-      if (*s_abort && rank == 0) {
-        const uint32_t n = p.stages;
-        for (uint32_t j = (issued > n ? issued - n : 0); j < issued; ++j)
-          mbar_wait_unabortable(&full[j % n], (j / n) & 1);
+        if (p.n1w) {
+          if (leader) tma_load_2d_pair(dst + h1_off, &tm_h1, kx, hrow1, bar, pol_h);
+        }
+        ++issued;
+        if (++kc == p.KC) kc = 0;
+        if (++s == p.stages) { s = 0; eph ^= 1u; }
       }
     }
+    // After an expired wait the even CTA drains the copies of both (its full
+    // barriers count them); the odd CTA's shared memory stays alive until the
+    // teardown handshake with the even CTA.
+    if (!ok && rank == 0 && leader) {
+      const uint32_t n = p.stages;
+      for (uint32_t j = (issued > n ? issued - n : 0); j < issued; ++j)
+        mbar_wait_unabortable(&full[j % n], (j / n) & 1);
+    }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // Even CTA: M = 256 MMAs over both CTAs' stages; the stages are freed in
-      // both CTAs by one multicast commit.
+      // both CTAs by one multicast commit.  (After an expired wait the results
+      // are void and the waits no-ops.)
+      const bool leader = elect_one();
       int s = 0;
       uint32_t ph = 0;
       for (int t = 0; t < p.ntiles; ++t) {
         const int buf = p.nacc == 2 ? t & 1 : 0, use = p.nacc == 2 ? t >> 1 : t;
         const uint32_t d0 = tmem + static_cast<uint32_t>(buf * (kTmemCols / 2));
-        if (use > 0) mbar_wait_cluster(&acc_empty[buf], (use - 1) & 1, s_abort);
+        const uint32_t d1 = d0 + static_cast<uint32_t>(p.n0w);
+        if (use > 0) {
+          if (leader) mbar_wait_cluster(&acc_empty[buf], (use - 1) & 1, s_abort);
+          __syncwarp();
+        }
         tc_fence_after();
         for (int it = 0; it < p.KC; ++it) {
           // (cta-scope wait: the copies' completion on this barrier orders them
           // for the MMAs issued after it, the odd CTA's included)
-          mbar_wait(&full[s], ph, s_abort);
+          warp_wait(&full[s], ph, s_abort);
           // Arm the stage's next use now: its copies are issued only after this
           // use's commit frees the stage.
-          mbar_arrive_expect_tx(&full[s], 2 * stage_tx);
+          if (leader) mbar_arrive_expect_tx(&full[s], 2 * stage_tx);
           tc_fence_after();
           const uint32_t base = smem_u32(smem + s * L.stage);
           const uint64_t da = smem_desc_sw128(base), db0 = smem_desc_sw128(base + kWChunkBytes);
+          const uint64_t db1 = smem_desc_sw128(base + h1_off);
 #pragma unroll
-          for (int k16 = 0; k16 < kKChunk / 16; ++k16)
-            tc_mma_f16_pair(d0, da + 2u * k16, db0 + 2u * k16, p.idesc0, (it | k16) != 0);
-          if (p.n1w) {
-            const uint64_t db1 = smem_desc_sw128(base + h1_off);
-#pragma unroll
-            for (int k16 = 0; k16 < kKChunk / 16; ++k16)
-              tc_mma_f16_pair(d0 + static_cast<uint32_t>(p.n0w), da + 2u * k16, db1 + 2u * k16, p.idesc1,
-                              (it | k16) != 0);
+          for (int k16 = 0; k16 < kKChunk / 16; ++k16) {
+            if (leader) tc_mma_f16_pair(d0, da + 2u * k16, db0 + 2u * k16, p.idesc0, (it | k16) != 0);
+            if (p.n1w) {
+              if (leader) tc_mma_f16_pair(d1, da + 2u * k16, db1 + 2u * k16, p.idesc1, (it | k16) != 0);
+            }
           }
-          tc_commit_pair(&empty[s]);
+          if (leader) tc_commit_pair(&empty[s]);
           if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
-        tc_commit_pair(&acc_full[buf]);
+        if (leader) tc_commit_pair(&acc_full[buf]);
         ++tiles_issued;
       }
-    } else if (lane == 0) {
+    } else {
       tiles_issued = p.ntiles;  // odd CTA: the even CTA's commits reach its acc_full too
     }
   } else {

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
   SeqTable &seqs = *reinterpret_cast<SeqTable *>(smem + L.off_seq);
   const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, true);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int c = blockIdx.x;
   // This CTA's vocabulary slice [v_lo, v_hi): equal row counts (within one),
   // cut into 128-row tiles; the last tile may be partial.
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
   griddep_wait();
   griddep_launch_dependents();
   const uint32_t tmem = *s_tmem;
-  int rounds_issued = 0;  // MMA thread: accumulator rounds committed
+  int rounds_issued = 0;  // MMA warp: accumulator rounds committed
   // Every CTA reads the same hidden rows: CTA c walks the K stages starting at
   // stage c mod NS, so at any moment about NC / NS CTAs (not all of them) load
   // the same hidden lines from L2.  Each logit's sum over K changes order only.
@@ -135,129 +135,127 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
 
   // ======================= phase A: logits + slice statistics =============
   if (warp == 0) {
-    if (lane == 0 && ntiles > 0) {
-      const uint64_t pol_w = l2_policy_evict_first();
-      const uint64_t pol_h = l2_policy_evict_last();
-      uint32_t wi = 0, hi = 0, w_issued = 0, h_issued = 0;
-      // Ring slots and parities advance by counters (no per-stage divisions).
-      int ws_ = 0, hs_ = 0;
-      uint32_t wph_ = 0, hph_ = 0;
-      int tdone = 0;
-      for (int r = 0; r < p.nrounds && tdone < ntiles; ++r) {
-        const int nt = min(p.round_tiles[r], ntiles - tdone);
-        for (int it = 0; it < p.NS; ++it) {
-          const int ks = it + k_rot < p.NS ? it + k_rot : it + k_rot - p.NS;
-          const int c0 = ks * p.KG;
-          const int nch = min(p.KG, p.KC - c0);
-          const bool box3 = (nch == p.KG) && (c0 + p.KG <= p.KCF);
-          {
-            const int s = hs_;
-            mbar_wait(&h_empty[s], hph_ ^ 1, s_abort);
-            if (!*s_abort) {
-              uint8_t *dst = h_ring + s * L.h_slot;
-              const int hk = p.Ncols * 128;  // bytes per k-chunk
-              mbar_arrive_expect_tx(&h_full[s], nch * hk);
-              if (box3) {
-                tma_load_3d(dst, &tm_h3, 0, 0, c0, &h_full[s], pol_h);
-              } else {
-                for (int j = 0; j < nch; ++j)
-                  tma_load_2d(dst + j * hk, &tm_h2, (c0 + j) * kKChunk, 0, &h_full[s], pol_h);
-              }
-              h_issued = hi + 1;
+    const bool leader = elect_one();
+    const uint64_t pol_w = l2_policy_evict_first();
+    const uint64_t pol_h = l2_policy_evict_last();
+    const uint32_t hk = p.Ncols * 128;  // hidden bytes per k-chunk
+    uint32_t w_issued = 0, h_issued = 0;
+    // Ring slots and parities advance by counters (no per-stage divisions).
+    int ws = 0, hs = 0;
+    uint32_t wph = 1, hph = 1;
+    bool ok = true;
+    int tdone = 0;
+    for (int r = 0; ok && r < p.nrounds && tdone < ntiles; ++r) {
+      const int nt = min(p.round_tiles[r], ntiles - tdone);
+      int ks = k_rot;
+      for (int it = 0; ok && it < p.NS; ++it) {
+        const int c0 = ks * p.KG;
+        const int nch = min(p.KG, p.KC - c0);
+        const bool box3 = (nch == p.KG) && (c0 + p.KG <= p.KCF);
+        if (++ks == p.NS) ks = 0;
+        ok = warp_wait(&h_empty[hs], hph, s_abort);
+        if (!ok) break;
+        {
+          uint8_t *dst = h_ring + hs * L.h_slot;
+          if (leader) {
+            mbar_arrive_expect_tx(&h_full[hs], nch * hk);
+            if (box3) {
+              tma_load_3d(dst, &tm_h3, 0, 0, c0, &h_full[hs], pol_h);
+            } else {
+              for (int j = 0; j < nch; ++j)
+                tma_load_2d(dst + j * hk, &tm_h2, (c0 + j) * kKChunk, 0, &h_full[hs], pol_h);
             }
-            ++hi;
-            if (++hs_ == p.HS) { hs_ = 0; hph_ ^= 1u; }
           }
-          for (int j = 0; j < nt; ++j) {
-            const int s = ws_;
-            mbar_wait(&w_empty[s], wph_ ^ 1, s_abort);
-            if (!*s_abort) {
-              uint8_t *dst = w_ring + s * L.w_slot;
-              const int row0 = v_lo + (tdone + j) * kTileV;
-              if (short_last && tdone + j == ntiles - 1) {
-                // Partial last tile: BRS-row boxes (BRS a multiple of 8), the k-chunks
-                // packed at BRS * 128-byte strides: one 3-D box per stage when it
-                // holds KG full chunks (small 2-D boxes stream far slower).  The
-                // slot's remaining rows feed accumulator lanes that are never read.
-                mbar_arrive_expect_tx(&w_full[s], nch * p.BRS * 128);
-                if (box3) {
-                  tma_load_3d(dst, &tm_w3s, 0, row0, c0, &w_full[s], pol_w);
-                } else {
-                  for (int jj = 0; jj < nch; ++jj)
-                    tma_load_2d(dst + jj * p.BRS * 128, &tm_w2s, (c0 + jj) * kKChunk, row0, &w_full[s], pol_w);
-                }
-              } else if (box3) {
-                mbar_arrive_expect_tx(&w_full[s], nch * kWChunkBytes);
-                tma_load_3d(dst, &tm_w3, 0, row0, c0, &w_full[s], pol_w);
-              } else {
-                mbar_arrive_expect_tx(&w_full[s], nch * kWChunkBytes);
-                for (int jj = 0; jj < nch; ++jj)
-                  tma_load_2d(dst + jj * kWChunkBytes, &tm_w2, (c0 + jj) * kKChunk, row0, &w_full[s], pol_w);
-              }
-              w_issued = wi + 1;
-            }
-            ++wi;
-            if (++ws_ == p.WS) { ws_ = 0; wph_ ^= 1u; }
-          }
+          ++h_issued;
+          if (++hs == p.HS) { hs = 0; hph ^= 1u; }
         }
-        tdone += nt;
+        for (int j = 0; j < nt; ++j) {
+          ok = warp_wait(&w_empty[ws], wph, s_abort);
+          if (!ok) break;
+          uint8_t *dst = w_ring + ws * L.w_slot;
+          const int row0 = v_lo + (tdone + j) * kTileV;
+          if (short_last && tdone + j == ntiles - 1) {
+            // Partial last tile: BRS-row boxes (BRS a multiple of 8), the k-chunks
+            // packed at BRS * 128-byte strides: one 3-D box per stage when it
+            // holds KG full chunks (small 2-D boxes stream far slower).  The
+            // slot's remaining rows feed accumulator lanes that are never read.
+            if (leader) {
+              mbar_arrive_expect_tx(&w_full[ws], nch * p.BRS * 128);
+              if (box3) {
+                tma_load_3d(dst, &tm_w3s, 0, row0, c0, &w_full[ws], pol_w);
+              } else {
+                for (int jj = 0; jj < nch; ++jj)
+                  tma_load_2d(dst + jj * p.BRS * 128, &tm_w2s, (c0 + jj) * kKChunk, row0, &w_full[ws], pol_w);
+              }
+            }
+          } else if (leader) {
+            mbar_arrive_expect_tx(&w_full[ws], nch * kWChunkBytes);
+            if (box3) {
+              tma_load_3d(dst, &tm_w3, 0, row0, c0, &w_full[ws], pol_w);
+            } else {
+              for (int jj = 0; jj < nch; ++jj)
+                tma_load_2d(dst + jj * kWChunkBytes, &tm_w2, (c0 + jj) * kKChunk, row0, &w_full[ws], pol_w);
+            }
+          }
+          ++w_issued;
+          if (++ws == p.WS) { ws = 0; wph ^= 1u; }
+        }
       }
-      if (*s_abort) {
-        // Every copy issued must land before the CTA's shared memory goes away.
-        for (uint32_t j = (w_issued > (uint32_t)p.WS ? w_issued - p.WS : 0); j < w_issued; ++j)
-          mbar_wait_unabortable(&w_full[j % p.WS], (j / p.WS) & 1);
-        for (uint32_t j = (h_issued > (uint32_t)p.HS ? h_issued - p.HS : 0); j < h_issued; ++j)
-          mbar_wait_unabortable(&h_full[j % p.HS], (j / p.HS) & 1);
-      }
+      tdone += nt;
+    }
+    if (!ok && leader) {
+      // Every copy issued must land before the CTA's shared memory goes away.
+      for (uint32_t j = (w_issued > (uint32_t)p.WS ? w_issued - p.WS : 0); j < w_issued; ++j)
+        mbar_wait_unabortable(&w_full[j % p.WS], (j / p.WS) & 1);
+      for (uint32_t j = (h_issued > (uint32_t)p.HS ? h_issued - p.HS : 0); j < h_issued; ++j)
+        mbar_wait_unabortable(&h_full[j % p.HS], (j / p.HS) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0 && ntiles > 0) {
-      // Ring slots and parities advance by counters (no per-stage divisions).
-      int ws_ = 0, hs_ = 0;
-      uint32_t wph_ = 0, hph_ = 0;
-      int tdone = 0;
-      for (int r = 0; r < p.nrounds && tdone < ntiles; ++r) {
-        const int nt = min(p.round_tiles[r], ntiles - tdone);
-        const int buf = r & 1;
-        // The half's previous round has been read.
-        if (r > 1) mbar_wait(&acc_empty[buf], ((r >> 1) - 1) & 1, s_abort);
+    const bool leader = elect_one();
+    int ws = 0, hs = 0;
+    uint32_t wph = 0, hph = 0;
+    int tdone = 0;
+    // (after an expired wait the results are void and the waits no-ops)
+    for (int r = 0; r < p.nrounds && tdone < ntiles; ++r) {
+      const int nt = min(p.round_tiles[r], ntiles - tdone);
+      const int buf = r & 1;
+      // The half's previous round has been read.
+      if (r > 1) warp_wait(&acc_empty[buf], ((r >> 1) - 1) & 1, s_abort);
+      tc_fence_after();
+      int ks = k_rot;
+      for (int it = 0; it < p.NS; ++it) {
+        const int nch = min(p.KG, p.KC - ks * p.KG);
+        if (++ks == p.NS) ks = 0;
+        warp_wait(&h_full[hs], hph, s_abort);
         tc_fence_after();
-        for (int it = 0; it < p.NS; ++it) {
-          const int ks = it + k_rot < p.NS ? it + k_rot : it + k_rot - p.NS;
-          const int nch = min(p.KG, p.KC - ks * p.KG);
-          const int hs = hs_;
-          mbar_wait(&h_full[hs], hph_, s_abort);
+        const uint32_t h_addr = smem_u32(h_ring + hs * L.h_slot);
+        for (int j = 0; j < nt; ++j) {
+          warp_wait(&w_full[ws], wph, s_abort);
           tc_fence_after();
-          const uint32_t h_addr = smem_u32(h_ring + hs * L.h_slot);
-          for (int j = 0; j < nt; ++j) {
-            const int ws = ws_;
-            mbar_wait(&w_full[ws], wph_, s_abort);
-            tc_fence_after();
-            const uint32_t w_addr = smem_u32(w_ring + ws * L.w_slot);
-            // k-chunk stride in the slot: a full tile's chunks are 16 KB apart,
-            // the short last tile's are packed (BRS rows each).
-            const uint32_t w_chunk = (short_last && tdone + j == ntiles - 1) ? static_cast<uint32_t>(p.BRS * 128)
-                                                                            : static_cast<uint32_t>(kWChunkBytes);
-            const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kHalfCols + j * p.Ncols);
-            for (int jj = 0; jj < nch; ++jj) {
-              // Each operand's descriptor is built once per k-chunk; a K step of
-              // 16 adds 32 bytes, 2 in the descriptor's address field.
-              const uint64_t da = smem_desc_sw128(w_addr + jj * w_chunk);
-              const uint64_t db = smem_desc_sw128(h_addr + jj * p.Ncols * 128);
+          const uint32_t w_addr = smem_u32(w_ring + ws * L.w_slot);
+          // k-chunk stride in the slot: a full tile's chunks are 16 KB apart,
+          // the short last tile's are packed (BRS rows each).
+          const uint32_t w_chunk = (short_last && tdone + j == ntiles - 1) ? static_cast<uint32_t>(p.BRS * 128)
+                                                                          : static_cast<uint32_t>(kWChunkBytes);
+          const uint32_t d_tmem = tmem + static_cast<uint32_t>(buf * kHalfCols + j * p.Ncols);
+          for (int jj = 0; jj < nch; ++jj) {
+            // Each operand's descriptor is built once per k-chunk; a K step of
+            // 16 adds 32 bytes, 2 in the descriptor's address field.
+            const uint64_t da = smem_desc_sw128(w_addr + jj * w_chunk);
+            const uint64_t db = smem_desc_sw128(h_addr + jj * p.Ncols * 128);
 #pragma unroll
-              for (int k16 = 0; k16 < kKChunk / 16; ++k16)
-                tc_mma_f16(d_tmem, da + 2u * k16, db + 2u * k16, p.idesc, (it | jj | k16) != 0);
-            }
-            tc_commit(&w_empty[ws]);
-            if (++ws_ == p.WS) { ws_ = 0; wph_ ^= 1u; }
+            for (int k16 = 0; k16 < kKChunk / 16; ++k16)
+              if (leader) tc_mma_f16(d_tmem, da + 2u * k16, db + 2u * k16, p.idesc, (it | jj | k16) != 0);
           }
-          tc_commit(&h_empty[hs]);
-          if (++hs_ == p.HS) { hs_ = 0; hph_ ^= 1u; }
+          if (leader) tc_commit(&w_empty[ws]);
+          if (++ws == p.WS) { ws = 0; wph ^= 1u; }
         }
-        tc_commit(&acc_full[buf]);
-        ++rounds_issued;
-        tdone += nt;
+        if (leader) tc_commit(&h_empty[hs]);
+        if (++hs == p.HS) { hs = 0; hph ^= 1u; }
       }
+      if (leader) tc_commit(&acc_full[buf]);
+      ++rounds_issued;
+      tdone += nt;
     }
   } else {
     // ---- epilogue warps: slice statistics per row, logits of sampled rows ----
@@ -370,41 +368,6 @@ static void slice_shape(int V, int NC, int *tiles_max, int *brs) {
   *brs = last == 0 ? kTileV : (last + 7) / 8 * 8;
 }
 
-// 3-D view of a row-major [rows, H] bf16 matrix: dims {64, rows, H/64},
-// strides {H*2, 128} bytes, box {64, box_rows, kg}; lands as [kg][box_rows][64]
-// with the 128-byte swizzle, i.e. kg canonical K-major tiles back to back.
-static bool encode_kslab_view(CUtensorMap *map, const void *base, int rows, int H, int box_rows,
-                              int kg) {
-  using EncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn fn = nullptr;
-  if (!fn) {
-    void *f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-            cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-      return false;
-    }
-    fn = reinterpret_cast<EncodeFn>(f);
-  }
-  cuuint64_t dims[3] = {64, static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(H / 64)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(H) * 2, 128};
-  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(kg)};
-  cuuint32_t es[3] = {1, 1, 1};
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
-                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    fail(SPADE_ERR_CUDA, "cuTensorMapEncodeTiled (k-slab view) failed (%d)", static_cast<int>(r));
-    return false;
-  }
-  return true;
-}
-
 // Whether the one-launch form takes the call (its limits bound top-p too, whose
 // search reads every row's logits): at most 256 rows, at most 32 tiles per SM,
 // and tiles x rows (rounded up to 8) within the 512 accumulator columns.
@@ -503,8 +466,8 @@ static spade_status prepare(Params &p, const void *hidden, const void *w_lm, int
       !encode_tmap_bf16_sw128(&m.h2, hidden, H, R, pitch, kKChunk, pl.Ncols))
     return SPADE_ERR_CUDA;
   if (p.KCF >= 1) {
-    if (!encode_kslab_view(&m.w3, w_lm, V, H, kTileV, p.KG) || !encode_kslab_view(&m.w3s, w_lm, V, H, p.BRS, p.KG) ||
-        !encode_kslab_view(&m.h3, hidden, R, H, pl.Ncols, p.KG))
+    if (!encode_tmap_rows_by_slab(&m.w3, w_lm, V, H, kTileV, p.KG) || !encode_tmap_rows_by_slab(&m.w3s, w_lm, V, H, p.BRS, p.KG) ||
+        !encode_tmap_rows_by_slab(&m.h3, hidden, R, H, pl.Ncols, p.KG))
       return SPADE_ERR_CUDA;
   } else {
     m.w3 = m.w2;  // never used: every stage takes the 2-D path

@@ -14,10 +14,12 @@
 //    O^T[d][row] += V^T P^T with M = 128 (head dim), both operands read from
 //    shared memory in MN-major form straight from the TMA tiles.  Head dim 64
 //    keeps M = 128 with a V tile whose second 64-dim slab stays zero.
-//  * Warp roles: warp 0 streams K and V tiles (TMA, 128 keys x all head dims
-//    per box) into a two-stage ring; warp 1 issues the MMAs (one elected thread)
+//  * Warp roles: warp 0 streams the K tiles and warp 10 the V tiles (TMA, 128
+//    keys x all head dims per box) into two-stage rings; warp 1 issues the MMAs
 //    and owns the tensor-memory allocation; warps 2-9 run the softmax and the
 //    epilogue, two per tensor-memory lane quadrant, each on half of the rows.
+//    Producers and MMA warp walk their loops as whole warps with one elected
+//    lane issuing (uniform operands, see elect_one).
 //    The next unit's Q is prefetched (cp.async) into a second buffer while
 //    the current one runs.
 //  * Lazy rescaling: the running row maxima only move when a score exceeds
@@ -40,7 +42,8 @@ constexpr int kKeys = 128;                       // keys per MMA chunk (two slic
 constexpr int kStages = 2;                       // K/V ring depth (chunks)
 constexpr int kSoftWarps = 8;                    // softmax / epilogue warps
 constexpr int kSoftThreads = 32 * kSoftWarps;
-constexpr int kThreads = 64 + kSoftThreads;      // + producer warp + MMA warp
+constexpr int kWarpV = 2 + kSoftWarps;           // warp that loads the V tiles
+constexpr int kThreads = 96 + kSoftThreads;      // + K producer, MMA and V producer warps
 constexpr int kSlab = kKeys * 128;               // one 64-dim slab of a chunk: 16 KB
 constexpr int kTile = 2 * kSlab;                 // K or V tile of a chunk: 32 KB
 constexpr int kQSlab = kRowBlock * 128;          // one 64-dim slab of Q: 8 KB
@@ -210,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + Smem::MISC + 8);
 
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = uniform_warp();
   const int lane = tid & 31;
 
   if (tid == 0) { *s_abort = 0; *s_last = 0; }
@@ -305,130 +308,130 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint32_t smem_base = smem_u32(smem);
 
-  if (warp == 0) {
-    // ============================ producer: TMA ============================
-    // Lane 0 loads the K tiles, lane 1 the V tiles: a K stage is refilled as
-    // soon as its S product is done, without waiting behind the V stage that
-    // only frees after the softmax and the PV product.
-    if (lane < 2) {
-      const bool is_v = lane == 1;
-      const CUtensorMap *tm2 = is_v ? &tm_v2 : &tm_k2;
-      const CUtensorMap *tm1 = is_v ? &tm_v1 : &tm_k1;
-      const int bar_empty = is_v ? kBarVEmpty : kBarKEmpty;
-      const int bar_full = is_v ? kBarVFull : kBarKFull;
-      uint8_t *const ring = smem + (is_v ? Smem::V : Smem::K);
-      const uint64_t pol = l2_policy_evict_first();
-      uint32_t it = 0, issued = 0;
-      bool expired = false;
-      for (int64_t x = x_begin; x < x_end;) {
-        const SegInfo si = x == x_begin ? seg0 : next_seg(sc, x, x_end);
-        if (si.n_here == 0) break;
-        const int row0 = (si.g.b * p.Hkv + si.g.kvh) * p.cap;
-        for (int c = 0; c < si.nchunk; ++c, ++it) {
-          const int st = it % kStages;
-          const uint32_t ph = (it / kStages) & 1;
-          const int nsl = min(2, si.n_here - 2 * c);
-          const int key0 = (si.g.ci + 2 * c) * kChunk;
-          // Cache rows of the chunk's slices: contiguous in a dense cache; in a
-          // paged one each slice lies in one page (page sizes are multiples of
-          // 64), found through the block table before the stage wait so that
-          // the table load overlaps it.
-          int row_a = row0 + key0, row_b = row_a + kChunk;
-          if (p.block_table) {
-            row_a = paged_row(p, si.g.b, si.g.kvh, key0);
-            row_b = nsl == 2 ? paged_row(p, si.g.b, si.g.kvh, key0 + kChunk) : 0;
-          }
-          uint8_t *tile = ring + st * kTile;
-          if (!mbar_wait(&bars[bar_empty + st], ph ^ 1, s_abort)) expired = true;
-          if (*s_abort) continue;
-          mbar_arrive_expect_tx(&bars[bar_full + st], nsl * (kSlab / kDMax) * kD);
-          if (nsl == 2 && row_b == row_a + kChunk) {
-            tma_load_3d(tile, tm2, 0, row_a, 0, &bars[bar_full + st], pol);
-          } else {
-            // One 64-key box per slice and slab; the second slice lands 64 rows in.
-            for (int i = 0; i < nsl; ++i) {
-              const int row = i ? row_b : row_a;
-              uint8_t *dst = tile + i * kChunk * 128;
-              tma_load_3d(dst, tm1, 0, row, 0, &bars[bar_full + st], pol);
-              if constexpr (kD == kDMax) tma_load_3d(dst + kSlab, tm1, 0, row, 1, &bars[bar_full + st], pol);
+  if (warp == 0 || warp == kWarpV) {
+    // ============================ producers: TMA ===========================
+    // A warp each for K and V: a K stage is refilled as soon as its S product is
+    // done, without waiting behind the V stage that only frees after the
+    // softmax and the PV product.
+    const bool is_v = warp == kWarpV;
+    const bool leader = elect_one();
+    const CUtensorMap *tm2 = is_v ? &tm_v2 : &tm_k2;
+    const CUtensorMap *tm1 = is_v ? &tm_v1 : &tm_k1;
+    uint64_t *const empty = bars + (is_v ? kBarVEmpty : kBarKEmpty);
+    uint64_t *const full = bars + (is_v ? kBarVFull : kBarKFull);
+    uint8_t *const ring = smem + (is_v ? Smem::V : Smem::K);
+    const uint64_t pol = l2_policy_evict_first();
+    uint32_t st = 0, ph = 1, issued = 0;
+    bool ok = true;
+    for (int64_t x = x_begin; ok && x < x_end;) {
+      const SegInfo si = x == x_begin ? seg0 : next_seg_warp(sc, x, x_end, lane);
+      const int n_here = uniform(si.n_here), nchunk = uniform(si.nchunk), ci = uniform(si.g.ci);
+      if (n_here == 0) break;
+      const int b = uniform(si.g.b), kvh = uniform(si.g.kvh);
+      const int row0 = (b * p.Hkv + kvh) * p.cap;
+      for (int c = 0; c < nchunk; ++c) {
+        const int nsl = min(2, n_here - 2 * c);
+        const int key0 = (ci + 2 * c) * kChunk;
+        // Cache rows of the chunk's slices: contiguous in a dense cache; in a
+        // paged one each slice lies in one page (page sizes are multiples of
+        // 64), found through the block table before the stage wait so that
+        // the table load overlaps it.
+        int row_a = row0 + key0, row_b = row_a + kChunk;
+        if (p.block_table) {
+          row_a = uniform(paged_row(p, b, kvh, key0));
+          row_b = nsl == 2 ? uniform(paged_row(p, b, kvh, key0 + kChunk)) : 0;
+        }
+        uint8_t *tile = ring + st * kTile;
+        ok = warp_wait(&empty[st], ph, s_abort);
+        if (!ok) break;
+        if (leader) mbar_arrive_expect_tx(&full[st], nsl * (kSlab / kDMax) * kD);
+        if (nsl == 2 && row_b == row_a + kChunk) {
+          if (leader) tma_load_3d(tile, tm2, 0, row_a, 0, &full[st], pol);
+        } else {
+          // One 64-key box per slice and slab; the second slice lands 64 rows in.
+          for (int i = 0; i < nsl; ++i) {
+            const int row = i ? row_b : row_a;
+            uint8_t *dst = tile + i * kChunk * 128;
+            if (leader) {
+              tma_load_3d(dst, tm1, 0, row, 0, &full[st], pol);
+              if constexpr (kD == kDMax) tma_load_3d(dst + kSlab, tm1, 0, row, 1, &full[st], pol);
             }
           }
-          issued = it + 1;
         }
-        x = si.seg_end;
+        ++issued;
+        if (++st == kStages) { st = 0; ph ^= 1u; }
       }
-      if (expired || *s_abort) {
-        atomicOr(p.status, SPADE_DEV_TIMEOUT);
-        // Drain: every copy issued must land before the CTA's smem goes away.
-        for (uint32_t j = (issued > kStages ? issued - kStages : 0); j < issued; ++j)
-          mbar_wait_unabortable(&bars[bar_full + j % kStages], (j / kStages) & 1);
-      }
+      x = si.seg_end;
+    }
+    if (!ok && leader) {
+      atomicOr(p.status, SPADE_DEV_TIMEOUT);
+      // Drain: every copy issued must land before the CTA's smem goes away.
+      for (uint32_t j = (issued > kStages ? issued - kStages : 0); j < issued; ++j)
+        mbar_wait_unabortable(&full[j % kStages], (j / kStages) & 1);
     }
   } else if (warp == 1) {
     // ============================ MMA issuer ===============================
-    if (lane == 0) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(128, NR);                           // K-major A, B
-      constexpr uint32_t idesc_pv = idesc_bf16_f32(128, NR) | (1u << 15) | (1u << 16);  // MN-major A, B
-      bool expired = false;
-      uint32_t it = 0, seg = 0;
-      // O^T += V^T P^T for chunk j (first: overwrite instead of accumulate;
-      // last: the segment's final product, signalled on OFinal too).
-      auto issue_pv = [&](uint32_t j, bool first, bool last) {
-        const int st = j % kStages;
-        const uint32_t ph = (j / kStages) & 1;
-        if (!mbar_wait(&bars[kBarVFull + st], ph, s_abort)) expired = true;
-        if (!mbar_wait(&bars[kBarPFull + st], ph, s_abort)) expired = true;
-        // The segment's first PV overwrites O^T: the previous epilogue has read it.
-        if (first && !mbar_wait(&bars[kBarSeg], seg & 1, s_abort)) expired = true;
-        tc_fence_after();
-        if (!*s_abort) {
-          const uint32_t v_addr = smem_base + Smem::V + st * kTile;
-          const uint32_t p_addr = smem_base + Smem::P + st * kPBytes;
+    constexpr uint32_t idesc_s = idesc_bf16_f32(128, NR);                           // K-major A, B
+    constexpr uint32_t idesc_pv = idesc_bf16_f32(128, NR) | (1u << 15) | (1u << 16);  // MN-major A, B
+    const bool leader = elect_one();
+    bool ok = true;  // (after an expired wait the results are void and the waits no-ops)
+    uint32_t it = 0, seg = 0;
+    // O^T += V^T P^T for chunk j (first: overwrite instead of accumulate;
+    // last: the segment's final product, signalled on OFinal too).
+    auto issue_pv = [&](uint32_t j, bool first, bool last) {
+      const int st = j % kStages;
+      const uint32_t ph = (j / kStages) & 1;
+      ok &= warp_wait(&bars[kBarVFull + st], ph, s_abort);
+      ok &= warp_wait(&bars[kBarPFull + st], ph, s_abort);
+      // The segment's first PV overwrites O^T: the previous epilogue has read it.
+      if (first) ok &= warp_wait(&bars[kBarSeg], seg & 1, s_abort);
+      tc_fence_after();
+      const uint64_t dv = desc_sw128(smem_base + Smem::V + st * kTile, kSlab, 1024);
+      const uint64_t dp = desc_sw128(smem_base + Smem::P + st * kPBytes, kSlab, 1024);
 #pragma unroll
-          for (int kk = 0; kk < kKeys / 16; ++kk)
-            tc_mma_f16(tmem + kColO, desc_sw128(v_addr + kk * 2048, kSlab, 1024),
-                       desc_sw128(p_addr + kk * 2048, kSlab, 1024), idesc_pv,
-                       (first && kk == 0) ? 0u : 1u);
-        }
+      for (int kk = 0; kk < kKeys / 16; ++kk)  // 16 keys: 2048 bytes, 128 in the address field
+        if (leader) tc_mma_f16(tmem + kColO, dv + 128u * kk, dp + 128u * kk, idesc_pv, (first && kk == 0) ? 0u : 1u);
+      if (leader) {
         tc_commit(&bars[kBarVEmpty + st]);
         tc_commit(&bars[kBarPFree + st]);
         tc_commit(&bars[kBarODone]);
         if (last) tc_commit(&bars[kBarOFinal]);
-      };
-      for (int64_t x = x_begin; x < x_end;) {
-        const SegInfo si = x == x_begin ? seg0 : next_seg(sc, x, x_end);
-        if (si.n_here == 0) break;
-        // Q staged: the segment's S products may start while the previous
-        // segment's epilogue still reads O^T.
-        if (!mbar_wait(&bars[kBarQ], seg & 1, s_abort)) expired = true;
+      }
+    };
+    for (int64_t x = x_begin; x < x_end;) {
+      const SegInfo si = x == x_begin ? seg0 : next_seg_warp(sc, x, x_end, lane);
+      const int nchunk = uniform(si.nchunk);
+      if (uniform(si.n_here) == 0) break;
+      // Q staged: the segment's S products may start while the previous
+      // segment's epilogue still reads O^T.
+      ok &= warp_wait(&bars[kBarQ], seg & 1, s_abort);
+      tc_fence_after();
+      const uint64_t dq = desc_sw128(smem_base + Smem::Q + (seg & 1) * 2 * kQSlab, 16, 1024);
+      for (int c = 0; c < nchunk; ++c, ++it) {
+        const int st = it % kStages;
+        const uint32_t ph = (it / kStages) & 1;
+        ok &= warp_wait(&bars[kBarKFull + st], ph, s_abort);
+        ok &= warp_wait(&bars[kBarSFree + st], ph ^ 1, s_abort);
         tc_fence_after();
-        const uint32_t q_addr = smem_base + Smem::Q + (seg & 1) * 2 * kQSlab;
-        for (int c = 0; c < si.nchunk; ++c, ++it) {
-          const int st = it % kStages;
-          const uint32_t ph = (it / kStages) & 1;
-          if (!mbar_wait(&bars[kBarKFull + st], ph, s_abort)) expired = true;
-          if (!mbar_wait(&bars[kBarSFree + st], ph ^ 1, s_abort)) expired = true;
-          tc_fence_after();
-          if (!*s_abort) {
-            const uint32_t k_addr = smem_base + Smem::K + st * kTile;
+        const uint64_t dk = desc_sw128(smem_base + Smem::K + st * kTile, 16, 1024);
+        const uint32_t d = tmem + kColS + static_cast<uint32_t>(st) * 64u;
 #pragma unroll
-            for (int kk = 0; kk < kD / 16; ++kk) {
-              const uint32_t off = (kk >> 2) * kSlab + (kk & 3) * 32;
-              const uint32_t qoff = (kk >> 2) * kQSlab + (kk & 3) * 32;
-              tc_mma_f16(tmem + kColS + st * 64, desc_sw128(k_addr + off, 16, 1024),
-                         desc_sw128(q_addr + qoff, 16, 1024), idesc_s, kk > 0 ? 1u : 0u);
-            }
-          }
+        for (int kk = 0; kk < kD / 16; ++kk) {
+          const uint32_t ko = ((kk >> 2) * kSlab + (kk & 3) * 32) >> 4;  // in the descriptors' address field
+          const uint32_t qo = ((kk >> 2) * kQSlab + (kk & 3) * 32) >> 4;
+          if (leader) tc_mma_f16(d, dk + ko, dq + qo, idesc_s, kk > 0 ? 1u : 0u);
+        }
+        if (leader) {
           tc_commit(&bars[kBarSFull + st]);
           tc_commit(&bars[kBarKEmpty + st]);
-          if (c > 0) issue_pv(it - 1, c == 1, false);
         }
-        issue_pv(it - 1, si.nchunk == 1, true);
-        ++seg;
-        x = si.seg_end;
+        if (c > 0) issue_pv(it - 1, c == 1, false);
       }
-      if (expired) atomicOr(p.status, SPADE_DEV_TIMEOUT);
+      issue_pv(it - 1, nchunk == 1, true);
+      ++seg;
+      x = si.seg_end;
     }
+    if (!ok && leader) atomicOr(p.status, SPADE_DEV_TIMEOUT);
   } else {
     // ===================== softmax and epilogue (warps 2-9) =================
     constexpr int NH = NR / 2;             // rows (S^T / O^T columns) per softmax warp
