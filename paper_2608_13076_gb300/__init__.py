@@ -1,10 +1,11 @@
 """SPADE verify step on GB300: Python binding of the C-ABI library libspade.so.
 
-This module only marshals arguments: it checks dtypes and layouts of torch
-tensors and passes raw device pointers, sizes and the current CUDA stream to
-the library's entry points.  Every step of the verify path runs in the
-library's CUDA kernels; there is no Python or CPU fallback, and a call fails
-loudly if the library is missing.
+This module only marshals arguments: the native extension (csrc/binding.cpp)
+checks dtypes and layouts of torch tensors and passes raw device pointers,
+sizes and the current CUDA stream to the library's entry points; helpers that
+are not on a verify step's path go through ctypes.  Every step of the verify
+path runs in the library's CUDA kernels; there is no Python or CPU fallback,
+and a call fails loudly if the library is missing.
 
 Entry points (same names as the C ABI in include/spade.h):
     spade_verify_attention  verify-position attention against the KV cache
@@ -15,6 +16,7 @@ Entry points (same names as the C ABI in include/spade.h):
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import torch
@@ -39,6 +41,7 @@ DEV_TIMEOUT = 0x4
 DEV_FALLBACK = 0x8
 
 _lib = None
+_native = None  # the extension module, once loaded
 
 
 class SpadeError(RuntimeError):
@@ -120,6 +123,22 @@ def load():
     return lib
 
 
+def native():
+    """The native extension that checks and passes a call's tensors (built with the library)."""
+    global _native
+    if _native is None:
+        load()
+        path = _build.NATIVE_PATH
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: build the CUDA library first "
+                               "(python -c 'import __graft_entry__ as g; g.build()')")
+        spec = importlib.util.spec_from_file_location("_spade_native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native = module
+    return _native
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -175,27 +194,10 @@ def attn_workspace(B, Hq, Hkv, D, cap, max_k, device="cuda"):
 def spade_verify_attention(q, k_cache, v_cache, ctx_lens, n_draft, cu_q, out, lse=None, *,
                            max_k, workspace, status, stream=None):
     """out[cu_q[b]+i, h] = softmax(q K^T / sqrt(D)) V over keys [0, ctx_b + i] (KV head h // G)."""
-    _need(q, "q", torch.bfloat16, 3)
-    _need(k_cache, "k_cache", torch.bfloat16, 4)
-    _need(v_cache, "v_cache", torch.bfloat16, 4)
-    for t, n in ((ctx_lens, "ctx_lens"), (n_draft, "n_draft"), (cu_q, "cu_q"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    _need(out, "out", torch.bfloat16, 3)
-    if lse is not None:
-        _need(lse, "lse", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    if v_cache.shape != k_cache.shape:
-        raise ValueError("k_cache and v_cache shapes differ")
-    R, Hq, D = q.shape
-    B, Hkv, cap, Dk = k_cache.shape
-    if Dk != D or tuple(out.shape) != (R, Hq, D) or ctx_lens.numel() != B or n_draft.numel() != B \
-            or cu_q.numel() != B + 1:
-        raise ValueError("inconsistent attention shapes")
-    rc = load().spade_verify_attention(
-        _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), _ptr(n_draft), _ptr(cu_q), _ptr(out),
-        _ptr(lse), B, Hq, Hkv, D, cap, int(max_k), R, _ptr(workspace), workspace.numel(),
-        _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).attention(
+        q, k_cache, v_cache, ctx_lens, n_draft, cu_q, out, lse, max_k, workspace, status, stream)
+    if rc:
+        _check_rc(rc)
     return out
 
 
@@ -206,16 +208,10 @@ def spade_verify_attention_noalloc(q, k_cache, v_cache, ctx_lens, n_draft, cu_q,
     Calls that overlap on the GPU share that array and race; the first call on
     a device resolves the array's address and should precede any stream capture.
     """
-    R, Hq, D = q.shape
-    B, Hkv, cap, _ = k_cache.shape
-    for t, n in ((q, "q"), (k_cache, "k_cache"), (v_cache, "v_cache"), (out, "out")):
-        _need(t, n, torch.bfloat16)
-    for t, n in ((ctx_lens, "ctx_lens"), (n_draft, "n_draft"), (cu_q, "cu_q"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    rc = load().spade_verify_attention_noalloc(
-        _ptr(q), _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), _ptr(n_draft), _ptr(cu_q), _ptr(out),
-        _ptr(lse), B, Hq, Hkv, D, cap, int(max_k), R, _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).attention_noalloc(
+        q, k_cache, v_cache, ctx_lens, n_draft, cu_q, out, lse, max_k, status, stream)
+    if rc:
+        _check_rc(rc)
     return out
 
 
@@ -270,37 +266,11 @@ def spade_verify_accept(hidden, w_lm, draft_tokens, draft_probs, uniforms, mode,
                         accepted_len, next_token, *, workspace, status, stream=None, temperature=None):
     """Greedy / rejection-sampling verification of every sequence (see include/spade.h); with
     ``temperature`` ([B] float32) the verifier's p is softmax(logits / T)."""
-    _need(hidden, "hidden", torch.bfloat16, 2)
-    _need(w_lm, "w_lm", torch.bfloat16, 2)
-    _need(uniforms, "uniforms", torch.float32, 1)
-    for t, n in ((draft_tokens, "draft_tokens"), (mode, "mode"), (cu_q, "cu_q"), (n_draft, "n_draft"),
-                 (accepted_len, "accepted_len"), (next_token, "next_token"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    if draft_probs is not None:
-        _need(draft_probs, "draft_probs", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    R, H = hidden.shape
-    V, H2 = w_lm.shape
-    B = n_draft.numel()
-    if H2 != H or uniforms.numel() != R or draft_tokens.numel() != R - B or cu_q.numel() != B + 1 \
-            or mode.numel() != B or accepted_len.numel() != B or next_token.numel() != B:
-        raise ValueError("inconsistent accept shapes")
-    if draft_probs is not None and tuple(draft_probs.shape) != (R - B, V):
-        raise ValueError("draft_probs must be [R - B, V]")
-    if temperature is None:
-        rc = load().spade_verify_accept(
-            _ptr(hidden), _ptr(w_lm), _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), _ptr(mode),
-            _ptr(cu_q), _ptr(n_draft), _ptr(accepted_len), _ptr(next_token), B, R, H, V,
-            _ptr(workspace), workspace.numel(), _ptr(status), _stream(stream))
-    else:
-        _need(temperature, "temperature", torch.float32, 1)
-        if temperature.numel() != B:
-            raise ValueError("temperature must be [B]")
-        rc = load().spade_verify_accept_temperature(
-            _ptr(hidden), _ptr(w_lm), _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), _ptr(mode),
-            _ptr(temperature), _ptr(cu_q), _ptr(n_draft), _ptr(accepted_len), _ptr(next_token), B, R, H, V,
-            _ptr(workspace), workspace.numel(), _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).accept(
+        hidden, w_lm, draft_tokens, draft_probs, uniforms, mode, cu_q, n_draft,
+        accepted_len, next_token, temperature, workspace, status, stream)
+    if rc:
+        _check_rc(rc)
     return accepted_len, next_token
 
 
@@ -308,34 +278,11 @@ def spade_verify_accept_commit(hidden, w_lm, draft_tokens, draft_probs, uniforms
                                accepted_len, next_token, k_cache, v_cache, ctx_lens, *, workspace,
                                status, stream=None):
     """spade_verify_accept followed by spade_kv_commit in one launch (see include/spade.h)."""
-    _need(hidden, "hidden", torch.bfloat16, 2)
-    _need(w_lm, "w_lm", torch.bfloat16, 2)
-    _need(uniforms, "uniforms", torch.float32, 1)
-    for t, n in ((draft_tokens, "draft_tokens"), (mode, "mode"), (cu_q, "cu_q"), (n_draft, "n_draft"),
-                 (accepted_len, "accepted_len"), (next_token, "next_token"), (status, "status"),
-                 (ctx_lens, "ctx_lens")):
-        _need(t, n, torch.int32, 1)
-    if draft_probs is not None:
-        _need(draft_probs, "draft_probs", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    _need(k_cache, "k_cache", torch.bfloat16, 4)
-    _need(v_cache, "v_cache", torch.bfloat16, 4)
-    R, H = hidden.shape
-    V, H2 = w_lm.shape
-    B = n_draft.numel()
-    Bc, Hkv, cap, D = k_cache.shape
-    if H2 != H or uniforms.numel() != R or draft_tokens.numel() != R - B or cu_q.numel() != B + 1 \
-            or mode.numel() != B or accepted_len.numel() != B or next_token.numel() != B \
-            or Bc != B or tuple(v_cache.shape) != tuple(k_cache.shape) or ctx_lens.numel() != B:
-        raise ValueError("inconsistent accept/commit shapes")
-    if draft_probs is not None and tuple(draft_probs.shape) != (R - B, V):
-        raise ValueError("draft_probs must be [R - B, V]")
-    rc = load().spade_verify_accept_commit(
-        _ptr(hidden), _ptr(w_lm), _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), _ptr(mode),
-        _ptr(cu_q), _ptr(n_draft), _ptr(accepted_len), _ptr(next_token), _ptr(k_cache), _ptr(v_cache),
-        _ptr(ctx_lens), B, R, H, V, Hkv, D, cap, _ptr(workspace), workspace.numel(), _ptr(status),
-        _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).accept_commit(
+        hidden, w_lm, draft_tokens, draft_probs, uniforms, mode, cu_q, n_draft,
+        accepted_len, next_token, k_cache, v_cache, ctx_lens, workspace, status, stream)
+    if rc:
+        _check_rc(rc)
     return accepted_len, next_token
 
 
@@ -345,44 +292,12 @@ def spade_verify_accept_sampling(hidden, w_lm, draft_tokens, draft_probs, unifor
     """spade_verify_accept with per-sequence ``temperature`` and ``top_p`` ([B] float32, either
     may be None) and, with k_cache / v_cache / ctx_lens given, the fused KV commit
     (see include/spade.h)."""
-    _need(hidden, "hidden", torch.bfloat16, 2)
-    _need(w_lm, "w_lm", torch.bfloat16, 2)
-    _need(uniforms, "uniforms", torch.float32, 1)
-    for t, n in ((draft_tokens, "draft_tokens"), (mode, "mode"), (cu_q, "cu_q"), (n_draft, "n_draft"),
-                 (accepted_len, "accepted_len"), (next_token, "next_token"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    if draft_probs is not None:
-        _need(draft_probs, "draft_probs", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    R, H = hidden.shape
-    V, H2 = w_lm.shape
-    B = n_draft.numel()
-    if H2 != H or uniforms.numel() != R or draft_tokens.numel() != R - B or cu_q.numel() != B + 1 \
-            or mode.numel() != B or accepted_len.numel() != B or next_token.numel() != B:
-        raise ValueError("inconsistent accept shapes")
-    if draft_probs is not None and tuple(draft_probs.shape) != (R - B, V):
-        raise ValueError("draft_probs must be [R - B, V]")
-    for t, n in ((temperature, "temperature"), (top_p, "top_p")):
-        if t is not None:
-            _need(t, n, torch.float32, 1)
-            if t.numel() != B:
-                raise ValueError(f"{n} must be [B]")
-    Hkv = D = cap = 0
-    if (k_cache is None) != (v_cache is None) or (k_cache is None) != (ctx_lens is None):
-        raise ValueError("give all of k_cache, v_cache, ctx_lens or none")
-    if k_cache is not None:
-        _need(k_cache, "k_cache", torch.bfloat16, 4)
-        _need(v_cache, "v_cache", torch.bfloat16, 4)
-        _need(ctx_lens, "ctx_lens", torch.int32, 1)
-        Bc, Hkv, cap, D = k_cache.shape
-        if Bc != B or tuple(v_cache.shape) != tuple(k_cache.shape) or ctx_lens.numel() != B:
-            raise ValueError("inconsistent cache shapes")
-    rc = load().spade_verify_accept_sampling(
-        _ptr(hidden), _ptr(w_lm), _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), _ptr(mode),
-        _ptr(temperature), _ptr(top_p), _ptr(cu_q), _ptr(n_draft), _ptr(accepted_len), _ptr(next_token),
-        _ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), B, R, H, V, Hkv, D, cap, _ptr(workspace),
-        workspace.numel(), _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).accept_sampling(
+        hidden, w_lm, draft_tokens, draft_probs, uniforms, mode, cu_q, n_draft,
+        accepted_len, next_token, temperature, top_p, k_cache, v_cache, ctx_lens, workspace, status,
+        stream)
+    if rc:
+        _check_rc(rc)
     return accepted_len, next_token
 
 
@@ -391,35 +306,11 @@ def spade_verify_accept_commit_paged(hidden, w_lm, draft_tokens, draft_probs, un
                                      workspace, status, stream=None):
     """spade_verify_accept_commit on paged caches: pools [num_pages, Hkv, page_size, D] and a
     block table [B, max_pages] (see include/spade.h)."""
-    _need(hidden, "hidden", torch.bfloat16, 2)
-    _need(w_lm, "w_lm", torch.bfloat16, 2)
-    _need(uniforms, "uniforms", torch.float32, 1)
-    for t, n in ((draft_tokens, "draft_tokens"), (mode, "mode"), (cu_q, "cu_q"), (n_draft, "n_draft"),
-                 (accepted_len, "accepted_len"), (next_token, "next_token"), (status, "status"),
-                 (ctx_lens, "ctx_lens")):
-        _need(t, n, torch.int32, 1)
-    if draft_probs is not None:
-        _need(draft_probs, "draft_probs", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    _need(k_pool, "k_pool", torch.bfloat16, 4)
-    _need(v_pool, "v_pool", torch.bfloat16, 4)
-    _need(block_table, "block_table", torch.int32, 2)
-    R, H = hidden.shape
-    V, H2 = w_lm.shape
-    B = n_draft.numel()
-    num_pages, Hkv, page_size, D = k_pool.shape
-    if H2 != H or uniforms.numel() != R or draft_tokens.numel() != R - B or cu_q.numel() != B + 1 \
-            or mode.numel() != B or accepted_len.numel() != B or next_token.numel() != B \
-            or tuple(v_pool.shape) != tuple(k_pool.shape) or ctx_lens.numel() != B or block_table.shape[0] != B:
-        raise ValueError("inconsistent accept/commit shapes")
-    if draft_probs is not None and tuple(draft_probs.shape) != (R - B, V):
-        raise ValueError("draft_probs must be [R - B, V]")
-    rc = load().spade_verify_accept_commit_paged(
-        _ptr(hidden), _ptr(w_lm), _ptr(draft_tokens), _ptr(draft_probs), _ptr(uniforms), _ptr(mode),
-        _ptr(cu_q), _ptr(n_draft), _ptr(accepted_len), _ptr(next_token), _ptr(k_pool), _ptr(v_pool),
-        _ptr(block_table), _ptr(ctx_lens), B, R, H, V, Hkv, D, page_size, num_pages, block_table.shape[1],
-        _ptr(workspace), workspace.numel(), _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).accept_commit_paged(
+        hidden, w_lm, draft_tokens, draft_probs, uniforms, mode, cu_q, n_draft,
+        accepted_len, next_token, k_pool, v_pool, block_table, ctx_lens, workspace, status, stream)
+    if rc:
+        _check_rc(rc)
     return accepted_len, next_token
 
 
@@ -439,110 +330,48 @@ def qkv_workspace(R, Hq, Hkv, D, device="cuda"):
 def spade_verify_qkv_rope(x, w_qkv, ctx_lens, n_draft, cu_q, q_out, k_cache, v_cache, *, Hq, Hkv,
                           rope_theta, max_k, workspace, status, stream=None):
     """q, k, v of the verify block (rotary embedding at ctx + i); K/V into cache slots ctx .. ctx + k."""
-    _need(x, "x", torch.bfloat16, 2)
-    _need(w_qkv, "w_qkv", torch.bfloat16, 2)
-    _need(q_out, "q_out", torch.bfloat16, 3)
-    _need(k_cache, "k_cache", torch.bfloat16, 4)
-    _need(v_cache, "v_cache", torch.bfloat16, 4)
-    for t, n in ((ctx_lens, "ctx_lens"), (n_draft, "n_draft"), (cu_q, "cu_q"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    R, H = x.shape
-    B, Hkv2, cap, D = k_cache.shape
-    if Hkv2 != Hkv or tuple(v_cache.shape) != tuple(k_cache.shape) or tuple(q_out.shape) != (R, Hq, D) \
-            or tuple(w_qkv.shape) != ((Hq + 2 * Hkv) * D, H) or ctx_lens.numel() != B or n_draft.numel() != B \
-            or cu_q.numel() != B + 1:
-        raise ValueError("inconsistent qkv_rope shapes")
-    _need(workspace, "workspace", torch.uint8, 1)
-    rc = load().spade_verify_qkv_rope(
-        _ptr(x), _ptr(w_qkv), _ptr(ctx_lens), _ptr(n_draft), _ptr(cu_q), _ptr(q_out), _ptr(k_cache), _ptr(v_cache),
-        B, R, H, Hq, Hkv, D, cap, int(max_k), float(rope_theta), _ptr(workspace), workspace.numel(), _ptr(status),
-        _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).qkv(
+        x, w_qkv, ctx_lens, n_draft, cu_q, q_out, k_cache, v_cache, Hq, Hkv, rope_theta, max_k, workspace, status,
+        stream)
+    if rc:
+        _check_rc(rc)
     return q_out
 
 
 # ---------------------------------------------------------------------------
 # Paged KV cache: pools [num_pages, Hkv, page_size, D], block_table [B, max_pages].
-def _need_paged(k_pool, v_pool, block_table):
-    _need(k_pool, "k_pool", torch.bfloat16, 4)
-    _need(v_pool, "v_pool", torch.bfloat16, 4)
-    _need(block_table, "block_table", torch.int32, 2)
-    if tuple(v_pool.shape) != tuple(k_pool.shape):
-        raise ValueError("k_pool and v_pool shapes differ")
-    num_pages, Hkv, page_size, D = k_pool.shape
-    return num_pages, Hkv, page_size, D, block_table.shape[1]
-
-
 def spade_verify_attention_paged(q, k_pool, v_pool, block_table, ctx_lens, n_draft, cu_q, out, lse=None, *,
                                  max_k, workspace, status, stream=None):
     """spade_verify_attention on a paged cache (see include/spade.h)."""
-    _need(q, "q", torch.bfloat16, 3)
-    _need(out, "out", torch.bfloat16, 3)
-    num_pages, Hkv, page_size, D, max_pages = _need_paged(k_pool, v_pool, block_table)
-    for t, n in ((ctx_lens, "ctx_lens"), (n_draft, "n_draft"), (cu_q, "cu_q"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    if lse is not None:
-        _need(lse, "lse", torch.float32, 2)
-    _need(workspace, "workspace", torch.uint8, 1)
-    R, Hq, Dq = q.shape
-    B = ctx_lens.numel()
-    if Dq != D or tuple(out.shape) != (R, Hq, D) or block_table.shape[0] != B or n_draft.numel() != B \
-            or cu_q.numel() != B + 1:
-        raise ValueError("inconsistent paged attention shapes")
-    rc = load().spade_verify_attention_paged(
-        _ptr(q), _ptr(k_pool), _ptr(v_pool), _ptr(block_table), _ptr(ctx_lens), _ptr(n_draft), _ptr(cu_q), _ptr(out),
-        _ptr(lse), B, Hq, Hkv, D, page_size, num_pages, max_pages, int(max_k), R, _ptr(workspace), workspace.numel(),
-        _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).attention_paged(
+        q, k_pool, v_pool, block_table, ctx_lens, n_draft, cu_q, out, lse, max_k, workspace, status, stream)
+    if rc:
+        _check_rc(rc)
     return out
 
 
 def spade_kv_commit_paged(k_pool, v_pool, block_table, ctx_lens, accepted_len, n_draft, *, status, stream=None):
     """spade_kv_commit on a paged cache (see include/spade.h)."""
-    num_pages, Hkv, page_size, D, max_pages = _need_paged(k_pool, v_pool, block_table)
-    for t, n in ((ctx_lens, "ctx_lens"), (accepted_len, "accepted_len"), (n_draft, "n_draft"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    B = ctx_lens.numel()
-    if block_table.shape[0] != B:
-        raise ValueError("block_table must have one row per sequence")
-    rc = load().spade_kv_commit_paged(_ptr(k_pool), _ptr(v_pool), _ptr(block_table), _ptr(ctx_lens),
-                                      _ptr(accepted_len), _ptr(n_draft), B, Hkv, D, page_size, num_pages,
-                                      max_pages, _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).commit_paged(
+        k_pool, v_pool, block_table, ctx_lens, accepted_len, n_draft, status, stream)
+    if rc:
+        _check_rc(rc)
 
 
 def spade_verify_qkv_rope_paged(x, w_qkv, block_table, ctx_lens, n_draft, cu_q, q_out, k_pool, v_pool, *, Hq,
                                 rope_theta, max_k, workspace, status, stream=None):
     """spade_verify_qkv_rope writing the block's K/V into a paged cache (see include/spade.h)."""
-    _need(x, "x", torch.bfloat16, 2)
-    _need(w_qkv, "w_qkv", torch.bfloat16, 2)
-    _need(q_out, "q_out", torch.bfloat16, 3)
-    num_pages, Hkv, page_size, D, max_pages = _need_paged(k_pool, v_pool, block_table)
-    for t, n in ((ctx_lens, "ctx_lens"), (n_draft, "n_draft"), (cu_q, "cu_q"), (status, "status")):
-        _need(t, n, torch.int32, 1)
-    R, H = x.shape
-    B = ctx_lens.numel()
-    if tuple(q_out.shape) != (R, Hq, D) or tuple(w_qkv.shape) != ((Hq + 2 * Hkv) * D, H) \
-            or block_table.shape[0] != B or n_draft.numel() != B or cu_q.numel() != B + 1:
-        raise ValueError("inconsistent paged qkv_rope shapes")
-    _need(workspace, "workspace", torch.uint8, 1)
-    rc = load().spade_verify_qkv_rope_paged(
-        _ptr(x), _ptr(w_qkv), _ptr(block_table), _ptr(ctx_lens), _ptr(n_draft), _ptr(cu_q), _ptr(q_out),
-        _ptr(k_pool), _ptr(v_pool), B, R, H, Hq, Hkv, D, page_size, num_pages, max_pages, int(max_k),
-        float(rope_theta), _ptr(workspace), workspace.numel(), _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).qkv_paged(
+        x, w_qkv, block_table, ctx_lens, n_draft, cu_q, q_out, k_pool, v_pool, Hq, rope_theta, max_k, workspace,
+        status, stream)
+    if rc:
+        _check_rc(rc)
     return q_out
 
 
 # ---------------------------------------------------------------------------
 def spade_kv_commit(k_cache, v_cache, ctx_lens, accepted_len, n_draft, *, status, stream=None):
     """ctx_lens += accepted_len + 1; rejected draft slots of the caches are cleared."""
-    _need(k_cache, "k_cache", torch.bfloat16, 4)
-    _need(v_cache, "v_cache", torch.bfloat16, 4)
-    for t, n in ((ctx_lens, "ctx_lens"), (accepted_len, "accepted_len"), (n_draft, "n_draft"),
-                 (status, "status")):
-        _need(t, n, torch.int32, 1)
-    B, Hkv, cap, D = k_cache.shape
-    rc = load().spade_kv_commit(_ptr(k_cache), _ptr(v_cache), _ptr(ctx_lens), _ptr(accepted_len),
-                                _ptr(n_draft), B, Hkv, D, cap, _ptr(status), _stream(stream))
-    _check_rc(rc)
+    rc = (_native or native()).commit(k_cache, v_cache, ctx_lens, accepted_len, n_draft, status, stream)
+    if rc:
+        _check_rc(rc)

@@ -1,8 +1,10 @@
-"""Builds libspade.so (the C-ABI library) in-tree with nvcc for sm_103a.
+"""Builds libspade.so (the C-ABI library) in-tree with nvcc for sm_103a, and its Python binding.
 
 Each .cu under csrc/ is compiled to an object in parallel, then linked into
 ``paper_2608_13076_gb300/lib/libspade.so`` with the CUDA runtime linked
-statically.  A rebuild happens only when a source is newer than the library.
+statically; csrc/binding.cpp becomes ``lib/_spade_native.so``, an extension
+module over the installed torch.  A rebuild happens only when a source is newer
+than the outputs.
 """
 from __future__ import annotations
 
@@ -10,6 +12,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -18,6 +21,8 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB_DIR = os.path.join(HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libspade.so")
+NATIVE_PATH = os.path.join(LIB_DIR, "_spade_native.so")
+BINDING = os.path.join(CSRC, "binding.cpp")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
@@ -35,15 +40,44 @@ def sources():
 
 
 def _deps():
-    return sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) \
+    return sources() + [BINDING] + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) \
         + [os.path.join(INCLUDE, "spade.h"), os.path.abspath(__file__)]
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
         return False
-    t = os.path.getmtime(LIB_PATH)
+    t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
     return all(os.path.getmtime(d) <= t for d in _deps())
+
+
+def _run(cmd, what):
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{what} failed:\n{r.stdout}\n{r.stderr}")
+    return r
+
+
+def _compile_binding(cuda_home):
+    """csrc/binding.cpp -> object, against the installed torch and Python headers."""
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    obj = os.path.join(BUILD_DIR, "binding.o")
+    _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-c", BINDING, "-o", obj,
+          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE, "-isystem", inc,
+          "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+          "-isystem", os.path.join(cuda_home, "include"), "-isystem", sysconfig.get_paths()["include"]],
+         "g++ on binding.cpp")
+    return obj
+
+
+def _link_binding(obj):
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = NATIVE_PATH + ".tmp"
+    _run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, LIB_PATH, "-L", lib, "-lc10", "-lc10_cuda",
+          "-ltorch_cpu", "-ltorch_python", f"-Wl,-rpath,$ORIGIN,-rpath,{lib}"], "link of the Python binding")
+    os.replace(tmp, NATIVE_PATH)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -64,14 +98,18 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(r.stdout, r.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=max(1, min(8, os.cpu_count() or 1))) as ex:
+    cuda_home = os.path.dirname(os.path.dirname(os.path.realpath(nvcc)))
+    with ThreadPoolExecutor(max_workers=max(1, min(16, os.cpu_count() or 1))) as ex:
+        binding = ex.submit(_compile_binding, cuda_home)
         objs = list(ex.map(compile_one, sources()))
+        binding_obj = binding.result()
     tmp = LIB_PATH + ".tmp"
-    cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs + ["-lcudart_static", "-ldl", "-lpthread", "-lrt"]
+    cmd = [nvcc] + ARCH + ["-shared", "-Xlinker", "-soname=libspade.so", "-o", tmp] + objs + ["-lcudart_static", "-ldl", "-lpthread", "-lrt"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB_PATH)
+    _link_binding(binding_obj)
     return LIB_PATH
 
 
