@@ -1,7 +1,7 @@
 // qkv_cluster.cu -- the verify block's QKV projection with rotary embedding
 // (the attention input side of f_l in x_{l+1} = x_l + f_l(x_l), Sec. III-A, for
-// the d+1 positions of the single forward pass, Sec. III-B) for up to 128 verify
-// rows, where streaming W bounds it.
+// the d+1 positions of the single forward pass, Sec. III-B): few verify rows,
+// where streaming W bounds it, and larger batches over wide layers.
 //
 // Design (GB300):
 //  * Clusters of two CTAs (76 of them cover every SM; clusters of three or more
@@ -30,6 +30,8 @@
 //  * Epilogue: accumulators go to shared memory; the columns of the verify rows
 //    that the peer finishes travel there by one bulk copy (scalar remote stores
 //    took 4.6 us), and each CTA sums, rotates and stores its half of the rows.
+//    With many rows the staging takes the ring's place once both CTAs' MMAs are
+//    done, 128 verify rows at a time.
 #include "qkv_common.cuh"
 
 namespace spade {
@@ -38,9 +40,11 @@ namespace pair {
 
 constexpr int kThreads = 320;                  // producer warp, MMA warp, eight epilogue warps
 constexpr int kEpiThreads = 256;
-constexpr int kMaxRows = 128;                  // verify rows
+constexpr int kMaxRows = 512;                  // verify rows
 constexpr int kMaxStages = 12;
-constexpr int kMinStages = 4;
+constexpr int kMinStages = 4;                  // staging beside the ring
+constexpr int kMinStagesOver = 3;              // staging in the ring's place
+constexpr int kBatch = 128;                    // verify rows staged at once in the ring's place
 constexpr int kMaxPiece = 16;                  // quads of a piece (a head of dimension 128)
 constexpr int kMaxQuads = 64;                  // quads of a cluster's range (512 rows)
 constexpr int kSmemBudget = 222 * 1024;
@@ -48,7 +52,7 @@ constexpr int kTileBytes = 128 * kKChunk * 2;  // one 128-row operand x one k-ch
 
 struct Maps {
   CUtensorMap w[kMaxPiece];  // boxes of 1 .. 16 quads (those in use)
-  CUtensorMap x;
+  CUtensorMap x0, x1;        // verify rows up to 256, the rest
 };
 
 struct Params {
@@ -58,16 +62,19 @@ struct Params {
   int KC;                // k-chunks (ceil(H / 64))
   int Ncols;             // verify rows rounded up to 16: MMA N
   int stages;
+  int over;              // staging in the ring's place
+  int batch;             // verify rows staged at once (R when the staging has its own room)
   uint32_t tmem_cols;
 };
 
 // Shared-memory plan (offsets from a 1024-byte aligned base): tables first, then
-// the ring, then the staging: this CTA's partial sums, and those received for the
-// verify rows that it finishes.
+// the ring, then the staging (or, in the ring's place, a pad for the last
+// operand's read): this CTA's partial sums of a batch of verify rows, and those
+// received for the rows that it finishes.
 struct Layout {
   int rseq, rpos, freq, qrow, bars, misc, ring, stage_bytes, row_stride, part, recv, total;
 };
-__host__ __device__ inline Layout layout(int R, int Ncols, int qmax, int stages) {
+__host__ __device__ inline Layout layout(int Ncols, int qmax, int stages, int over, int batch) {
   Layout L;
   L.rseq = 0;
   L.rpos = L.rseq + kMaxRows * 4;
@@ -77,11 +84,12 @@ __host__ __device__ inline Layout layout(int R, int Ncols, int qmax, int stages)
   L.misc = L.bars + (2 * kMaxStages + 2) * 8;
   L.ring = (L.misc + 32 + 1023) & ~1023;
   L.stage_bytes = qmax * 1024 + Ncols * 128;  // 8 W rows per quad, then the x rows
-  L.part = L.ring + stages * L.stage_bytes;
+  const int end = L.ring + stages * L.stage_bytes;
   L.row_stride = qmax * 8 + 4;                // floats per staged verify row
-  L.recv = L.part + R * L.row_stride * 4;
-  const int staging = (R + (R + 1) / 2) * L.row_stride * 4;
-  L.total = L.part + (staging > kTileBytes ? staging : kTileBytes) + 1024;  // + slack for the 1024-byte alignment
+  const int staging = (batch + (batch + 1) / 2) * L.row_stride * 4;
+  L.part = over ? L.ring : end;
+  L.recv = L.part + batch * L.row_stride * 4;
+  L.total = end + (over || staging < kTileBytes ? kTileBytes : staging) + 1024;  // + slack for the 1024-byte alignment
   return L;
 }
 
@@ -90,11 +98,14 @@ __device__ __forceinline__ void epi_bar() {
   asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
 }
 
+// kBig: more than 128 verify rows are possible (a second N-chunk, staging in the
+// ring's place); the small form has neither test in its loops.
+template <bool kBig>
 __global__ void __launch_bounds__(kThreads, 1)
     qkv_cluster_kernel(const __grid_constant__ Params p, const __grid_constant__ Maps maps) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  const Layout L = layout(p.c.R, p.Ncols, p.qmax, p.stages);
+  const Layout L = layout(p.Ncols, p.qmax, p.stages, p.over, p.batch);
   int32_t *s_rseq = reinterpret_cast<int32_t *>(smem + L.rseq);
   int32_t *s_rpos = reinterpret_cast<int32_t *>(smem + L.rpos);
   float *s_freq = reinterpret_cast<float *>(smem + L.freq);
@@ -114,9 +125,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int rows = nq * 8;                  // W rows of the cluster
   const int ntile = (rows + 127) / 128;     // 128-row operands
   const int qph = p.c.D / 8;                // quads per head
-  // Verify rows [0, h0) are finished by CTA 0, [h0, R) by CTA 1.
-  const int h0 = (p.c.R + 1) / 2;
-  const int n_own = rank ? p.c.R - h0 : h0, n_send = p.c.R - n_own;
+  const int n0 = kBig ? min(p.Ncols, 256) : p.Ncols, n1 = kBig ? p.Ncols - n0 : 0;  // MMA N-chunks
+  // Of the nb verify rows of a batch, the first half is finished by CTA 0.
+  auto own_rows = [rank](int nb) { return rank ? nb - (nb + 1) / 2 : (nb + 1) / 2; };
   // This CTA's half of K.  Every cluster reads the same x rows: each starts at
   // another chunk, so that they do not all load the same lines from L2 at once.
   const int kc0 = p.KC * static_cast<int>(rank) / 2, nk = p.KC * (static_cast<int>(rank) + 1) / 2 - kc0;
@@ -126,7 +137,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) *s_abort = 0;
   for (int j = tid; j < p.c.D / 2; j += kThreads) s_freq[j] = p.c.inv_freq[j];
   if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&maps.x);
+    tma_prefetch_desc(&maps.x0);
+    if (n1) tma_prefetch_desc(&maps.x1);
     // Pieces: one box per head.  A box lands as its pairs' rows of the first
     // half, then of the second; s_qrow: where a quad's four rows of each half start.
     for (int q = q0; q < q0 + nq;) {
@@ -147,7 +159,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(acc_full, 1);
       mbar_init(recv_full, 1);
       fence_mbar_init();
-      if (n_own > 0) mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(n_own * L.row_stride * 4));
+      mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(own_rows(min(p.batch, p.c.R)) * L.row_stride * 4));
     }
     __syncwarp();
     tmem_alloc(s_tmem, p.tmem_cols);
@@ -185,7 +197,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (leader) tma_load_4d(stage + q * 1024, &maps.w[take - 1], kx, j * 4, 0, h, &full[s], pol_w);
         q += take;
       }
-      if (leader) tma_load_2d(stage + xoff, &maps.x, kx, 0, &full[s], pol_x);
+      if (leader) tma_load_2d(stage + xoff, &maps.x0, kx, 0, &full[s], pol_x);
+      if (n1) {
+        if (leader) tma_load_2d(stage + xoff + n0 * 128, &maps.x1, kx, n0, &full[s], pol_x);
+      }
       if (++kc == kc0 + nk) kc = kc0;
       if (++s == p.stages) { s = 0; ph ^= 1u; }
     }
@@ -198,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     // ============================ MMA issuer ===============================
     const bool leader = elect_one();
-    const uint32_t idesc = idesc_bf16_f32(128, p.Ncols);
+    const uint32_t idesc0 = idesc_bf16_f32(128, n0), idesc1 = idesc_bf16_f32(128, n1 ? n1 : 16);
     int s = 0;
     uint32_t ph = 0;
     bool ok = true;
@@ -208,13 +223,17 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t base = smem_u32(smem + L.ring + s * L.stage_bytes);
       // Descriptors built once per operand; a K step of 16 adds 32 bytes, 2 in
       // the descriptor's address field.
-      const uint64_t db = smem_desc_sw128(base + xoff);
+      const uint64_t db0 = smem_desc_sw128(base + xoff), db1 = smem_desc_sw128(base + xoff + n0 * 128);
       for (int t = 0; t < ntile; ++t) {
         const uint64_t da = smem_desc_sw128(base + t * kTileBytes);
         const uint32_t d = tmem + static_cast<uint32_t>(t * p.Ncols);
 #pragma unroll
-        for (int kk = 0; kk < kKChunk / 16; ++kk)
-          if (leader) tc_mma_f16(d, da + 2u * kk, db + 2u * kk, idesc, (it > 0 || kk > 0) ? 1u : 0u);
+        for (int kk = 0; kk < kKChunk / 16; ++kk) {
+          if (leader) tc_mma_f16(d, da + 2u * kk, db0 + 2u * kk, idesc0, (it > 0 || kk > 0) ? 1u : 0u);
+          if (n1) {
+            if (leader) tc_mma_f16(d + 256u, da + 2u * kk, db1 + 2u * kk, idesc1, (it > 0 || kk > 0) ? 1u : 0u);
+          }
+        }
       }
       if (leader) tc_commit(&empty[s]);
       if (++s == p.stages) { s = 0; ph ^= 1u; }
@@ -224,67 +243,82 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
     }
   } else {
-    // ===================== epilogue warps: stage the partial sums ==========
-    const int et = tid - 64, q4 = warp & 3, part = (warp - 2) >> 2;
-    build_rows(p.c, s_rseq, s_rpos, et, kEpiThreads, [] { epi_bar(); });
+    // ===================== epilogue warps: wait for the accumulators =======
+    build_rows(p.c, s_rseq, s_rpos, tid - 64, kEpiThreads, [] { epi_bar(); });
     if (nk > 0) {
       if (!mbar_wait(acc_full, 0, s_abort)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
       tc_fence_after();
     }
-    // Two warps per lane quarter, each every second 16 columns.
-    const int R = p.c.R;
-    for (int t = 0; t < ntile; ++t) {
-      if (t * 128 + q4 * 32 >= rows) break;  // (whole warps: rows is a multiple of 8)
-      const int row = t * 128 + q4 * 32 + lane;
-      const uint32_t a = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(t * p.Ncols);
-      for (int c = 16 * part; c < p.Ncols; c += 32) {
-        uint32_t v[16];
-        if (nk > 0) {
-          tmem_ld8(a + c, v);
-          tmem_ld8(a + c + 8, v + 8);
-          tmem_wait_ld();
-        } else {  // (one k-chunk in all: this CTA has none)
+  }
+  if constexpr (kBig) {
+    __syncwarp();
+    __syncthreads();
+    cluster_sync();  // both rings are idle: their place becomes staging
+  }
+  const OutMap om = out_map(p.c);
+  float *part = reinterpret_cast<float *>(smem + L.part);
+  const float *recv = reinterpret_cast<const float *>(smem + L.recv);
+  uint32_t phase = 0;
+  for (int b0 = 0; b0 < p.c.R; b0 += p.batch, phase ^= 1u) {
+    const int nb = kBig ? min(p.batch, p.c.R - b0) : p.c.R, n_own = own_rows(nb), n_send = nb - n_own;
+    const int first = rank ? nb - n_own : 0, first_send = rank ? 0 : n_own;  // within the batch
+    if (warp >= 2) {
+      // Two warps per lane quarter, each every second 16 columns.
+      const int q4 = warp & 3;
+      for (int t = 0; t < ntile; ++t) {
+        if (t * 128 + q4 * 32 >= rows) break;  // (whole warps: rows is a multiple of 8)
+        const int row = t * 128 + q4 * 32 + lane;
+        const uint32_t a = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(t * p.Ncols + b0);
+        for (int c = 16 * ((warp - 2) >> 2); c < nb; c += 32) {
+          uint32_t v[16];
+          if (nk > 0) {
+            tmem_ld8(a + c, v);
+            tmem_ld8(a + c + 8, v + 8);
+            tmem_wait_ld();
+          } else {  // (one k-chunk in all: this CTA has none)
 #pragma unroll
-          for (int e = 0; e < 16; ++e) v[e] = 0u;
-        }
-        if (row < rows) {
-          float *to = reinterpret_cast<float *>(smem + L.part) + c * L.row_stride + row;
+            for (int e = 0; e < 16; ++e) v[e] = 0u;
+          }
+          if (row < rows) {
+            float *to = part + c * L.row_stride + row;
 #pragma unroll
-          for (int e = 0; e < 16; ++e)
-            if (c + e < R) to[e * L.row_stride] = __uint_as_float(v[e]);
+            for (int e = 0; e < 16; ++e)
+              if (c + e < nb) to[e * L.row_stride] = __uint_as_float(v[e]);
+          }
         }
       }
+      // The peer's rows travel in one copy.
+      fence_proxy_async_smem();
+      epi_bar();
+      if (tid == 64 && n_send > 0)
+        bulk_copy_cluster(cluster_map(recv, rank ^ 1u), part + first_send * L.row_stride,
+                          static_cast<uint32_t>(n_send * L.row_stride * 4), cluster_map(recv_full, rank ^ 1u));
     }
-    tc_fence_before();
-    // The peer's rows travel in one copy.
-    fence_proxy_async_smem();
-    epi_bar();
-    const uint8_t *send = smem + L.part + (rank ? 0 : h0) * L.row_stride * 4;
-    if (et == 0 && n_send > 0)
-      bulk_copy_cluster(cluster_map(smem + L.recv, rank ^ 1u), send, static_cast<uint32_t>(n_send * L.row_stride * 4),
-                        cluster_map(recv_full, rank ^ 1u));
-  }
-  __syncwarp();
-  __syncthreads();
-  {
-    const int n0 = rank ? h0 : 0;
-    const float *own = reinterpret_cast<const float *>(smem + L.part) + n0 * L.row_stride;
-    const float *recv = reinterpret_cast<const float *>(smem + L.recv);
-    if (n_own > 0 && !mbar_wait_unabortable(recv_full, 0)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
-    const OutMap om = out_map(p.c);
+    __syncwarp();
+    __syncthreads();
+    if (!mbar_wait_unabortable(recv_full, phase)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
     for (int it = tid; it < n_own * nq; it += kThreads) {
       const int n = it / nq, q = it - n * nq;
-      const int b = s_rseq[n0 + n];
+      const int r = b0 + first + n;
+      const int b = s_rseq[r];
       if (b < 0) continue;
-      const int at1 = n * L.row_stride + s_qrow[2 * q], at2 = n * L.row_stride + s_qrow[2 * q + 1];
+      const float *o = part + (first + n) * L.row_stride, *i = recv + n * L.row_stride;
+      const int r1 = s_qrow[2 * q], r2 = s_qrow[2 * q + 1];
       float y1[4], y2[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        y1[e] = own[at1 + e] + recv[at1 + e];
-        y2[e] = own[at2 + e] + recv[at2 + e];
+        y1[e] = o[r1 + e] + i[r1 + e];
+        y2[e] = o[r2 + e] + i[r2 + e];
       }
       const int Q = q0 + q, hg = Q / qph;
-      store_quad(om, s_freq, b, n0 + n, s_rpos[n0 + n], hg, (Q - hg * qph) * 4, y1, y2);
+      store_quad(om, s_freq, b, r, s_rpos[r], hg, (Q - hg * qph) * 4, y1, y2);
+    }
+    if (kBig && b0 + p.batch < p.c.R) {
+      if (tid == 0)
+        mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(own_rows(min(p.batch, p.c.R - b0 - p.batch)) * L.row_stride * 4));
+      __syncwarp();
+      __syncthreads();
+      cluster_sync();  // both CTAs have read their staging, and their copies have left it
     }
   }
   tc_fence_before();
@@ -294,7 +328,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem, p.tmem_cols);
   }
-  cluster_sync();  // the copy to the peer has left this CTA's shared memory
+  cluster_sync();  // the last copy to the peer has left this CTA's shared memory
 }
 
 // W [(Hq + 2 Hkv) D, H] as {H, D / 2 pairs, 2 halves, heads}, box {64, pairs, 2, 1},
@@ -321,25 +355,44 @@ static Params plan(const Call &c, int sms) {
   if (cols > 512 || p.qmax > kMaxQuads) return p;
   p.tmem_cols = 32;
   while (p.tmem_cols < static_cast<uint32_t>(cols)) p.tmem_cols *= 2;
-  const Layout L = layout(c.R, p.Ncols, p.qmax, 0);
-  const int n = (kSmemBudget - L.total) / L.stage_bytes;
-  p.stages = n > kMaxStages ? kMaxStages : n;
+  auto depth = [&](int over, int batch) {
+    const Layout L = layout(p.Ncols, p.qmax, 0, over, batch);
+    const int n = (kSmemBudget - L.total) / L.stage_bytes;
+    return n > kMaxStages ? kMaxStages : n;
+  };
+  int n = depth(0, c.R);
+  if (c.R <= 128 && n >= kMinStages) {
+    p.stages = n;
+    p.batch = c.R;
+    return p;
+  }
+  // More rows: every cluster reads all of x, so its range must have enough W rows
+  // (64) for the x rows it loads; the stream-K form has 128 per x row.
+  n = depth(1, kBatch);
+  const Layout L = layout(p.Ncols, p.qmax, n, 1, kBatch);
+  if (p.qmax >= 8 && n >= kMinStagesOver && L.recv + kBatch / 2 * L.row_stride * 4 <= L.ring + n * L.stage_bytes) {
+    p.stages = n;
+    p.over = 1;
+    p.batch = kBatch;
+  }
   return p;
 }
 
 }  // namespace pair
 
-// The cluster form streams W at the rate its ring allows: it takes the call when
-// at least kMinStages fit (fewer rows, or ranges of fewer quads); larger calls
-// spend their time in the MMAs and the rows' traffic, and the stream-K form
-// gives an SM 128 rows of W per x row it loads.
-bool cluster_fits(const Call &c, int sms) { return pair::plan(c, sms).stages >= pair::kMinStages; }
+// Up to 128 rows the cluster form streams W at the rate its ring allows and is
+// taken when at least four stages fit: 14.0 us at 72 rows against 20.5 us of the
+// stream-K form. Above, see plan().
+bool cluster_fits(const Call &c, int sms) { return pair::plan(c, sms).stages > 0; }
 
 spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int sms, cudaStream_t stream) {
   using namespace pair;
   const Params p = plan(c, sms);
   Maps m;
-  if (!encode_tmap_bf16_sw128(&m.x, x, c.H, c.R, static_cast<uint64_t>(c.H) * 2, kKChunk, p.Ncols)) return SPADE_ERR_CUDA;
+  const uint64_t pitch = static_cast<uint64_t>(c.H) * 2;
+  const int n0 = p.Ncols < 256 ? p.Ncols : 256;
+  if (!encode_tmap_bf16_sw128(&m.x0, x, c.H, c.R, pitch, kKChunk, n0)) return SPADE_ERR_CUDA;
+  if (p.Ncols > n0 && !encode_tmap_bf16_sw128(&m.x1, x, c.H, c.R, pitch, kKChunk, p.Ncols - n0)) return SPADE_ERR_CUDA;
   // The piece sizes that some cluster's range has.
   const int qph = c.D / 8;
   uint32_t used = 0;
@@ -354,14 +407,16 @@ spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int
   }
   static bool configured = false;
   if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(qkv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(qkv_cluster)");
+    for (auto kern : {qkv_cluster_kernel<false>, qkv_cluster_kernel<true>}) {
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(qkv_cluster)");
+    }
     configured = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.nclusters);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = layout(c.R, p.Ncols, p.qmax, p.stages).total;
+  cfg.dynamicSmemBytes = layout(p.Ncols, p.qmax, p.stages, p.over, p.batch).total;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -372,7 +427,7 @@ spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, qkv_cluster_kernel, p, m);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, p.over ? qkv_cluster_kernel<true> : qkv_cluster_kernel<false>, p, m);
   if (e != cudaSuccess) return cuda_fail(e, "qkv_cluster launch");
   return SPADE_OK;
 }
