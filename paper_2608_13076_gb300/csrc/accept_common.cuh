@@ -34,8 +34,7 @@ constexpr int kTmemCols = 512;
 constexpr int kSmemMax = 227 * 1024;                // shared memory a CTA may have
 constexpr int kWChunkBytes = kTileV * kKChunk * 2;  // 16 KB: one tile x one k-chunk
 constexpr int kBlk = 16;       // verify rows per statistics block
-constexpr int kTStride = kBlk + 1;
-constexpr int kTBufBytes = kEpiWarps * 32 * kTStride * 4;  // the warps' transpose buffers
+constexpr int kTBufBytes = kBlk * 32 * 4;           // one statistics warp's transpose buffer
 constexpr float kLog2e = 1.4426950408889634f;
 
 // One accept call: inputs, outputs and workspace.
@@ -334,22 +333,23 @@ __device__ __forceinline__ RowTables row_tables(uint8_t *mem, int nrows, bool uq
   t.keep = reinterpret_cast<unsigned *>((uq ? t.q : t.it) + nrows);
   return t;
 }
-// Filled by the epilogue warps (thread et of kEpiThreads) while the first
-// stages already stream.
+// Filled by the epilogue warps (thread et of kN) while the first stages already
+// stream.
+template <int kN>
 __device__ __forceinline__ void setup_rows(const Call &p, int nrows, SeqTable &seqs, const RowTables &t, int et) {
-  for (int n = et; n < nrows; n += kEpiThreads) { t.draft[n] = -1; t.it[n] = 1.f; }
-  for (int w = et; w < nrows / kBlk; w += kEpiThreads) t.keep[w] = 0u;
-  fill_table(p, seqs, et / 32, kEpiWarps, et % 32, true);
-  named_bar(1, kEpiThreads);
+  for (int n = et; n < nrows; n += kN) { t.draft[n] = -1; t.it[n] = 1.f; }
+  for (int w = et; w < nrows / kBlk; w += kN) t.keep[w] = 0u;
+  fill_table(p, seqs, et / 32, (kN / 32), et % 32, true);
+  named_bar(1, kN);
   // The rows' sequences (one warp per sequence), then one thread per row, so
   // that the loads of all rows are in flight together.
-  for (int b = et / 32; b < p.B; b += kEpiWarps) {
+  for (int b = et / 32; b < p.B; b += (kN / 32)) {
     const SeqInfo q = table_info(seqs, b);
     if (!q.valid) continue;
     for (int i = et % 32; i <= q.k; i += 32) t.draft[q.r0 + i] = b;
   }
-  named_bar(1, kEpiThreads);
-  for (int n = et; n < p.R; n += kEpiThreads) {
+  named_bar(1, kN);
+  for (int n = et; n < p.R; n += kN) {
     const int b = t.draft[n];
     if (b < 0) continue;
     const SeqInfo q = table_info(seqs, b);
@@ -362,7 +362,7 @@ __device__ __forceinline__ void setup_rows(const Call &p, int nrows, SeqTable &s
       t.q[n] = q.stoch && d >= 0 && d < p.V ? __ldg(&p.draft_probs[static_cast<size_t>(n - b) * p.V + d]) : 0.f;
     }
   }
-  named_bar(1, kEpiThreads);
+  named_bar(1, kN);
 }
 
 // Sets the words that the rows phase's groups exchange to unset (thread i of n
@@ -391,61 +391,102 @@ __device__ __forceinline__ void blk_init(BlkStat &st, int lane) {
   }
 }
 
+// Two fp32 operations in one instruction, each rounded as the scalar one.
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Statistics of 16 verify rows (r0 ..) over one warp's 32 vocabulary entries
-// (v0 + lane), read from the 16 accumulator columns at `taddr`.  A 32 x 17
-// shared-memory transpose gives lane (row = lane % 16, half = lane / 16) one
-// row over 16 entries, reduced serially; the two halves meet by a shuffle each
-// for the maximum and the sum.  The argmax search runs only when the block
-// raises a row's running maximum.  Rows marked in `rows.keep` also store
-// their logits, 128 contiguous bytes per row and warp.
-__device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0, int v0, int v_hi, const RowTables &rows,
-                                           float *T, int lane, BlkStat &st) {
-  uint32_t raw[kBlk];
-  tmem_ld8(taddr, raw);
-  tmem_ld8(taddr + 8, raw + 8);
-  tmem_wait_ld();
-  const bool mine = v0 + lane < v_hi;  // lanes past the slice are masked
-  const unsigned keep = rows.keep[r0 / kBlk];
-  if (keep != 0u) {
-    float *dst = p.logits + static_cast<size_t>(r0) * p.ldl + v0 + lane;
-#pragma unroll
-    for (int r = 0; r < kBlk; ++r)
-      if ((keep >> r) & 1u) {
-        if (mine) dst[static_cast<size_t>(r) * p.ldl] = __uint_as_float(raw[r]);
-      }
-  }
-#pragma unroll
-  for (int r = 0; r < kBlk; ++r) T[lane * kTStride + r] = mine ? __uint_as_float(raw[r]) : -INFINITY;
-  __syncwarp();
-  const int row = lane % kBlk, vb = (lane / kBlk) * kBlk;  // 16 entries from v0 + vb on
+// (v0 + lane), `raw` the lane's accumulator columns.  A 16 x 32 shared-memory
+// transpose (16-byte chunk j of row r at chunk j ^ (r % 8): the stores and the
+// 16-byte loads are free of bank conflicts) gives lane (row = lane % 16,
+// half = lane / 16) one row over 16 entries, reduced serially in pairs; the two
+// halves meet by a shuffle each for the maximum and the sum.  The argmax search
+// runs only when the block raises a row's running maximum.  Rows marked in
+// `rows.keep` also store their logits, 128 contiguous bytes per row and warp.
+__device__ __forceinline__ void stat_block(const Call &p, uint32_t (&raw)[kBlk], int r0, int v0, int v_hi,
+                                           const RowTables &rows, float *T, int lane, BlkStat &st) {
+  const int row = lane % kBlk, half = lane / kBlk, vb = half * kBlk;  // 16 entries from v0 + vb on
   const int n = r0 + row;
   const float it = rows.it[n];  // logits at the row's temperature, l / T
   const float rm = st.m[row];
-  float x[kBlk];
-  float m = -INFINITY;
+  const int d = rows.draft[n] - (v0 + vb);
+  const unsigned keep = rows.keep[r0 / kBlk];
+  const bool whole = v0 + 32 <= v_hi;  // (warp-uniform)
+  if (keep != 0u && v0 + lane < v_hi) {
+    float *dst = p.logits + static_cast<size_t>(r0) * p.ldl + v0 + lane;
+    if (keep == 0xffffu) {
 #pragma unroll
-  for (int i = 0; i < kBlk; ++i) {
-    x[i] = __fmul_rn(T[(vb + i) * kTStride + row], it);
-    m = fmaxf(m, x[i]);
-  }
-  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, kBlk));
-  const float M = fmaxf(rm, m);
-  float a0 = 0.f, a1 = 0.f;
-  if (M != -INFINITY) {
+      for (int r = 0; r < kBlk; ++r) dst[static_cast<size_t>(r) * p.ldl] = __uint_as_float(raw[r]);
+    } else {
 #pragma unroll
-    for (int i = 0; i < kBlk; i += 2) {
-      a0 += ex2((x[i] - M) * kLog2e);
-      a1 += ex2((x[i + 1] - M) * kLog2e);
+      for (int r = 0; r < kBlk; ++r)
+        if ((keep >> r) & 1u) dst[static_cast<size_t>(r) * p.ldl] = __uint_as_float(raw[r]);
     }
   }
-  a0 += a1;
+  if (!whole) {
+#pragma unroll
+    for (int r = 0; r < kBlk; ++r)
+      if (v0 + lane >= v_hi) raw[r] = 0xff800000u;  // lanes past the slice: -infinity
+  }
+#pragma unroll
+  for (int r = 0; r < kBlk; ++r) T[r * 32 + ((((lane >> 2) ^ (r & 7)) << 2) | (lane & 3))] = __uint_as_float(raw[r]);
+  __syncwarp();
+  uint64_t x[kBlk / 2];
+  const uint64_t it2 = f2_pack(it, it);
+#pragma unroll
+  for (int j = 0; j < kBlk / 4; ++j) {
+    const float4 v = *reinterpret_cast<const float4 *>(T + row * 32 + (((half * 4 + j) ^ (row & 7)) << 2));
+    x[2 * j] = f2_mul(f2_pack(v.x, v.y), it2);
+    x[2 * j + 1] = f2_mul(f2_pack(v.z, v.w), it2);
+  }
+  float m = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < kBlk / 2; ++j) {
+    const float2 v = f2_unpack(x[j]);
+    m = fmaxf(m, v.x);
+    m1 = fmaxf(m1, v.y);
+  }
+  m = fmaxf(m, m1);
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, kBlk));
+  const float M = fmaxf(rm, m);
+  const float ref = M == -INFINITY ? 0.f : M;
+  const uint64_t ref2 = f2_pack(-ref, -ref), log2e2 = f2_pack(kLog2e, kLog2e);
+  uint64_t a2 = 0;
+#pragma unroll
+  for (int j = 0; j < kBlk / 2; ++j) {
+    const float2 e = f2_unpack(f2_mul(f2_add(x[j], ref2), log2e2));
+    a2 = f2_add(a2, f2_pack(ex2(e.x), ex2(e.y)));
+  }
+  const float2 a = f2_unpack(a2);
+  float a0 = a.x + a.y;
   a0 += __shfl_xor_sync(0xffffffffu, a0, kBlk);
   const bool raised = m > rm;
   int idx = INT_MAX;
   if (__any_sync(0xffffffffu, raised)) {
 #pragma unroll
-    for (int i = kBlk - 1; i >= 0; --i)
-      if (x[i] == m) idx = v0 + vb + i;
+    for (int j = kBlk / 2 - 1; j >= 0; --j) {
+      const float2 v = f2_unpack(x[j]);
+      if (v.y == m) idx = v0 + vb + 2 * j + 1;
+      if (v.x == m) idx = v0 + vb + 2 * j;
+    }
     idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, kBlk));  // the lowest index of the maximum
   }
   if (lane < kBlk && M != -INFINITY) {
@@ -455,9 +496,15 @@ __device__ __forceinline__ void stat_block(const Call &p, uint32_t taddr, int r0
       st.i[row] = idx;
     }
   }
-  const int d = rows.draft[n] - (v0 + vb);
-  if (d >= 0 && d < kBlk && v0 + vb + d < v_hi) p.ldraft[n] = __fmul_rn(T[(vb + d) * kTStride + row], it);
+  if (d >= 0 && d < kBlk && v0 + vb + d < v_hi)
+    p.ldraft[n] = __fmul_rn(T[row * 32 + (((half * 4 + (d >> 2)) ^ (row & 7)) << 2) + (d & 3)], it);
   __syncwarp();
+}
+
+// The accumulator columns of a block (complete after tmem_wait_ld).
+__device__ __forceinline__ void load_block(uint32_t taddr, uint32_t (&raw)[kBlk]) {
+  tmem_ld8(taddr, raw);
+  tmem_ld8(taddr + 8, raw + 8);
 }
 
 // Merge of the epilogue warps' statistics ([kEpiWarps][nblk], written and

@@ -11,8 +11,8 @@
 //  * Each CTA owns a contiguous vocabulary slice, cut into tiles of equal height
 //    (at most 128 rows): the pair's MMA covers one tile of each.
 //  * Rows up to 256 leave room for two accumulators, and the statistics of a
-//    tile run under the next one's MMAs; more rows fill tensor memory, and the
-//    eight statistics warps release it N-chunk by N-chunk.
+//    tile run under the next one's MMAs; more rows fill tensor memory, and
+//    sixteen statistics warps empty it between tiles.
 //  * The rows of sampled sequences store their fp32 logits (coalesced 128-byte
 //    rows straight from the accumulators).  A draw then reads one stored row
 //    instead of streaming W again: 118 MB written against 1.56 GB re-read at
@@ -23,6 +23,16 @@ namespace spade {
 namespace accept {
 
 constexpr int kMaxStages = 8;
+// Four statistics warps per tensor-memory lane quarter: the statistics of more
+// than 256 rows do not run under the next tile's MMAs, and eight warps leave
+// their latencies uncovered (this launch at 389 rows x 5120 x 152064: 405 us with
+// eight, 380 with sixteen and blocks reduced in pairs; 343 without statistics.
+// Blocks held in registers, so that the next tile's MMAs start under them, gave
+// nothing more: the launch is then short of power, 1.4 kW, not of time).
+constexpr int kPairWarps = 16;
+constexpr int kPairEpi = 32 * kPairWarps;
+constexpr int kPairThreads = 64 + kPairEpi;
+constexpr int kParts = kPairWarps / 4;
 
 struct PairParams {
   Call c;
@@ -47,13 +57,14 @@ __host__ __device__ inline PairSmem pair_layout(int Ncols, int stages) {
   s.off_seq = (s.off_misc + 16 + 15) & ~15;
   s.off_rows = s.off_seq + static_cast<int>(sizeof(SeqTable));
   s.off_stat = s.off_rows + row_table_bytes(Ncols, false);
-  // A statistics warp keeps every second block of rows.
-  s.off_tbuf = (s.off_stat + kEpiWarps * ((Ncols / kBlk + 1) / 2) * static_cast<int>(sizeof(BlkStat)) + 15) & ~15;
-  s.total = s.off_tbuf + kTBufBytes + 1024;
+  // A statistics warp keeps every kParts-th block of rows.
+  const int per = (Ncols / kBlk + kParts - 1) / kParts;
+  s.off_tbuf = (s.off_stat + kPairWarps * per * static_cast<int>(sizeof(BlkStat)) + 127) & ~127;
+  s.total = s.off_tbuf + kPairWarps * kTBufBytes + 1024;
   return s;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
+__global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
     const __grid_constant__ PairParams p, const __grid_constant__ CUtensorMap tm_w,
     const __grid_constant__ CUtensorMap tm_h0, const __grid_constant__ CUtensorMap tm_h1) {
   extern __shared__ uint8_t smem_raw[];
@@ -82,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
   if (tid == 0) {
     *s_abort = 0;
     for (int s = 0; s < p.stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * kEpiWarps); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * kPairWarps); }
     mbar_init(fin, 1);
     if (rank == 0)  // arm every stage's first use with both CTAs' bytes
       for (int s = 0; s < p.stages; ++s) mbar_arrive_expect_tx(&full[s], 2 * stage_tx);
@@ -197,10 +208,10 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
     // ---- statistics warps ----
     const int et = tid - 64, ew = warp - 2, q4 = warp & 3, part = ew >> 2;
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    float *T = reinterpret_cast<float *>(smem + L.off_tbuf) + ew * (32 * kTStride);
-    clear_exchange(p.c, c * kEpiThreads + et, p.c.NC * kEpiThreads);
-    setup_rows(p.c, p.Ncols, *reinterpret_cast<SeqTable *>(smem + L.off_seq), rows, et);
-    const int nblk = p.Ncols / kBlk, per = (nblk + 1) / 2;
+    float *T = reinterpret_cast<float *>(smem + L.off_tbuf + ew * kTBufBytes);
+    clear_exchange(p.c, c * kPairEpi + et, p.c.NC * kPairEpi);
+    setup_rows<kPairEpi>(p.c, p.Ncols, *reinterpret_cast<SeqTable *>(smem + L.off_seq), rows, et);
+    const int nblk = p.Ncols / kBlk, per = (nblk + kParts - 1) / kParts;
     BlkStat *stats = reinterpret_cast<BlkStat *>(smem + L.off_stat) + ew * per;
     for (int j = 0; j < per; ++j) blk_init(stats[j], lane);
     __syncwarp();
@@ -214,8 +225,12 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
       const uint32_t col = tmem + lane_base + static_cast<uint32_t>(buf * (kTmemCols / 2));
       if (v0 < hi) {
 #pragma unroll 1
-        for (int bk = part; bk < nblk; bk += 2)
-          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, hi, rows, T, lane, stats[bk >> 1]);
+        for (int bk = part; bk < nblk; bk += kParts) {
+          uint32_t raw[kBlk];
+          load_block(col + bk * kBlk, raw);
+          tmem_wait_ld();
+          stat_block(p.c, raw, bk * kBlk, v0, hi, rows, T, lane, stats[bk / kParts]);
+        }
       }
       // The accumulator is read: the MMA thread counts both CTAs' warps.
       tc_fence_before();
@@ -226,15 +241,15 @@ __global__ void __launch_bounds__(kThreads, 1) lm_head_pairs_kernel(
       }
     }
     // Merge the warps' statistics and publish this CTA's slice partials.
-    named_bar(1, kEpiThreads);
+    named_bar(1, kPairEpi);
     const BlkStat *all = reinterpret_cast<const BlkStat *>(smem + L.off_stat);
-    for (int n = et; n < p.c.R; n += kEpiThreads) {
+    for (int n = et; n < p.c.R; n += kPairEpi) {
       const int bk = n / kBlk;
       float m = -INFINITY, z = 0.f;
       int idx = INT_MAX;
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
-        const BlkStat &st = all[((bk & 1) * 4 + w) * per + (bk >> 1)];
+        const BlkStat &st = all[((bk % kParts) * 4 + w) * per + bk / kParts];
         stat_merge(m, z, idx, st.m[n % kBlk], st.s[n % kBlk], st.i[n % kBlk]);
       }
       __stcg(&p.c.pstat[static_cast<size_t>(n) * p.c.NC + c], make_float4(m, z, __int_as_float(idx), 0.f));
@@ -309,7 +324,7 @@ spade_status launch_lm_head_pairs(const Call &c, const void *hidden, const void 
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c.NC);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(kPairThreads);
   cfg.dynamicSmemBytes = pair_layout(p.Ncols, p.stages).total;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];

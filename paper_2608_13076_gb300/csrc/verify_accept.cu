@@ -68,7 +68,7 @@ __host__ __device__ inline Smem smem_layout(const Params &p) {
   s.off_rows = s.off_seq + static_cast<int>(sizeof(SeqTable));
   s.off_stat = s.off_rows + row_table_bytes(p.Ncols, true);
   s.off_tbuf = (s.off_stat + kEpiWarps * (p.Ncols / kBlk) * static_cast<int>(sizeof(BlkStat)) + 127) & ~127;
-  s.total = s.off_tbuf + kTBufBytes + 1024;
+  s.total = s.off_tbuf + kEpiWarps * kTBufBytes + 1024;
   return s;
 }
 
@@ -264,9 +264,9 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
     const int q4 = warp & 3;             // TMEM lane quarter this warp may access
     const int part = ew >> 2;            // which of the quarter's two warps
     const uint32_t lane_base = static_cast<uint32_t>(q4 * 32) << 16;
-    float *T = reinterpret_cast<float *>(smem + L.off_tbuf) + ew * (32 * kTStride);
+    float *T = reinterpret_cast<float *>(smem + L.off_tbuf + ew * kTBufBytes);
     clear_exchange(p.c, c * kEpiThreads + et, p.c.NC * kEpiThreads);
-    setup_rows(p.c, p.Ncols, seqs, rows, et);
+    setup_rows<kEpiThreads>(p.c, p.Ncols, seqs, rows, et);
     // The quarter's two warps take the (tile, 16-row block) items in turn; each
     // keeps running statistics of every block, in shared memory (one copy of
     // the block's code, whatever the row count).
@@ -287,8 +287,12 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
         if (v0 >= v_hi) break;  // the slice ends before this quarter of its last tile
         const uint32_t col = tmem + lane_base + static_cast<uint32_t>(buf * kHalfCols + j * p.Ncols);
 #pragma unroll 1
-        for (int bk = (t * nblk + part) & 1; bk < nblk; bk += 2)
-          stat_block(p.c, col + bk * kBlk, bk * kBlk, v0, v_hi, rows, T, lane, stats[bk]);
+        for (int bk = (t * nblk + part) & 1; bk < nblk; bk += 2) {
+          uint32_t raw[kBlk];
+          load_block(col + bk * kBlk, raw);
+          tmem_wait_ld();
+          stat_block(p.c, raw, bk * kBlk, v0, v_hi, rows, T, lane, stats[bk]);
+        }
       }
       tc_fence_before();
       __syncwarp();
