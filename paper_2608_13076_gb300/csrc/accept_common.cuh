@@ -523,10 +523,10 @@ __device__ __forceinline__ void publish_slice(const Call &p, const BlkStat *stat
 }
 
 // Shared memory of the rows phase.
-constexpr int kPiece = 8192;       // entries of a share that the draw holds in shared memory at once
+constexpr int kPiece = 8192;       // entries of a share that the draw takes at a time
 constexpr int kMaxPieces = 80;     // 622592 entries, the largest vocabulary
 struct RowsSmem {
-  uint64_t bar;          // bulk copies of a piece
+  uint64_t bar[2];       // bulk copies of a piece, by buffer
   int n_st, n_gr, first, nl, owner_piece, owner_warp, retry, abort;
   ff2 tgt, before;
   ff2 pm[kMaxPieces][kWarps];  // masses of the warps' parts of each piece of this CTA's share
@@ -537,19 +537,20 @@ struct RowsSmem {
   int arg[kMaxR], d[kMaxR], ok[kMaxR];
   int tkey[kMaxR];       // nucleus key threshold (INT_MIN: all of p)
   union alignas(16) {
-    struct {
-      float l[kPiece], q[kPiece];     // the piece's logits (then its terms) and draft distribution
-    } piece;
+    float piece[2 * kPiece];  // a piece's logits (then its terms) and draft distribution: the first buffer
     float bins[kWarps][kNucSubs * kNucBins * 32];  // nucleus search
   };
   // Nucleus search only (one-launch path, at most 256 rows):
   int npre[kMaxRes];
   unsigned nab[kMaxRes];
   // Call::pool bytes: unsigned hist[rows][kNucBins], uint16_t cnt[items][32]
-  // (list lengths per item and lane), float list[items][entries][32].
-  uint8_t pool[16];
+  // (list lengths per item and lane), float list[items][entries][32]; then, if it
+  // is large enough, the draw's second buffer of a piece.
+  alignas(16) uint8_t pool[16];
 };
-constexpr size_t kRowsBytesPlain = offsetof(RowsSmem, piece) + 2 * kPiece * sizeof(float);
+constexpr int kPieceBytes = 2 * kPiece * sizeof(float);
+constexpr size_t kRowsBytesPlain = offsetof(RowsSmem, piece) + kPieceBytes;
+constexpr size_t kRowsBytesDouble = offsetof(RowsSmem, pool) + kPieceBytes;
 static_assert(offsetof(RowsSmem, piece) % 16 == 0, "bulk copies need 16-byte alignment");
 constexpr int kPoolPerRow = kNucBins * 4 + 32 * 2;  // bins and list lengths of one searched row
 
@@ -970,30 +971,41 @@ struct Dist {
 // read distinct banks).
 __device__ __forceinline__ int lane_block(int len) { return ((len + kThreads - 1) / kThreads) | 1; }
 
-// Loads entries [e0, e0 + len) of the logits row (and of q) into shared memory,
-// replaces the logits by the terms of the distribution and returns the
-// inclusive prefix of this lane's block sum over the warp.  The piece arrives
-// by bulk copies (q by plain loads when its rows are not 16-byte aligned).
+__device__ __forceinline__ float *piece_buf(RowsSmem &s, int buf) {
+  return buf == 0 ? s.piece : reinterpret_cast<float *>(s.pool);
+}
+// Issues the bulk copies of entries [e0, e0 + len) of the logits row (and of q) into
+// a buffer that no thread uses (warp kCopyWarp, after a barrier; a whole warp, as
+// the copies' operands live in uniform registers).
+constexpr int kCopyWarp = 2;  // (on a scheduler with two of the ten warps)
+__device__ __forceinline__ void piece_copy(const Call &p, RowsSmem &s, const Dist &t, int e0, int len, int buf) {
+  float *sl = piece_buf(s, buf);
+  const bool leader = elect_one(), bulk_q = t.q != nullptr && p.qvec;
+  const uint32_t bytes = static_cast<uint32_t>(uniform((len + 3) & ~3)) * 4u;
+  const float *lsrc = uniform(t.lg + e0), *qsrc = uniform(t.q + e0);
+  if (leader) {
+    fence_proxy_async();  // earlier generic accesses, and the logits' stores, come first
+    mbar_arrive_expect_tx(&s.bar[buf], bulk_q ? 2 * bytes : bytes);
+    bulk_load(sl, lsrc, bytes, &s.bar[buf]);
+    if (bulk_q) bulk_load(sl + kPiece, qsrc, bytes, &s.bar[buf]);
+  }
+  __syncwarp();
+}
+// Waits for a piece, replaces its logits by the terms of the distribution and
+// returns the inclusive prefix of this lane's block sum over the warp.  (q comes by
+// plain loads when its rows are not 16-byte aligned.)
 // The terms are fp32; sums are compensated (the terms are >= 0, so ordering the
 // two addends by size makes the error term exact).
-__device__ __forceinline__ ff2 piece_terms(const Call &p, RowsSmem &s, const Dist &t, int e0, int len, uint32_t parity,
-                                        int tid, int warp, int lane) {
-  float *sl = s.piece.l, *sq = s.piece.q;
-  const bool bulk_q = t.q != nullptr && p.qvec;
-  if (tid == 0) {
-    fence_proxy_async();  // earlier generic accesses, and the logits' stores, come first
-    const uint32_t bytes = static_cast<uint32_t>((len + 3) & ~3) * 4u;
-    mbar_arrive_expect_tx(&s.bar, bulk_q ? 2 * bytes : bytes);
-    bulk_load(sl, t.lg + e0, bytes, &s.bar);
-    if (bulk_q) bulk_load(sq, t.q + e0, bytes, &s.bar);
-  }
-  if (t.q != nullptr && !bulk_q) {
+__device__ __forceinline__ ff2 piece_terms(const Call &p, RowsSmem &s, const Dist &t, int e0, int len, int buf,
+                                           uint32_t parity, int tid, int warp, int lane) {
+  float *sl = piece_buf(s, buf), *sq = sl + kPiece;
+  if (t.q != nullptr && !p.qvec) {
 #pragma unroll 4
     for (int e = tid; e < len; e += kThreads) sq[e] = __ldg(t.q + e0 + e);
   }
   // (the copies read valid memory: this wait does not give up on an earlier
   // expired wait, so that no copy is left in flight at exit)
-  if (!mbar_wait_unabortable(&s.bar, parity)) {
+  if (!mbar_wait_unabortable(&s.bar[buf], parity)) {
     atomicOr(p.status, SPADE_DEV_TIMEOUT);
     s.abort = 1;
   }
@@ -1001,16 +1013,39 @@ __device__ __forceinline__ ff2 piece_terms(const Call &p, RowsSmem &s, const Dis
   const int bs = lane_block(len);
   const int b0 = (warp * 32 + lane) * bs, b1 = min(len, b0 + bs);
   float sh = 0.f, lo = 0.f;
-#pragma unroll 4
-  for (int e = b0; e < b1; ++e) {
-    const float lv = __fmul_rn(sl[e], t.IT);
-    const bool in = t.tkey == INT_MIN || nuc_key(lv, t.base) >= t.tkey;
-    const float pv = in ? ex2((lv - t.M) * kLog2e) * t.invS : 0.f;
-    const float x = t.q != nullptr ? fmaxf(0.f, pv - sq[e]) : pv;
-    sl[e] = x;
-    const float sm = sh + x;
-    lo += (fmaxf(sh, x) - sm) + fminf(sh, x);
-    sh = sm;
+  // Four entries' loads come before any of their stores (entry by entry, each load
+  // waits for the store before it); bound by its ~17 instructions an entry.
+  const float nM = -t.M;
+#pragma unroll 1
+  for (int e = b0; e < b1; e += 4) {
+    float x[4], qx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool in = e + j < b1;
+      x[j] = in ? sl[e + j] : -INFINITY;
+      qx[j] = in && t.q != nullptr ? sq[e + j] : 0.f;
+    }
+    float pv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      x[j] = __fmul_rn(x[j], t.IT);
+      pv[j] = ex2((x[j] + nM) * kLog2e) * t.invS;
+    }
+    if (t.tkey != INT_MIN) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (nuc_key(x[j], t.base) < t.tkey) pv[j] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float v = t.q != nullptr ? fmaxf(0.f, pv[j] - qx[j]) : pv[j];
+      if (e + j < b1) {
+        sl[e + j] = v;
+        const float sm = sh + v;
+        lo += (fmaxf(sh, v) - sm) + fminf(sh, v);
+        sh = sm;
+      }
+    }
   }
   return warp_scan_ff(ff_norm(sh, lo), lane);
 }
@@ -1023,8 +1058,11 @@ __device__ __forceinline__ ff2 piece_terms(const Call &p, RowsSmem &s, const Dis
 // with no mass is retried on p (every CTA sees the same total, so all retry
 // together).  Bound by the latency of its few dependent steps, and by fetching
 // its code: loops are rolled.
+// A share of more than one piece has the next piece's copies in flight under this
+// one's sums where shared memory holds two (389 rows, 32 of 64 sequences sampled,
+// shares of 38016 entries: the second launch 30 -> 26 us with that and terms taken four at a time).
 // `commit`: the group's first CTA updates the cache while the masses travel.
-// `parity`: phase of the copies' mbarrier, advanced by every piece.
+// `parity`: phases of the buffers' mbarriers (bit: buffer), flipped by every piece.
 __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, const SeqInfo &q, int a, int rank, int gs,
                                            int lo, int hi, bool commit, uint32_t &parity, int tid, int warp,
                                            int lane) {
@@ -1039,16 +1077,24 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
   t.tkey = s.tkey[a];
   const float u = p.uniforms[q.r0 + q.k];
   const int npiece = (hi - lo + kPiece - 1) / kPiece;
+  const int nbuf = p.pool >= kPieceBytes ? 2 : 1;
+  auto copy = [&](int j) {
+    if (warp == kCopyWarp && j < npiece) piece_copy(p, s, t, lo + j * kPiece, min(kPiece, hi - lo - j * kPiece), j % nbuf);
+  };
   ff2 incl;
   int i = 0, attempt = 0;
   bool again = false;  // the owner takes the piece that holds the target once more
+  for (int j = 0; j < nbuf; ++j) copy(j);
 #pragma unroll 1
   for (;;) {  // (one copy of the piece's code)
-    incl = piece_terms(p, s, t, lo + i * kPiece, min(kPiece, hi - lo - i * kPiece), parity, tid, warp, lane);
-    parity ^= 1u;
+    const int buf = i % nbuf;
+    incl = piece_terms(p, s, t, lo + i * kPiece, min(kPiece, hi - lo - i * kPiece), buf, (parity >> buf) & 1u, tid, warp,
+                       lane);
+    parity ^= 1u << buf;
     if (again) break;
     if (lane == 31) s.pm[i][warp] = incl;
     block_sync();
+    copy(i + nbuf);
     if (++i < npiece) continue;
     unsigned long long *zp = p.zpart + (static_cast<size_t>(attempt) * p.B + b) * kMaxGroup;
     if (warp == 0) {
@@ -1109,14 +1155,17 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
       attempt = 1;
       t.q = nullptr;
       i = 0;
+      for (int j = 0; j < nbuf; ++j) copy(j);
       continue;
     }
     if (s.owner_piece < 0) return;
     if (s.owner_piece == npiece - 1) break;
     i = s.owner_piece;
+    copy(i);
     again = true;
   }
   const int e0 = lo + s.owner_piece * kPiece, len = min(kPiece, hi - e0);
+  const float *terms = piece_buf(s, s.owner_piece % nbuf);
   if (warp != s.owner_warp) return;
   // The lane block, then the entry.
   const ff2 left = s.tgt;
@@ -1133,7 +1182,7 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
 #pragma unroll 1
   for (int c = b0; c < b1 && !over; c += 32) {
     const int e = c + lane;
-    const float x = e < b1 ? s.piece.l[e] : 0.f;
+    const float x = e < b1 ? terms[e] : 0.f;
     const ff2 reach = ff_add(run, warp_scan_ff(ff2{x, 0.f}, lane));
     const unsigned xh = __ballot_sync(0xffffffffu, hit != 0u && x > 0.f && ff_gt(reach, left));
     const unsigned xp = __ballot_sync(0xffffffffu, x > 0.f);
@@ -1151,7 +1200,7 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
 // another's words (every CTA is resident: cooperative launches).
 __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const SeqTable &seqs, const RowTables &rows, int c,
                                            int nctas) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   if (warp == 0) {
     int ns = 0, ng = 0;
     for (int b0 = 0; b0 < p.B; b0 += 32) {
@@ -1168,7 +1217,8 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const Seq
       s.n_st = ns;
       s.n_gr = ng;
       s.abort = 0;
-      mbar_init(&s.bar, 1);
+      mbar_init(&s.bar[0], 1);
+      mbar_init(&s.bar[1], 1);
       fence_mbar_init();
     }
   } else if (c == 0) {

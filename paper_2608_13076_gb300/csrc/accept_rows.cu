@@ -24,14 +24,14 @@ spade_status launch_accept_rows(const Call &c, int sms, cudaStream_t stream) {
   static bool configured = false;
   if (!configured) {
     const cudaError_t e = cudaFuncSetAttribute(accept_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(kRowsBytesPlain));
+                                               static_cast<int>(kRowsBytesDouble));
     if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(accept_rows)");
     configured = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sms < kMaxNC ? sms : kMaxNC);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kRowsBytesPlain;  // no nucleus search on this path
+  cfg.dynamicSmemBytes = kRowsBytesDouble;  // two buffers for the draw's pieces
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

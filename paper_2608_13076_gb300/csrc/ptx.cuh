@@ -105,6 +105,10 @@ SPADE_DEVICE bool mbar_wait_unabortable(uint64_t *bar, uint32_t parity) {
 SPADE_DEVICE int uniform_warp() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0); }
 // The same value on every lane, in a uniform register (a warp's lanes agree on v).
 SPADE_DEVICE int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+template <class T>
+SPADE_DEVICE T *uniform(T *v) {
+  return reinterpret_cast<T *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(v), 0));
+}
 SPADE_DEVICE bool elect_one() {
   uint32_t r;
   asm volatile(

@@ -631,6 +631,7 @@ static spade_status verify_accept_impl(const void *hidden, const void *w_lm,
     c.num_pages = cm->num_pages;
   }
   if (L.two_launches) {
+    c.pool = kPieceBytes;  // (no nucleus search on this path)
     st = launch_lm_head_pairs(c, hidden, w_lm, H, s);
     return st != SPADE_OK ? st : launch_accept_rows(c, sms, s);
   }
