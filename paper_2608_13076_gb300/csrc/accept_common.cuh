@@ -554,22 +554,8 @@ constexpr size_t kRowsBytesDouble = offsetof(RowsSmem, pool) + kPieceBytes;
 static_assert(offsetof(RowsSmem, piece) % 16 == 0, "bulk copies need 16-byte alignment");
 constexpr int kPoolPerRow = kNucBins * 4 + 32 * 2;  // bins and list lengths of one searched row
 
-// Bounded poll of an exchanged word until its writer has set it.  After an
+// Bounded poll of an exchanged mass until its writer has set it.  After an
 // expired wait of the CTA every later poll gives up at once.
-__device__ __forceinline__ unsigned poll_word(const Call &p, RowsSmem &s, const unsigned *a) {
-  unsigned v = ld_relaxed(a);
-  if (v != kUnset) return v;
-  const uint64_t t0 = globaltimer();
-  while ((v = ld_relaxed(a)) == kUnset) {
-    if (*const_cast<volatile int *>(&s.abort)) return 0u;
-    if (globaltimer() - t0 > kWaitLimitNs) {
-      *const_cast<volatile int *>(&s.abort) = 1;
-      atomicOr(p.status, SPADE_DEV_TIMEOUT);
-      return 0u;
-    }
-  }
-  return v;
-}
 __device__ __forceinline__ ff2 poll_mass(const Call &p, RowsSmem &s, const unsigned long long *a) {
   unsigned long long v = ld_relaxed64(a);
   if (v == kUnset64) {
@@ -900,19 +886,26 @@ __device__ __forceinline__ void nucleus(const Call &p, RowsSmem &s, int b, const
         unsigned v[kMaxGroup];  // every CTA's bins in flight at once
 #pragma unroll
         for (int c = 0; c < kMaxGroup; ++c) v[c] = c < gs && c != rank ? ld_relaxed(src + c * stride) : 0u;
+        // The late ones again, all in flight at once (one after the other, a round
+        // spent 5 us here with 19 CTAs).
+        uint64_t t0 = 0;
 #pragma unroll 1
-        for (int again = 1; again;) {  // late ones (all lanes of a warp retry together)
-          again = 0;
+        for (;;) {
+          bool late = false;
 #pragma unroll
-          for (int c = 0; c < kMaxGroup; ++c) again |= v[c] == kUnset;
-          if (again) {
-#pragma unroll 1
-            for (int c = 0; c < gs; ++c)
-              if (c != rank) poll_word(p, s, src + c * stride);
-#pragma unroll
-            for (int c = 0; c < kMaxGroup; ++c) v[c] = c < gs && c != rank ? ld_relaxed(src + c * stride) : 0u;
-            if (*const_cast<volatile int *>(&s.abort)) break;
+          for (int c = 0; c < kMaxGroup; ++c) late |= v[c] == kUnset;
+          if (!__any_sync(0xffffffffu, late)) break;
+          const uint64_t now = globaltimer();
+          if (t0 == 0) t0 = now;
+          const bool expired = now - t0 > kWaitLimitNs;
+          if (__any_sync(0xffffffffu, expired || *const_cast<volatile int *>(&s.abort))) {
+            *const_cast<volatile int *>(&s.abort) = 1;
+            atomicOr(p.status, SPADE_DEV_TIMEOUT);
+            break;
           }
+#pragma unroll
+          for (int c = 0; c < kMaxGroup; ++c)
+            if (v[c] == kUnset) v[c] = ld_relaxed(src + c * stride);
         }
         __syncwarp();
 #pragma unroll
