@@ -289,6 +289,9 @@ __device__ __forceinline__ SeqInfo seq_info(const Call &p, int b) {
 struct SeqTable {
   int r0[kMaxB], k[kMaxB];
   unsigned valid[kMaxB / 32], stoch[kMaxB / 32];
+  int st[kMaxB];  // sampled sequences, ascending
+  int gr[kMaxB];  // greedy and invalid ones
+  int n_st, n_gr;
 };
 __device__ __forceinline__ SeqInfo table_info(const SeqTable &t, int b) {
   const unsigned bit = 1u << (b % 32);
@@ -303,13 +306,40 @@ __device__ __forceinline__ void fill_table(const Call &p, SeqTable &t, int w, in
       q = seq_info(p, b);
       t.r0[b] = q.r0;
       t.k[b] = q.k;
-      if (!q.valid && report) atomicOr(p.status, SPADE_DEV_BAD_INDEX);
+      if (report) {
+        const int md = p.mode[b];
+        bool bad = !q.valid || (md != 0 && md != 1) || (md == 1 && p.draft_probs == nullptr && p.n_draft[b] > 0);
+        if (p.top_p != nullptr) {
+          const float tp = __ldg(p.top_p + b);
+          bad |= !(tp > 0.f && tp <= 1.f);
+        }
+        if (bad) atomicOr(p.status, SPADE_DEV_BAD_INDEX);
+      }
     }
     const unsigned mv = __ballot_sync(0xffffffffu, q.valid), ms = __ballot_sync(0xffffffffu, q.stoch);
     if (lane == 0) {
       t.valid[b0 / 32] = mv;
       t.stoch[b0 / 32] = ms;
     }
+  }
+}
+
+// The lists of sampled and of other sequences, by one warp, once the table is full.
+__device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int lane) {
+  int ns = 0, ng = 0;
+  for (int b0 = 0; b0 < p.B; b0 += 32) {
+    const int b = b0 + lane;
+    const unsigned in = p.B - b0 >= 32 ? 0xffffffffu : (1u << (p.B - b0)) - 1u;
+    const unsigned ms = t.stoch[b0 / 32] & in, mg = ~t.stoch[b0 / 32] & in;
+    const unsigned bit = 1u << lane, below = bit - 1u;
+    if (ms & bit) t.st[ns + __popc(ms & below)] = b;
+    if (mg & bit) t.gr[ng + __popc(mg & below)] = b;
+    ns += __popc(ms);
+    ng += __popc(mg);
+  }
+  if (lane == 0) {
+    t.n_st = ns;
+    t.n_gr = ng;
   }
 }
 
@@ -348,6 +378,7 @@ __device__ __forceinline__ void setup_rows(const Call &p, int nrows, SeqTable &s
     if (!q.valid) continue;
     for (int i = et % 32; i <= q.k; i += 32) t.draft[q.r0 + i] = b;
   }
+  if (et / 32 == kN / 32 - 1) fill_lists(p, seqs, et % 32);  // (for the one-launch form's rows phase)
   named_bar(1, kN);
   for (int n = et; n < p.R; n += kN) {
     const int b = t.draft[n];
@@ -527,11 +558,9 @@ constexpr int kPiece = 8192;       // entries of a share that the draw takes at 
 constexpr int kMaxPieces = 80;     // 622592 entries, the largest vocabulary
 struct RowsSmem {
   uint64_t bar[2];       // bulk copies of a piece, by buffer
-  int n_st, n_gr, first, nl, owner_piece, owner_warp, retry, abort;
+  int first, nl, owner_piece, owner_warp, retry, abort;
   ff2 tgt, before;
   ff2 pm[kMaxPieces][kWarps];  // masses of the warps' parts of each piece of this CTA's share
-  int st[kMaxB];         // sampled sequences, ascending
-  int gr[kMaxB];         // greedy and invalid ones
   float m[kMaxR], z[kMaxR];           // rows of the sequence at hand: maximum, sum of exponentials
   float u[kMaxR], q[kMaxR], l[kMaxR]; // uniform, q(draft), draft logit
   int arg[kMaxR], d[kMaxR], ok[kMaxR];
@@ -1194,39 +1223,14 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
 __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const SeqTable &seqs, const RowTables &rows, int c,
                                            int nctas) {
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
-  if (warp == 0) {
-    int ns = 0, ng = 0;
-    for (int b0 = 0; b0 < p.B; b0 += 32) {
-      const int b = b0 + lane;
-      const unsigned in = p.B - b0 >= 32 ? 0xffffffffu : (1u << (p.B - b0)) - 1u;
-      const unsigned ms = seqs.stoch[b0 / 32] & in, mg = ~seqs.stoch[b0 / 32] & in;
-      const unsigned bit = 1u << lane, below = bit - 1u;
-      if (ms & bit) s.st[ns + __popc(ms & below)] = b;
-      if (mg & bit) s.gr[ng + __popc(mg & below)] = b;
-      ns += __popc(ms);
-      ng += __popc(mg);
-    }
-    if (lane == 0) {
-      s.n_st = ns;
-      s.n_gr = ng;
-      s.abort = 0;
-      mbar_init(&s.bar[0], 1);
-      mbar_init(&s.bar[1], 1);
-      fence_mbar_init();
-    }
-  } else if (c == 0) {
-    for (int b = tid - 32; b < p.B; b += kThreads - 32) {
-      const int md = p.mode[b];
-      bool bad = (md != 0 && md != 1) || (md == 1 && p.draft_probs == nullptr && p.n_draft[b] > 0);
-      if (p.top_p != nullptr) {
-        const float tp = __ldg(p.top_p + b);
-        bad |= !(tp > 0.f && tp <= 1.f);
-      }
-      if (bad) atomicOr(p.status, SPADE_DEV_BAD_INDEX);
-    }
+  // (every sequence's decisions meet at barriers before the first copy or poll)
+  if (tid == 0) {
+    s.abort = 0;
+    mbar_init(&s.bar[0], 1);
+    mbar_init(&s.bar[1], 1);
+    fence_mbar_init();
   }
-  block_sync();
-  const int ns = s.n_st, ng = s.n_gr;
+  const int ns = seqs.n_st, ng = seqs.n_gr;
   const int ngroups = min(ns, nctas);
   const int gs = ns == 0 ? 1 : max(1, min(min(nctas / ngroups, kMaxGroup), (p.V + kMinShare - 1) / kMinShare));
   if (c < ngroups * gs) {
@@ -1236,7 +1240,7 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const Seq
     uint32_t parity = 0;
 #pragma unroll 1
     for (int i = g; i < ns; i += ngroups) {
-      const int b = s.st[i];
+      const int b = seqs.st[i];
       const SeqInfo q = table_info(seqs, b);
       decide_rows(p, s, rows, b, q, rank == 0, warp, lane);
       const float top = seq_top_p(p, b);
@@ -1253,7 +1257,7 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const Seq
   }
 #pragma unroll 1
   for (int i = nctas - 1 - c; i < ng; i += nctas) {
-    const int b = s.gr[i];
+    const int b = seqs.gr[i];
     const SeqInfo q = table_info(seqs, b);
     if (!q.valid) {
       if (tid == 0) {
