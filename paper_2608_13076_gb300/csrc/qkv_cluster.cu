@@ -31,7 +31,7 @@
 //    that the peer finishes travel there by one bulk copy (scalar remote stores
 //    took 4.6 us), and each CTA sums, rotates and stores its half of the rows.
 //    With many rows the staging takes the ring's place once both CTAs' MMAs are
-//    done, 128 verify rows at a time.
+//    done, as many verify rows at a time as fit.
 #include "qkv_common.cuh"
 
 namespace spade {
@@ -44,7 +44,7 @@ constexpr int kMaxRows = 512;                  // verify rows
 constexpr int kMaxStages = 12;
 constexpr int kMinStages = 4;                  // staging beside the ring
 constexpr int kMinStagesOver = 3;              // staging in the ring's place
-constexpr int kBatch = 128;                    // verify rows staged at once in the ring's place
+constexpr int kBatch = 128;                    // verify rows that the ring's place must take at once
 constexpr int kMaxPiece = 16;                  // quads of a piece (a head of dimension 128)
 constexpr int kMaxQuads = 64;                  // quads of a cluster's range (512 rows)
 constexpr int kSmemBudget = 222 * 1024;
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const Layout L = layout(p.Ncols, p.qmax, p.stages, p.over, p.batch);
-  int32_t *s_rseq = reinterpret_cast<int32_t *>(smem + L.rseq);
+  uint32_t *s_row = reinterpret_cast<uint32_t *>(smem + L.rseq);
   int32_t *s_rpos = reinterpret_cast<int32_t *>(smem + L.rpos);
   float *s_freq = reinterpret_cast<float *>(smem + L.freq);
   uint16_t *s_qrow = reinterpret_cast<uint16_t *>(smem + L.qrow);
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ===================== epilogue warps: wait for the accumulators =======
-    build_rows(p.c, s_rseq, s_rpos, tid - 64, kEpiThreads, [] { epi_bar(); });
+    build_rows(p.c, s_row, s_rpos, tid - 64, kEpiThreads, [] { epi_bar(); });
     if (nk > 0) {
       if (!mbar_wait(acc_full, 0, s_abort)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
       tc_fence_after();
@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const OutMap om = out_map(p.c);
   float *part = reinterpret_cast<float *>(smem + L.part);
   const float *recv = reinterpret_cast<const float *>(smem + L.recv);
+  const int dn = kThreads / nq, dq = kThreads - dn * nq, qsh = p.c.D == 128 ? 4 : 3;
   uint32_t phase = 0;
   for (int b0 = 0; b0 < p.c.R; b0 += p.batch, phase ^= 1u) {
     const int nb = kBig ? min(p.batch, p.c.R - b0) : p.c.R, n_own = own_rows(nb), n_send = nb - n_own;
@@ -297,21 +298,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
     __syncthreads();
     if (!mbar_wait_unabortable(recv_full, phase)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
-    for (int it = tid; it < n_own * nq; it += kThreads) {
-      const int n = it / nq, q = it - n * nq;
+    // Items (verify row, quad), kThreads apart.
+    for (int n = tid / nq, q = tid - n * nq; n < n_own;) {
       const int r = b0 + first + n;
-      const int b = s_rseq[r];
-      if (b < 0) continue;
-      const float *o = part + (first + n) * L.row_stride, *i = recv + n * L.row_stride;
-      const int r1 = s_qrow[2 * q], r2 = s_qrow[2 * q + 1];
-      float y1[4], y2[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        y1[e] = o[r1 + e] + i[r1 + e];
-        y2[e] = o[r2 + e] + i[r2 + e];
+      const uint32_t row = s_row[r];
+      if (row != kNoRow) {
+        const float *o = part + (first + n) * L.row_stride, *i = recv + n * L.row_stride;
+        const int r1 = s_qrow[2 * q], r2 = s_qrow[2 * q + 1];
+        const float4 o1 = *reinterpret_cast<const float4 *>(o + r1), o2 = *reinterpret_cast<const float4 *>(o + r2);
+        const float4 i1 = *reinterpret_cast<const float4 *>(i + r1), i2 = *reinterpret_cast<const float4 *>(i + r2);
+        float y1[4] = {o1.x + i1.x, o1.y + i1.y, o1.z + i1.z, o1.w + i1.w};
+        float y2[4] = {o2.x + i2.x, o2.y + i2.y, o2.z + i2.z, o2.w + i2.w};
+        const int Q = q0 + q, hg = Q >> qsh;
+        store_quad(om, s_freq, row, r, s_rpos[r], hg, (Q - (hg << qsh)) * 4, y1, y2);
       }
-      const int Q = q0 + q, hg = Q / qph;
-      store_quad(om, s_freq, b, r, s_rpos[r], hg, (Q - hg * qph) * 4, y1, y2);
+      n += dn;
+      q += dq;
+      if (q >= nq) { q -= nq; ++n; }
     }
     if (kBig && b0 + p.batch < p.c.R) {
       if (tid == 0)
@@ -373,7 +376,11 @@ static Params plan(const Call &c, int sms) {
   if (p.qmax >= 8 && n >= kMinStagesOver && L.recv + kBatch / 2 * L.row_stride * 4 <= L.ring + n * L.stage_bytes) {
     p.stages = n;
     p.over = 1;
-    p.batch = kBatch;
+    // As few batches as fit, of nearly equal sizes (multiples of 16): each costs
+    // its barriers and an exchange (389 rows in two of 208 at most instead of
+    // four of 128: 40.7 -> 34.5 us with the row table's cache rows).
+    const int fit = n * L.stage_bytes / (L.row_stride * 6) / 16 * 16, nb = (c.R + fit - 1) / fit;
+    p.batch = ((c.R + nb - 1) / nb + 15) / 16 * 16;
   }
   return p;
 }

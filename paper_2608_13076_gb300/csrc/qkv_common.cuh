@@ -44,12 +44,15 @@ __device__ __forceinline__ void rope_angle(int pos, float f, float *sn, float *c
   __sincosf(r + e, sn, cs);
 }
 
-// Row table (thread et of nt, `bar` a barrier among them): sequence and position
-// of every verify row; rows of invalid sequences are marked -1, and CTA 0
-// reports them.
+// Row table (thread et of nt, `bar` a barrier among them): position of every
+// verify row and its row in the caches, at KV head 0 (32 bits: 2^32 rows of the
+// smallest head are 550 GB); rows of invalid sequences are marked kNoRow, and
+// CTA 0 reports them.  (Looked up as the rows are stored, pages and divisions
+// made up a third of the epilogue at 389 paged rows.)
+constexpr uint32_t kNoRow = 0xffffffffu;
 template <class Bar>
-__device__ __forceinline__ void build_rows(const Call &p, int32_t *s_rseq, int32_t *s_rpos, int et, int nt, Bar bar) {
-  for (int r = et; r < p.R; r += nt) s_rseq[r] = -1;
+__device__ __forceinline__ void build_rows(const Call &p, uint32_t *s_row, int32_t *s_rpos, int et, int nt, Bar bar) {
+  for (int r = et; r < p.R; r += nt) s_row[r] = kNoRow;
   bar();
   for (int b = et; b < p.B; b += nt) {
     const int c = p.ctx_lens[b], k = p.n_draft[b];
@@ -69,8 +72,14 @@ __device__ __forceinline__ void build_rows(const Call &p, int32_t *s_rseq, int32
       continue;
     }
     for (int i = 0; i <= k; ++i) {
-      s_rseq[q0 + i] = b;
-      s_rpos[q0 + i] = c + i;
+      const int pos = c + i;
+      if (p.block_table) {
+        const uint32_t pg = p.block_table[static_cast<int64_t>(b) * p.max_pages + pos / p.page_size];
+        s_row[q0 + i] = pg * p.Hkv * p.page_size + pos % p.page_size;
+      } else {
+        s_row[q0 + i] = static_cast<uint32_t>(b) * p.Hkv * p.cap + pos;
+      }
+      s_rpos[q0 + i] = pos;
     }
   }
   bar();
@@ -80,19 +89,19 @@ __device__ __forceinline__ void build_rows(const Call &p, int32_t *s_rseq, int32
 // inlined the compiler would reload the parameters after every store).
 struct OutMap {
   __nv_bfloat16 *q_out, *k_cache, *v_cache;
-  const int32_t *block_table;
-  int Hq, Hkv, D, cap, page_size, max_pages;
+  int Hq, Hkv, D;
+  int head_rows;  // cache rows from one KV head to the next
 };
 __device__ __forceinline__ OutMap out_map(const Call &c) {
-  return OutMap{c.q_out, c.k_cache, c.v_cache, c.block_table, c.Hq, c.Hkv, c.D, c.cap, c.page_size, c.max_pages};
+  return OutMap{c.q_out, c.k_cache, c.v_cache, c.Hq, c.Hkv, c.D, c.block_table ? c.page_size : c.cap};
 }
 
 // Four consecutive rotary pairs (j0 .. j0 + 3 with j0 + D/2 ..; y1, y2) of head hg
 // (among the Hq + 2 Hkv of the projection) of verify row r: rotation of query and
-// key pairs and the bf16 stores, to q_out or the cache slot of the row's
-// sequence b at position pos.  4 bf16 = 8 bytes at each half (j0 a multiple of
+// key pairs and the bf16 stores, to q_out or the row's cache row (see
+// build_rows).  4 bf16 = 8 bytes at each half (j0 a multiple of
 // 4, rows 16-byte aligned).
-__device__ __forceinline__ void store_quad(const OutMap &p, const float *s_freq, int b, int r, int pos, int hg, int j0,
+__device__ __forceinline__ void store_quad(const OutMap &p, const float *s_freq, uint32_t row, int r, int pos, int hg, int j0,
                                            float (&y1)[4], float (&y2)[4]) {
   const int half = p.D / 2;
   if (hg < p.Hq + p.Hkv) {
@@ -111,12 +120,7 @@ __device__ __forceinline__ void store_quad(const OutMap &p, const float *s_freq,
   } else {
     const int hk = hg < p.Hq + p.Hkv ? hg - p.Hq : hg - p.Hq - p.Hkv;
     __nv_bfloat16 *cache = hg < p.Hq + p.Hkv ? p.k_cache : p.v_cache;
-    if (p.block_table) {
-      const int pg = p.block_table[static_cast<int64_t>(b) * p.max_pages + pos / p.page_size];
-      dst = cache + ((static_cast<size_t>(pg) * p.Hkv + hk) * p.page_size + pos % p.page_size) * p.D;
-    } else {
-      dst = cache + ((static_cast<size_t>(b) * p.Hkv + hk) * p.cap + pos) * p.D;
-    }
+    dst = cache + (static_cast<size_t>(row) + static_cast<uint32_t>(hk) * p.head_rows) * p.D;
   }
   *reinterpret_cast<uint2 *>(dst + j0) = make_uint2(pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]));
   *reinterpret_cast<uint2 *>(dst + j0 + half) = make_uint2(pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]));

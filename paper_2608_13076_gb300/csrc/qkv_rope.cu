@@ -122,7 +122,7 @@ __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"
 // the loads of every item and kPB parts before using any (the reduction is
 // bound by L2 latency, so the rounds of loads are what it costs).
 template <int kIB, int kPB>
-__device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq, const int32_t *s_rpos,
+__device__ __noinline__ void reduce_tile(const Params &p, const uint32_t *s_row, const int32_t *s_rpos,
                                          const float *s_freq, int t, int c_first, int nparts, int r0,
                                          int r1, int th, int nth) {
   const OutMap om = out_map(p.c);
@@ -137,7 +137,8 @@ __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq,
   const size_t slot = static_cast<size_t>(Ncols) * kTileM;
   const int nitems = (r1 - r0) * kQuads;
   for (int it0 = th; it0 < nitems; it0 += nth * kIB) {
-    int rr[kIB], d1[kIB], hl[kIB], jj[kIB], bb[kIB];
+    int rr[kIB], d1[kIB], hl[kIB], jj[kIB];
+    uint32_t bb[kIB];
     float y1[kIB][4], y2[kIB][4];
 #pragma unroll
     for (int i = 0; i < kIB; ++i) {
@@ -147,7 +148,7 @@ __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq,
       hl[i] = pp / half;
       jj[i] = pp % half;
       d1[i] = hl[i] * D + jj[i];
-      bb[i] = it < nitems ? s_rseq[rr[i]] : -1;
+      bb[i] = it < nitems ? s_row[rr[i]] : kNoRow;
 #pragma unroll
       for (int e = 0; e < 4; ++e) y1[i][e] = y2[i][e] = 0.f;
     }
@@ -157,7 +158,7 @@ __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq,
       for (int i = 0; i < kIB; ++i)
 #pragma unroll
         for (int s = 0; s < kPB; ++s)
-          if (bb[i] >= 0 && s0 + s < nparts) {
+          if (bb[i] != kNoRow && s0 + s < nparts) {
             const float *ps = base + (s0 + s) * slot + rr[i] * kTileM + d1[i];
             a[i][s] = __ldcg(reinterpret_cast<const float4 *>(ps));
             c[i][s] = __ldcg(reinterpret_cast<const float4 *>(ps + half));
@@ -166,17 +167,16 @@ __device__ __noinline__ void reduce_tile(const Params &p, const int32_t *s_rseq,
       for (int i = 0; i < kIB; ++i)
 #pragma unroll
         for (int s = 0; s < kPB; ++s)
-          if (bb[i] >= 0 && s0 + s < nparts) {
+          if (bb[i] != kNoRow && s0 + s < nparts) {
             y1[i][0] += a[i][s].x; y1[i][1] += a[i][s].y; y1[i][2] += a[i][s].z; y1[i][3] += a[i][s].w;
             y2[i][0] += c[i][s].x; y2[i][1] += c[i][s].y; y2[i][2] += c[i][s].z; y2[i][3] += c[i][s].w;
           }
     }
 #pragma unroll
     for (int i = 0; i < kIB; ++i) {
-      const int b = bb[i];
-      if (b < 0) continue;
+      if (bb[i] == kNoRow) continue;
       // (head among the Hq + 2 Hkv of the projection)
-      store_quad(om, s_freq, b, rr[i], s_rpos[rr[i]], t * hpt + hl[i], jj[i], y1[i], y2[i]);
+      store_quad(om, s_freq, bb[i], rr[i], s_rpos[rr[i]], t * hpt + hl[i], jj[i], y1[i], y2[i]);
     }
   }
 }
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const Layout L = layout(p.Ncols, p.stages, p.KG);
-  int32_t *s_rseq = reinterpret_cast<int32_t *>(smem + L.rseq);
+  uint32_t *s_row = reinterpret_cast<uint32_t *>(smem + L.rseq);
   int32_t *s_rpos = reinterpret_cast<int32_t *>(smem + L.rpos);
   uint64_t *bar_full = reinterpret_cast<uint64_t *>(smem + L.bars);
   uint64_t *bar_empty = bar_full + kMaxStages;
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Row table: sequence and position of every verify row.  Only the tile
     // reductions read it, so it is built here while the producer and the MMA
     // warp already stream the first units.
-    build_rows(p.c, s_rseq, s_rpos, et, kEpiThreads, [] { __syncwarp(); epi_bar(); });
+    build_rows(p.c, s_row, s_rpos, et, kEpiThreads, [] { __syncwarp(); epi_bar(); });
     bool expired = false;
     int seg = 0;
     for (int u = u0; u < u1; ++seg) {
@@ -381,9 +381,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (et == 0) { s_fin[0] = t; s_fin[1] = c_first; s_fin[2] = nparts; }
           } else {
             if (nparts == 1)
-              reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, et, kEpiThreads);
+              reduce_tile<6, 1>(p, s_row, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, et, kEpiThreads);
             else
-              reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, et, kEpiThreads);
+              reduce_tile<3, 3>(p, s_row, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, et, kEpiThreads);
             if (et == 0 && nparts > 1) p.counters[t] = 0;  // every part has arrived: reset for the next call
           }
         }
@@ -398,9 +398,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (s_fin[0] >= 0) {
     const int t = s_fin[0], c_first = s_fin[1], nparts = s_fin[2];
     if (nparts == 1)
-      reduce_tile<6, 1>(p, s_rseq, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, tid, kThreads);
+      reduce_tile<6, 1>(p, s_row, s_rpos, s_freq, t, c_first, 1, 0, p.c.R, tid, kThreads);
     else
-      reduce_tile<3, 3>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, tid, kThreads);
+      reduce_tile<3, 3>(p, s_row, s_rpos, s_freq, t, c_first, nparts, 0, p.c.R, tid, kThreads);
     if (tid == 0 && nparts > 1) p.counters[t] = 0;  // every part has arrived: reset for the next call
   }
   // Row slabs of the split tiles (slabs > 1): item i = t * slabs + s goes to
@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok) {
       const int r0 = static_cast<int>(static_cast<int64_t>(p.c.R) * sl / p.slabs);
       const int r1 = static_cast<int>(static_cast<int64_t>(p.c.R) * (sl + 1) / p.slabs);
-      reduce_tile<2, 6>(p, s_rseq, s_rpos, s_freq, t, c_first, nparts, r0, r1, tid, kThreads);
+      reduce_tile<2, 6>(p, s_row, s_rpos, s_freq, t, c_first, nparts, r0, r1, tid, kThreads);
     }
     __syncthreads();  // every load of the parts is done
     if (tid == 0 && ok && add_acq_rel(&slabs_done[t], 1) == p.slabs - 1) {
