@@ -8,6 +8,7 @@
 
 #include <cfloat>
 #include <cstdint>
+#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -223,86 +224,101 @@ __device__ __forceinline__ size_t out_row(const Params &p, int q_row0, int kvh, 
 }
 
 // Log-sum-exp merge of the nparts partials (slots slot0 ..) of one unit into
-// the bf16 output and the lse, run by warps cw = 0..nw-1 of the CTA that
-// finished the unit last.  Online merge over batches of kBatch partials; each
-// warp step takes RPW rows, so RPW * kBatch partial rows per lane are in
-// flight together.
-template <int D, int RPW = 2>
-__device__ void merge_partials(const Params &p, int64_t slot0, int nparts, int nrow, int rb,
-                               int kvh, int q_row0, int cw, int nw, int lane) {
+// the bf16 output and the lse, by the kMergeWarps softmax warps of the CTA that
+// finished the unit last (thread stid, warp cw; named barrier 1 among them).
+// Warp cw takes rows cw, cw + kMergeWarps, ...; the values of the first kBatch parts
+// are loaded, then thread r reduces row r's maxima and sums over all parts: every
+// load of up to kBatch parts is in flight at once, and the row arithmetic (weights'
+// maximum, 1 / L, lse, the output row's division) is done once per row, not by every
+// lane (Llama-3-8B step: 31.0 -> 29.8 us, 389 ragged paged rows: 174.8 -> 171.8).
+// `s_row`: three floats per row of shared memory.
+constexpr int kMergeWarps = 8;
+template <int D>
+__device__ __forceinline__ void merge_partials(const Params &p, int64_t slot0, int nparts, int nrow, int rb, int kvh,
+                                               int q_row0, float *s_row, int stid, int cw, int lane) {
   constexpr int PER = D / 32;
-  constexpr int kBatch = 4;
-  for (int rl0 = RPW * cw; rl0 < nrow; rl0 += RPW * nw) {
-    float M[RPW], Lsum[RPW], acc[RPW][PER];
+  constexpr int kBatch = 4, kRows = 5;
+  using Vec = typename std::conditional<PER == 4, float4, float2>::type;
+  const float *base = p.partials + slot0 * slot_floats(D);
+  float *s_m = s_row, *s_inv = s_row + kRowBlock;
+  uint32_t *s_out = reinterpret_cast<uint32_t *>(s_row + 2 * kRowBlock);  // output rows, fewer than 2^32
+  bool stats = false;
+#pragma unroll 1
+  for (int r0 = cw; r0 < nrow || !stats; r0 += kMergeWarps * kRows) {
+    float acc[kRows][PER];
 #pragma unroll
-    for (int h = 0; h < RPW; ++h) {
-      M[h] = -INFINITY;
-      Lsum[h] = 0.f;
+    for (int h = 0; h < kRows; ++h)
 #pragma unroll
       for (int e = 0; e < PER; ++e) acc[h][e] = 0.f;
-    }
+#pragma unroll 1
     for (int s0 = 0; s0 < nparts; s0 += kBatch) {
-      float mv[RPW][kBatch], lv[RPW][kBatch], ov[RPW][kBatch][PER];
+      Vec ov[kRows][kBatch];
+      float mv[kRows][kBatch];
 #pragma unroll
-      for (int h = 0; h < RPW; ++h) {
-        const int rl = min(rl0 + h, nrow - 1);
+      for (int h = 0; h < kRows; ++h) {
+        const int rl = r0 + kMergeWarps * h;
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-          if (s0 + j < nparts) {
-            const float *ps = p.partials + (slot0 + s0 + j) * slot_floats(D);
-            mv[h][j] = __ldcg(ps + kRowBlock * D + rl);
-            lv[h][j] = __ldcg(ps + kRowBlock * D + kRowBlock + rl);
-            if constexpr (PER == 4) {
-              const float4 v = __ldcg(reinterpret_cast<const float4 *>(ps + rl * D + lane * 4));
-              ov[h][j][0] = v.x; ov[h][j][1] = v.y; ov[h][j][2] = v.z; ov[h][j][3] = v.w;
-            } else {
-              const float2 v = __ldcg(reinterpret_cast<const float2 *>(ps + rl * D + lane * 2));
-              ov[h][j][0] = v.x; ov[h][j][1] = v.y;
-            }
-          } else {
-            mv[h][j] = -INFINITY;
-            lv[h][j] = 0.f;
-#pragma unroll
-            for (int e = 0; e < PER; ++e) ov[h][j][e] = 0.f;
-          }
+          const bool in = rl < nrow && s0 + j < nparts;
+          const float *ps = base + static_cast<int64_t>(s0 + j) * slot_floats(D);
+          mv[h][j] = in ? __ldcg(ps + kRowBlock * D + rl) : -INFINITY;
+          if (in) ov[h][j] = __ldcg(reinterpret_cast<const Vec *>(ps + rl * D) + lane);
+          else ov[h][j] = Vec{};
         }
       }
+      if (!stats) {
+        if (stid < nrow) {
+          float M = -INFINITY, L = 0.f;
+#pragma unroll 1
+          for (int t0 = 0; t0 < nparts; t0 += kBatch) {
+            float m[kBatch], l[kBatch];
 #pragma unroll
-      for (int h = 0; h < RPW; ++h) {
-        float Mn = M[h];
+            for (int j = 0; j < kBatch; ++j) {
+              const float *ps = base + static_cast<int64_t>(t0 + j) * slot_floats(D) + kRowBlock * D + stid;
+              m[j] = t0 + j < nparts ? __ldcg(ps) : -INFINITY;
+              l[j] = t0 + j < nparts ? __ldcg(ps + kRowBlock) : 0.f;
+            }
+            float Mn = M;
 #pragma unroll
-        for (int j = 0; j < kBatch; ++j) Mn = fmaxf(Mn, mv[h][j]);
-        const float U = (Mn == -INFINITY) ? 0.f : Mn;
-        const float f = ex2(M[h] - U);
-        Lsum[h] *= f;
+            for (int j = 0; j < kBatch; ++j) Mn = fmaxf(Mn, m[j]);
+            const float U = Mn == -INFINITY ? 0.f : Mn;
+            L *= ex2(M - U);
 #pragma unroll
-        for (int e = 0; e < PER; ++e) acc[h][e] *= f;
+            for (int j = 0; j < kBatch; ++j) L += ex2(m[j] - U) * l[j];
+            M = Mn;
+          }
+          s_m[stid] = M == -INFINITY ? 0.f : M;
+          s_inv[stid] = 1.f / L;
+          const size_t orow = out_row(p, q_row0, kvh, rb, stid);
+          s_out[stid] = static_cast<uint32_t>(orow);
+          if (p.lse) p.lse[orow] = (M + log2f(L)) * 0.69314718055994531f;
+        }
+        named_bar(1, 32 * kMergeWarps);
+        stats = true;
+      }
+#pragma unroll
+      for (int h = 0; h < kRows; ++h) {
+        const float M = s_m[min(r0 + kMergeWarps * h, kRowBlock - 1)];
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-          const float w = ex2(mv[h][j] - U);
-          Lsum[h] += w * lv[h][j];
+          const float w = ex2(mv[h][j] - M);
+          const float *o = reinterpret_cast<const float *>(&ov[h][j]);
 #pragma unroll
-          for (int e = 0; e < PER; ++e) acc[h][e] += w * ov[h][j][e];
+          for (int e = 0; e < PER; ++e) acc[h][e] = fmaf(w, o[e], acc[h][e]);
         }
-        M[h] = Mn;
       }
     }
 #pragma unroll
-    for (int h = 0; h < RPW; ++h) {
-      const int rl = rl0 + h;
+    for (int h = 0; h < kRows; ++h) {
+      const int rl = r0 + kMergeWarps * h;
       if (rl < nrow) {
-        const size_t orow = out_row(p, q_row0, kvh, rb, rl);
-        const float inv = 1.f / Lsum[h];
-        if constexpr (PER == 4) {
-          uint2 v;
-          v.x = pack_bf16(acc[h][0] * inv, acc[h][1] * inv);
-          v.y = pack_bf16(acc[h][2] * inv, acc[h][3] * inv);
-          *reinterpret_cast<uint2 *>(p.out + orow * D + lane * 4) = v;
-        } else {
-          *reinterpret_cast<uint32_t *>(p.out + orow * D + lane * 2) =
-              pack_bf16(acc[h][0] * inv, acc[h][1] * inv);
-        }
-        if (p.lse && lane == 0) p.lse[orow] = (M[h] + log2f(Lsum[h])) * 0.69314718055994531f;
+        const float inv = s_inv[rl];
+        __nv_bfloat16 *dst = p.out + static_cast<size_t>(s_out[rl]) * D + lane * PER;
+        if constexpr (PER == 4)
+          *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf16(acc[h][0] * inv, acc[h][1] * inv),
+                                                       pack_bf16(acc[h][2] * inv, acc[h][3] * inv));
+        else
+          *reinterpret_cast<uint32_t *>(dst) = pack_bf16(acc[h][0] * inv, acc[h][1] * inv);
       }
     }
   }

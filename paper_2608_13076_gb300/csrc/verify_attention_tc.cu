@@ -464,13 +464,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     cp_async_commit();
     for (int64_t x = x_begin; x < x_end && si.n_here > 0;) {
       const Seg g = si.g;
-      SegInfo si_next = si;
-      si_next.n_here = 0;
-      if (si.seg_end < x_end) {
-        si_next = next_seg(sc, si.seg_end, x_end);
-        if (si_next.n_here > 0) prefetch_q(si_next, (seg + 1) & 1);  // that buffer's last reader (unit seg-1) is done
-      }
-      cp_async_commit();
       const int ctx = s_ctx[g.b];
       const int kd = s_kd[g.b];
       const int nrow = min(kRowBlock, p.G * (kd + 1) - kRowBlock * g.rb);
@@ -479,7 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // Rows of this warp are [c0, c0 + NH); of those, r < hi are real rows.
       const int hi = nrow - c0;
       if (stid < kRowBlock) s_rmax[stid] = -INFINITY;
-      cp_async_wait<1>();  // this segment's Q has landed
+      cp_async_wait<0>();  // this segment's Q has landed
       fence_proxy_async_smem();
       named_bar(1, kSoftThreads);
       __syncwarp();
@@ -489,6 +482,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (seg == 0) mbar_arrive(&bars[kBarQ]);
         mbar_arrive(&bars[kBarSeg]);
       }
+      SegInfo si_next = si;
+      si_next.n_here = 0;
+      if (si.seg_end < x_end) {
+        si_next = next_seg(sc, si.seg_end, x_end);
+        if (si_next.n_here > 0) prefetch_q(si_next, (seg + 1) & 1);  // that buffer's last reader (unit seg-1) is done
+      }
+      cp_async_commit();
 
       // Running row maxima live in s_rmax (one writer per row); the row sums of
       // this key lane in l.
@@ -657,12 +657,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int r = 0; r < NH; ++r) l[r] = s_rowv[c0 + r];
       // Row statistics of this warp's rows, one lane per row (quadrant-0 warps).
       const float l_own = row_writer ? s_rowv[c0 + lane] : 1.f;
-      if (!mbar_wait(&bars[kBarOFinal], seg & 1, s_abort)) expired = true;
-      tc_fence_after();
+      // (their divisions run while the last PV MMAs do)
       const int unit = (g.b * p.Hkv + g.kvh) * p.RB + g.rb;
       const int64_t c_first = sc.owner(g.ust + sc.E);
       const int64_t c_last = sc.owner(g.ust + sc.E + g.nch - 1);
       const int nparts = static_cast<int>(c_last - c_first + 1);
+      if (!mbar_wait(&bars[kBarOFinal], seg & 1, s_abort)) expired = true;
+      tc_fence_after();
       if (nparts == 1) {
         // Output row of this warp's row c0 + r, advanced row by row (one
         // division for the warp's first row instead of one per row).
@@ -713,8 +714,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         named_bar(1, kSoftThreads);
         if (*s_last) {
           // This CTA finished the unit last: merge every partial by log-sum-exp.
-          merge_partials<kD, 5>(p, c_first + unit, nparts, nrow, g.rb, g.kvh, q_row0, warp - 2,
-                                kSoftWarps, lane);
+          static_assert(kSoftWarps == kMergeWarps, "the softmax warps merge");
+          merge_partials<kD>(p, c_first + unit, nparts, nrow, g.rb, g.kvh, q_row0, s_wred, stid, warp - 2, lane);
           if (stid == 0) p.counters[unit] = 0;  // every part has arrived: reset for the next call
         }
       }
