@@ -292,6 +292,9 @@ struct SeqTable {
   int st[kMaxB];  // sampled sequences, ascending
   int gr[kMaxB];  // greedy and invalid ones
   int n_st, n_gr;
+  // This CTA among the groups that draw: groups, CTAs in each, its group and rank,
+  // and its share [lo, hi) of the vocabulary.
+  int ngroups, gs, g, rank, lo, hi;
 };
 __device__ __forceinline__ SeqInfo table_info(const SeqTable &t, int b) {
   const unsigned bit = 1u << (b % 32);
@@ -324,8 +327,17 @@ __device__ __forceinline__ void fill_table(const Call &p, SeqTable &t, int w, in
   }
 }
 
-// The lists of sampled and of other sequences, by one warp, once the table is full.
-__device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int lane) {
+// This CTA's share [lo, hi) of the vocabulary in a group of gs, shares a
+// multiple of 4 entries (logits rows are read as float4).
+__device__ __forceinline__ void share_of(int V, int gs, int rank, int *lo, int *hi) {
+  const int per = ((V + gs - 1) / gs + 3) & ~3;
+  *lo = min(V, rank * per);
+  *hi = min(V, *lo + per);
+}
+
+// The lists of sampled and of other sequences and CTA c's place among nctas, by
+// one warp, once the table is full.
+__device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int c, int nctas, int lane) {
   int ns = 0, ng = 0;
   for (int b0 = 0; b0 < p.B; b0 += 32) {
     const int b = b0 + lane;
@@ -340,6 +352,11 @@ __device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int lane)
   if (lane == 0) {
     t.n_st = ns;
     t.n_gr = ng;
+    t.ngroups = min(ns, nctas);
+    t.gs = ns == 0 ? 1 : max(1, min(min(nctas / t.ngroups, kMaxGroup), (p.V + kMinShare - 1) / kMinShare));
+    t.g = c / t.gs;
+    t.rank = c - t.g * t.gs;
+    share_of(p.V, t.gs, t.rank, &t.lo, &t.hi);
   }
 }
 
@@ -378,7 +395,7 @@ __device__ __forceinline__ void setup_rows(const Call &p, int nrows, SeqTable &s
     if (!q.valid) continue;
     for (int i = et % 32; i <= q.k; i += 32) t.draft[q.r0 + i] = b;
   }
-  if (et / 32 == kN / 32 - 1) fill_lists(p, seqs, et % 32);  // (for the one-launch form's rows phase)
+  if (et / 32 == kN / 32 - 1) fill_lists(p, seqs, blockIdx.x, p.NC, et % 32);  // (for the one-launch form's rows phase)
   named_bar(1, kN);
   for (int n = et; n < p.R; n += kN) {
     const int b = t.draft[n];
@@ -735,14 +752,6 @@ __device__ __forceinline__ void commit_seq(const Call &p, int b, int k, int a, i
     p.vc[off] = zero;
   }
   if (tid == 0) p.ctx_lens[b] = lo;
-}
-
-// This CTA's share [lo, hi) of the vocabulary in a group of gs, shares a
-// multiple of 4 entries (logits rows are read as float4).
-__device__ __forceinline__ void share_of(int V, int gs, int rank, int *lo, int *hi) {
-  const int per = ((V + gs - 1) / gs + 3) & ~3;
-  *lo = min(V, rank * per);
-  *hi = min(V, *lo + per);
 }
 
 // Adds four values of a row to a lane's bins.  `v` holds scaled logits; a value
@@ -1118,17 +1127,18 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
     block_sync();
     copy(i + nbuf);
     if (++i < npiece) continue;
+    ff2 share{0.f, 0.f};
     unsigned long long *zp = p.zpart + (static_cast<size_t>(attempt) * p.B + b) * kMaxGroup;
     if (warp == 0) {
       // This share's mass: lane w sums the pieces of warp w's parts, in order.
       ff2 z{0.f, 0.f};
       for (int j = 0; j < npiece && lane < kWarps; ++j) z = ff_add(z, s.pm[j][lane]);
-      z = ff_shfl(warp_scan_ff(z, lane), 31);
-      if (lane == 0) post_mass(&zp[rank], z);
+      share = ff_shfl(warp_scan_ff(z, lane), 31);
+      if (lane == 0 && gs > 1) post_mass(&zp[rank], share);
     }
     if (attempt == 0 && commit && rank == 0) commit_seq(p, b, q.k, a, tid);
     if (warp == 0) {
-      const ff2 mine = lane < gs ? poll_mass(p, s, &zp[lane]) : ff2{0.f, 0.f};
+      const ff2 mine = gs == 1 && lane == 0 ? share : (gs > 1 && lane < gs ? poll_mass(p, s, &zp[lane]) : ff2{0.f, 0.f});
       __syncwarp();
       const ff2 reach = warp_scan_ff(mine, lane);
       const ff2 tot = ff_shfl(reach, 31);
@@ -1231,12 +1241,9 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const Seq
     fence_mbar_init();
   }
   const int ns = seqs.n_st, ng = seqs.n_gr;
-  const int ngroups = min(ns, nctas);
-  const int gs = ns == 0 ? 1 : max(1, min(min(nctas / ngroups, kMaxGroup), (p.V + kMinShare - 1) / kMinShare));
-  if (c < ngroups * gs) {
-    const int g = c / gs, rank = c - g * gs;
-    int lo, hi;
-    share_of(p.V, gs, rank, &lo, &hi);
+  const int ngroups = seqs.ngroups, gs = seqs.gs;
+  if (seqs.g < ngroups) {
+    const int g = seqs.g, rank = seqs.rank, lo = seqs.lo, hi = seqs.hi;
     uint32_t parity = 0;
 #pragma unroll 1
     for (int i = g; i < ns; i += ngroups) {

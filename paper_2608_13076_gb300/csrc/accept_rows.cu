@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(kThreads, 1) accept_rows_kernel(const __grid_c
   griddep_launch_dependents();
   fill_table(c, seqs, threadIdx.x / 32, kWarps, threadIdx.x % 32, false);  // (reported by the first launch)
   block_sync();
-  if (threadIdx.x < 32) fill_lists(c, seqs, threadIdx.x);
+  if (threadIdx.x < 32) fill_lists(c, seqs, blockIdx.x, gridDim.x, threadIdx.x);
   block_sync();
   rows_phase(c, *reinterpret_cast<RowsSmem *>(smem_rows), seqs, RowTables{}, blockIdx.x, gridDim.x);
 }
