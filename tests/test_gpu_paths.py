@@ -1,0 +1,146 @@
+"""Kernel variants and dispatch branches at the sizes where each can go wrong: edges of tiles, MMA
+widths, pieces and batches, the smallest and largest of a range.  Against the float64 oracle under
+the tolerances of ``tests.parity``; paged caches against the dense call, bit for bit.
+"""
+import pytest
+import torch
+
+import paper_2608_13076_gb300 as spade
+from paper_2608_13076_gb300 import workloads as W
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev(gpu_lib):
+    return torch.device("cuda:0")
+
+
+def _spec(name, seed, **over):
+    base = dict(B=1, Hq=4, Hkv=2, D=128, H=256, V=1000, ctx=(1, 90), k=(0, 0), mode="greedy", seed=seed)
+    return W.WorkloadSpec(name, **{**base, **over})
+
+
+# The projection.  At most 128 rows: a cluster of two CTAs per range of rotary pairs, each with half
+# of the k-chunks (H = 64: one of them has none).  More rows over wide layers (at least eight quads
+# of pairs per cluster): a second MMA chunk above 256 rows, the exchange in one to three batches.
+# More rows over narrow layers, or more than fit the ring: the form with partial sums in a workspace.
+QKV = {
+    "one_row_one_chunk": dict(H=64),
+    "n16": dict(B=2, k=(7, 7), H=72),
+    "n17_d64": dict(B=1, k=(16, 16), H=136, D=64, Hq=6),
+    "rows128": dict(B=16, k=(7, 7), H=520, Hq=32, Hkv=4),
+    "rows129_wide": dict(B=3, k=(42, 42), H=200, Hq=32, Hkv=4),
+    "rows256_wide": dict(B=32, k=(7, 7), H=128, Hq=32, Hkv=8),
+    "rows272_wide_d64": dict(B=34, k=(7, 7), H=192, D=64, Hq=60, Hkv=10),
+    "rows389_wide": dict(B=64, k=(1, 10), H=200, Hq=40, Hkv=8),
+    "rows512_wide": dict(B=64, k=(7, 7), H=128, Hq=32, Hkv=4),
+    "rows129_narrow": dict(B=3, k=(42, 42), H=200),
+}
+
+
+@pytest.mark.parametrize("name", sorted(QKV))
+def test_qkv_forms(dev, name):
+    spec = _spec(name, 300 + len(name), **QKV[name])
+    wl = W.make_workload(spec, device=dev, cache_pad=3)
+    x, w = W.make_qkv_inputs(spec, wl["R"], device=dev)
+    pg = W.to_paged(wl, 64, seed=5)
+    k0, v0 = wl["k_cache"].clone(), wl["v_cache"].clone()
+    q, st = parity.gpu_qkv_rope(wl, x, w)
+    qp, stp = torch.full_like(q, float("nan")), spade.status_tensor(dev)
+    ws = spade.qkv_workspace(wl["R"], wl["Hq"], wl["Hkv"], wl["D"], device=dev)
+    spade.spade_verify_qkv_rope_paged(x, w, pg["block_table"], wl["ctx_lens"], wl["n_draft"], wl["cu_q"], qp,
+                                      pg["k_pool"], pg["v_pool"], Hq=wl["Hq"], rope_theta=spec.rope_theta,
+                                      max_k=int(wl["n_draft"].max()), workspace=ws, status=stp)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and int(stp.item()) == 0
+    parity.check_qkv_rope(wl, x, w, q, k0, v0)
+    assert torch.equal(qp, q)
+    for b in range(wl["B"]):  # the verify slots, page by page
+        lo, n = int(wl["ctx_lens"][b]), int(wl["n_draft"][b]) + 1
+        for s in range(lo, lo + n):
+            page = int(pg["block_table"][b, s // 64])
+            assert torch.equal(pg["k_pool"][page, :, s % 64], wl["k_cache"][b, :, s])
+            assert torch.equal(pg["v_pool"][page, :, s % 64], wl["v_cache"][b, :, s])
+
+
+# The LM head.  Row counts around the statistics' blocks of 16, around the one-launch limit, and the
+# most rows of the two-launch form; slices that end inside a tile and inside a warp's 32 entries.
+ROWS = {"r1": (1, 0, 1), "r16": (2, 7, 1), "r17": (1, 16, 1), "r256": (32, 7, 1), "r257": (1, 256, 2),
+        "r400": (50, 7, 2), "r512": (64, 7, 2)}
+
+
+@pytest.mark.parametrize("mode", ["greedy", "stochastic"])
+@pytest.mark.parametrize("name", sorted(ROWS))
+def test_lm_head_row_counts(dev, name, mode):
+    B, k, launches = ROWS[name]
+    wl = W.make_workload(_spec(name, 320 + B, B=B, k=(k, k), V=9003, mode=mode, target_accept=0.7), device=dev)
+    B, R, H, V = wl["B"], wl["R"], wl["H"], wl["V"]
+    assert spade.spade_accept_launches(B, R, H, V) == launches
+    ws = spade.accept_workspace(B, R, H, V, device=dev)
+    acc, tok, st = parity.gpu_accept(wl, workspace=ws)
+    torch.cuda.synchronize()
+    assert int(st.item()) & ~spade.DEV_FALLBACK == 0
+    logits = parity.oracle_logits(wl)
+    assert parity.compare_accept(acc, tok, parity.oracle_accept_from_logits(wl, logits))["mismatch_unflagged"] == 0
+    worst = parity.compare_row_stats(spade.read_accept_stats(ws, B, R, H, V), logits, wl)
+    assert worst["argmax_mismatch"] == 0 and max(worst["max"], worst["lse"], worst["draft_logit"]) <= 1.0, worst
+
+
+# The draw.  Shares of one piece and of several (more than 8192 entries: two buffers, and the owner's
+# piece again), groups of one CTA and of more, q rows that bulk copies can and cannot read.
+DRAW = {
+    "one_cta_one_piece": dict(B=2, k=(4, 4), V=1024),
+    "one_cta_three_pieces": dict(B=80, k=(1, 1), V=20000),
+    "one_cta_unaligned": dict(B=80, k=(1, 1), V=20001),
+    "two_ctas_unaligned": dict(B=60, k=(2, 2), V=33002),
+    "two_launches_aligned": dict(B=60, k=(4, 4), V=40000),
+    "two_launches_unaligned": dict(B=60, k=(4, 4), V=40003),
+    "two_launches_one_cta": dict(B=130, k=(1, 2), V=20004),
+}
+
+
+@pytest.mark.parametrize("name", sorted(DRAW))
+def test_draw_shares(dev, name):
+    spec = _spec(name, 340 + len(name), H=128, mode="stochastic", target_accept=0.7, logit_scale=4.0, **DRAW[name])
+    wl = W.make_workload(spec, device=dev)
+    if name.startswith("two_launches"):
+        assert spade.spade_accept_launches(wl["B"], wl["R"], wl["H"], wl["V"]) == 2
+    acc, tok, st = parity.gpu_accept(wl)
+    torch.cuda.synchronize()
+    assert int(st.item()) & ~spade.DEV_FALLBACK == 0
+    cmp = parity.compare_accept(acc, tok, parity.oracle_accept(wl))
+    assert cmp["mismatch_unflagged"] == 0 and cmp["flagged"] < wl["B"] // 2, cmp
+
+
+# The nucleus search.  Flat logits put nearly every entry in one bin of the first round, so the kept
+# lists overflow and the values are read again; one CTA per group (nothing exchanged) and several.
+@pytest.mark.parametrize("B,V,scale", [(2, 160000, 0.05), (80, 20000, 0.05), (80, 3001, 4.0)])
+def test_top_p_lists(dev, B, V, scale):
+    k = 3 if B == 2 else 1
+    spec = _spec("topp_lists", 360 + B, B=B, k=(k, k), H=128, V=V, mode="stochastic", target_accept=0.6, logit_scale=scale)
+    wl = W.make_workload(spec, device=dev)
+    top_p = torch.linspace(0.4, 0.9, B)
+    acc, tok, st = parity.gpu_accept_sampling(wl, top_p=top_p.to(dev))
+    torch.cuda.synchronize()
+    assert int(st.item()) & ~spade.DEV_FALLBACK == 0
+    ref = parity.oracle_accept_from_logits(wl, parity.oracle_logits(wl), top_p=top_p.numpy())
+    assert parity.compare_accept(acc, tok, ref)["mismatch_unflagged"] == 0
+    # (a flat nucleus holds tens of thousands of tokens: the drawn one must lie in it)
+    assert int(tok.min()) >= 0 and int(tok.max()) < V
+
+
+# Attention units split into many parts: the merge's batches of four parts and its rows' remainders.
+@pytest.mark.parametrize("D,G,k,ctx", [(128, 1, 0, 20000), (64, 1, 0, 700), (128, 5, 6, 9000), (64, 8, 7, 20000),
+                                       (128, 8, 7, 600), (128, 3, 8, 330)])
+def test_attention_merge(dev, D, G, k, ctx):
+    wl = W.make_workload(_spec("merge", 380 + G, Hq=G, Hkv=1, D=D, ctx=(ctx, ctx), k=(k, k)), device=dev)
+    out, lse, st = parity.gpu_attention(wl)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    ref, ref_lse = parity.oracle_attention(wl)
+    n, bad, worst = parity.compare_attention(out, ref)
+    assert bad == 0, worst
+    # fp32 sums of at most 20008 exponentials, scores of bf16 products: far below 1e-3
+    assert abs(parity.to_np(lse) - ref_lse).max() < 1e-3
