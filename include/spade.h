@@ -106,11 +106,13 @@ typedef enum {
  *               zero the workspace again before the next one).  Calls that
  *               share a workspace must be ordered.
  * Every pointer is a 16-byte aligned device pointer.  The contraction is split
- * over every SM; the split parts' fp32 sums meet in the workspace and are
- * added in a fixed order, so results do not depend on timing.  The kernel
- * keeps every block of the grid resident at once (cooperative launch, with
- * programmatic dependent launch): the CTAs that finish a split tile wait,
- * bounded, for the other CTAs' partial sums.
+ * over every SM and its parts' fp32 sums are added in a fixed order, so results
+ * do not depend on timing.  Up to 128 rows, and up to 512 over wide layers, two
+ * CTAs of a cluster each take half of H and add their sums in shared memory:
+ * the workspace is not touched.  Other calls add the parts in the workspace;
+ * that kernel keeps every block of the grid resident at once (cooperative
+ * launch): the CTAs that finish a split tile wait, bounded, for the other CTAs'
+ * partial sums.  Both are launched with programmatic dependent launch.
  */
 spade_status spade_verify_qkv_rope(const void *x, const void *w_qkv, const int32_t *ctx_lens,
                                    const int32_t *n_draft, const int32_t *cu_q, void *q_out,
@@ -223,7 +225,9 @@ spade_status spade_verify_attention_noalloc(const void *q, const void *k_cache,
  *   accepted_len  int32 [B] written;  next_token int32 [B] written
  *   workspace     scratch of spade_accept_workspace_size(...) bytes, 256-byte
  *                 aligned, ZEROED ONCE by the caller; completed calls leave the
- *                 parts that must start at zero zeroed again.
+ *                 parts that must start at zero zeroed again.  It has room for
+ *                 the fp32 logits of every row (R V floats); those of rows of
+ *                 sampled sequences are stored there.
  *   status        device int32, SPADE_DEV_* bits OR-ed in
  * The kernel keeps every block of the grid resident at once (cooperative
  * launch) and meets at bounded device-wide barriers; if a barrier expires the
@@ -303,28 +307,27 @@ size_t spade_accept_workspace_size(int32_t B, int32_t R, int32_t H, int32_t V);
 
 /*
  * Kernel launches one spade_verify_accept (or spade_verify_accept_commit) call
- * makes for these sizes on the current device: 1 when the logits of all R
- * rows stay on chip, 2 when they do not (a statistics pass over all rows --
- * on pairs of SMs sharing each MMA when the grid is even -- then a pass that
- * recomputes only the rows to sample); 0 on invalid sizes.  For launch
- * accounting and graph capture; no device work.
+ * makes for these sizes on the current device: 1 (up to 256 rows, statistics
+ * and decisions in one kernel) or 2 (a statistics pass over all rows on pairs
+ * of SMs sharing each MMA, then the decisions and draws, from the logits that
+ * the first stored); 0 on invalid sizes.  For launch accounting and graph
+ * capture; no device work.
  */
 int32_t spade_accept_launches(int32_t B, int32_t R, int32_t H, int32_t V);
 
 /*
  * Where a completed spade_verify_accept (or spade_verify_accept_commit) call
  * leaves its merged per-row softmax statistics inside the workspace, for
- * tests and diagnostics that check the on-chip logits without writing them
- * out (Sec. III-A: p = softmax(o), o = g(x_L)).  For row r (0 <= r < R):
+ * tests and diagnostics that check the logits without writing all of them out
+ * (Sec. III-A: p = softmax(o), o = g(x_L)).  For row r (0 <= r < R):
  *   float4 at byte row_stats_offset + 16 * r: x = max_x logits[r, x],
  *     y = sum_x exp(logits[r, x] - x-component), z = argmax_x logits[r, x]
  *     (int32 bits, lowest index on ties), w = accept bit of the row (int32
  *     bits; 1 iff the row's draft passed its test);
  *   float at byte draft_logit_offset + 4 * r: logits[r, d] of the row's draft
  *     token d (rows i < k_b only; other entries are not written).
- * The statistics are stored in several copies `replica_stride` float4 apart;
- * the first copy is the one described.  Valid until the next call that uses
- * the workspace.  Returns SPADE_ERR_INVALID_ARG on null outputs or bad sizes.
+ * One copy is stored; `replica_stride` is its length in float4 (R).  Valid
+ * until the next call that uses the workspace.  Returns SPADE_ERR_INVALID_ARG on null outputs or bad sizes.
  */
 spade_status spade_accept_stats_layout(int32_t B, int32_t R, int32_t H, int32_t V,
                                        size_t *row_stats_offset, size_t *draft_logit_offset,

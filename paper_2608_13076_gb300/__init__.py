@@ -250,7 +250,7 @@ def read_accept_stats(workspace, B, R, H, V):
 
 
 def spade_accept_launches(B, R, H, V):
-    """Kernel launches of one accept call: 1 (logits on chip) or 2 (statistics pass, then sampling pass)."""
+    """Kernel launches of one accept call: 1, or 2 (statistics, then decisions and draws)."""
     return int(load().spade_accept_launches(B, R, H, V))
 
 

@@ -9,8 +9,10 @@
 //  * y = x W^T is a dense contraction, so it runs on the tensor cores:
 //    tcgen05.mma kind::f16 (bf16 in, fp32 in tensor memory) with W's output
 //    rows on the MMA M side (128-row tiles: one head of dimension 128, or two
-//    of dimension 64, per tile) and the R verify rows on N.  At R = 72 the
-//    work is bound by streaming W from HBM (50 MB for the Llama-3-8B layer).
+//    of dimension 64, per tile) and the R verify rows on N.
+//  * This is the form for more than 128 rows over layers too narrow for the
+//    clusters of qkv_cluster.cu, and for rows that do not fit their ring; the
+//    entry points are here too.
 //  * Stream-K over (tile, k-chunk of 64) units: the units are laid end to end
 //    and cut into one equal range per SM, so every SM streams the same share
 //    of W whatever the tile count.  A ring stage holds up to KG = 2 chunks of
@@ -32,7 +34,9 @@
 //    and values to cache slot ctx_b + i of their sequence (or, for a paged
 //    cache, where the block table puts that slot).
 //  * Warp roles: warp 0 streams W and x tiles with TMA into a ring of stages;
-//    warp 1 issues the MMAs (one elected thread) and owns the tensor memory;
+//    warp 1 issues the MMAs and owns the tensor memory (both walk their loops as
+//    whole warps with an elected lane issuing: the operands of these instructions
+//    live in uniform registers);
 //    warps 2-5 drain accumulators, publish partials and run the reduction.
 //  * Programmatic dependent launch: barriers, tensor memory and tensor-map
 //    prefetch come before the wait on the previous kernel; the attention that
