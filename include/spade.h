@@ -230,7 +230,8 @@ spade_status spade_verify_attention_noalloc(const void *q, const void *k_cache,
  *                 sampled sequences are stored there.
  *   status        device int32, SPADE_DEV_* bits OR-ed in
  * The kernel keeps every block of the grid resident at once (cooperative
- * launch) and meets at bounded device-wide barriers; if a barrier expires the
+ * launch; one cluster for up to 1024 entries, whose blocks meet at the cluster's
+ * barrier) and meets at bounded device-wide barriers; if a barrier expires the
  * outputs are invalid and SPADE_DEV_TIMEOUT is set; zero the workspace again
  * before the next call.
  */

@@ -114,6 +114,23 @@ def test_draw_shares(dev, name):
     assert cmp["mismatch_unflagged"] == 0 and cmp["flagged"] < wl["B"] // 2, cmp
 
 
+# Vocabularies of at most eight tiles run as one cluster, larger ones as a cooperative grid: one CTA, a
+# ragged last tile, the largest cluster and the smallest grid beyond it, with every option at once.
+@pytest.mark.parametrize("V", [100, 129, 1024, 1025])
+@pytest.mark.parametrize("mode", ["greedy", "mixed"])
+def test_small_vocabularies(dev, V, mode):
+    spec = _spec("small_v", 350 + V, B=6, k=(0, 5), V=V, mode=mode, target_accept=0.7, logit_scale=3.0)
+    wl = W.make_workload(spec, device=dev)
+    T, top_p = torch.linspace(0.7, 1.4, 6), torch.linspace(0.5, 1.0, 6)
+    before = {k: wl[k].clone() for k in ("k_cache", "v_cache", "ctx_lens", "n_draft")}
+    acc, tok, st = parity.gpu_accept_sampling(wl, temperature=T.to(dev), top_p=top_p.to(dev), commit=True)
+    torch.cuda.synchronize()
+    assert int(st.item()) & ~spade.DEV_FALLBACK == 0
+    ref = parity.oracle_accept_from_logits(wl, parity.oracle_logits(wl), temperature=T.numpy(), top_p=top_p.numpy())
+    assert parity.compare_accept(acc, tok, ref)["mismatch_unflagged"] == 0
+    parity.check_commit_windows(before, wl["k_cache"], wl["v_cache"], wl["ctx_lens"], acc)
+
+
 # The nucleus search.  Flat logits put nearly every entry in one bin of the first round, so the kept
 # lists overflow and the values are read again; one CTA per group (nothing exchanged) and several.
 @pytest.mark.parametrize("B,V,scale", [(2, 160000, 0.05), (80, 20000, 0.05), (80, 3001, 4.0)])
