@@ -72,7 +72,7 @@ struct Params {
 // operand's read): this CTA's partial sums of a batch of verify rows, and those
 // received for the rows that it finishes.
 struct Layout {
-  int rseq, rpos, freq, qrow, bars, misc, ring, stage_bytes, row_stride, part, recv, total;
+  int rseq, rpos, freq, qrow, bars, misc, ring, stage_bytes, row_stride, part, recv, region, total;
 };
 __host__ __device__ inline Layout layout(int Ncols, int qmax, int stages, int over, int batch) {
   Layout L;
@@ -81,14 +81,15 @@ __host__ __device__ inline Layout layout(int Ncols, int qmax, int stages, int ov
   L.freq = L.rpos + kMaxRows * 4;
   L.qrow = L.freq + 64 * 4;  // uint16 [kMaxQuads][2]
   L.bars = L.qrow + kMaxQuads * 4;
-  L.misc = L.bars + (2 * kMaxStages + 2) * 8;
+  L.misc = L.bars + (2 * kMaxStages + 3) * 8;
   L.ring = (L.misc + 32 + 1023) & ~1023;
   L.stage_bytes = qmax * 1024 + Ncols * 128;  // 8 W rows per quad, then the x rows
   const int end = L.ring + stages * L.stage_bytes;
   L.row_stride = qmax * 8 + 4;                // floats per staged verify row
-  const int staging = (batch + (batch + 1) / 2) * L.row_stride * 4;
+  const int staging = (batch + (batch + 1) / 2) * L.row_stride * 4;  // (a multiple of 16)
   L.part = over ? L.ring : end;
   L.recv = L.part + batch * L.row_stride * 4;
+  L.region = staging;  // the next batch's (in the ring's place)
   L.total = end + (over || staging < kTileBytes ? kTileBytes : staging) + 1024;  // + slack for the 1024-byte alignment
   return L;
 }
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t *full = reinterpret_cast<uint64_t *>(smem + L.bars);
   uint64_t *empty = full + kMaxStages;
   uint64_t *acc_full = empty + kMaxStages;
-  uint64_t *recv_full = acc_full + 1;  // the peer's partial sums have landed
+  uint64_t *recv_full = acc_full + 1;  // [2]: the peer's partial sums of a batch have landed
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.misc);
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.misc + 8);
 
@@ -128,6 +129,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n0 = kBig ? min(p.Ncols, 256) : p.Ncols, n1 = kBig ? p.Ncols - n0 : 0;  // MMA N-chunks
   // Of the nb verify rows of a batch, the first half is finished by CTA 0.
   auto own_rows = [rank](int nb) { return rank ? nb - (nb + 1) / 2 : (nb + 1) / 2; };
+  // Arms the barrier of batch i (if there is one) with the bytes that the peer sends.
+  const int nbatch = kBig ? (p.c.R + p.batch - 1) / p.batch : 1;
+  auto arm = [&](int i) {
+    if (i < nbatch)
+      mbar_arrive_expect_tx(&recv_full[i & 1],
+                            static_cast<uint32_t>(own_rows(min(p.batch, p.c.R - i * p.batch)) * L.row_stride * 4));
+  };
   // This CTA's half of K.  Every cluster reads the same x rows: each starts at
   // another chunk, so that they do not all load the same lines from L2 at once.
   const int kc0 = p.KC * static_cast<int>(rank) / 2, nk = p.KC * (static_cast<int>(rank) + 1) / 2 - kc0;
@@ -157,9 +165,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&empty[s], 1);
       }
       mbar_init(acc_full, 1);
-      mbar_init(recv_full, 1);
+      mbar_init(&recv_full[0], 1);
+      mbar_init(&recv_full[1], 1);
       fence_mbar_init();
-      mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(own_rows(min(p.batch, p.c.R)) * L.row_stride * 4));
+      arm(0);
+      if (kBig) arm(1);
     }
     __syncwarp();
     tmem_alloc(s_tmem, p.tmem_cols);
@@ -256,57 +266,69 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster_sync();  // both rings are idle: their place becomes staging
   }
   const OutMap om = out_map(p.c);
-  float *part = reinterpret_cast<float *>(smem + L.part);
-  const float *recv = reinterpret_cast<const float *>(smem + L.recv);
-  const int dn = kThreads / nq, dq = kThreads - dn * nq, qsh = p.c.D == 128 ? 4 : 3;
-  uint32_t phase = 0;
-  for (int b0 = 0; b0 < p.c.R; b0 += p.batch, phase ^= 1u) {
-    const int nb = kBig ? min(p.batch, p.c.R - b0) : p.c.R, n_own = own_rows(nb), n_send = nb - n_own;
-    const int first = rank ? nb - n_own : 0, first_send = rank ? 0 : n_own;  // within the batch
-    if (warp >= 2) {
-      // Two warps per lane quarter, each every second 16 columns.
-      const int q4 = warp & 3;
-      for (int t = 0; t < ntile; ++t) {
-        if (t * 128 + q4 * 32 >= rows) break;  // (whole warps: rows is a multiple of 8)
-        const int row = t * 128 + q4 * 32 + lane;
-        const uint32_t a = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(t * p.Ncols + b0);
-        for (int c = 16 * ((warp - 2) >> 2); c < nb; c += 32) {
-          uint32_t v[16];
-          if (nk > 0) {
-            tmem_ld8(a + c, v);
-            tmem_ld8(a + c + 8, v + 8);
-            tmem_wait_ld();
-          } else {  // (one k-chunk in all: this CTA has none)
+  // Batches alternate between two regions: this CTA's sums of the batch's rows, then
+  // those received from the peer for the rows that this CTA finishes.
+  auto part_of = [&](int i) { return reinterpret_cast<float *>(smem + L.part + (kBig ? i & 1 : 0) * L.region); };
+  auto recv_of = [&](int i) { return reinterpret_cast<float *>(smem + L.recv + (kBig ? i & 1 : 0) * L.region); };
+  // Batch i from tensor memory to its region, and the peer's rows on their way
+  // (epilogue warps).
+  auto stage = [&](int i) {
+    const int b0 = i * p.batch, nb = kBig ? min(p.batch, p.c.R - b0) : p.c.R;
+    const int n_own = own_rows(nb), n_send = nb - n_own, first_send = rank ? 0 : n_own;
+    float *part = part_of(i);
+    // Two warps per lane quarter, each every second 16 columns.
+    const int q4 = warp & 3;
+    for (int t = 0; t < ntile; ++t) {
+      if (t * 128 + q4 * 32 >= rows) break;  // (whole warps: rows is a multiple of 8)
+      const int row = t * 128 + q4 * 32 + lane;
+      const uint32_t a = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + static_cast<uint32_t>(t * p.Ncols + b0);
+      for (int c = 16 * ((warp - 2) >> 2); c < nb; c += 32) {
+        uint32_t v[16];
+        if (nk > 0) {
+          tmem_ld8(a + c, v);
+          tmem_ld8(a + c + 8, v + 8);
+          tmem_wait_ld();
+        } else {  // (one k-chunk in all: this CTA has none)
 #pragma unroll
-            for (int e = 0; e < 16; ++e) v[e] = 0u;
-          }
-          if (row < rows) {
-            float *to = part + c * L.row_stride + row;
+          for (int e = 0; e < 16; ++e) v[e] = 0u;
+        }
+        if (row < rows) {
+          float *to = part + c * L.row_stride + row;
 #pragma unroll
-            for (int e = 0; e < 16; ++e)
-              if (c + e < nb) to[e * L.row_stride] = __uint_as_float(v[e]);
-          }
+          for (int e = 0; e < 16; ++e)
+            if (c + e < nb) to[e * L.row_stride] = __uint_as_float(v[e]);
         }
       }
-      // The peer's rows travel in one copy.
-      fence_proxy_async_smem();
-      epi_bar();
-      if (tid == 64 && n_send > 0)
-        bulk_copy_cluster(cluster_map(recv, rank ^ 1u), part + first_send * L.row_stride,
-                          static_cast<uint32_t>(n_send * L.row_stride * 4), cluster_map(recv_full, rank ^ 1u));
     }
+    // The peer's rows travel in one copy.
+    fence_proxy_async_smem();
+    epi_bar();
+    if (tid == 64 && n_send > 0)
+      bulk_copy_cluster(cluster_map(recv_of(i), rank ^ 1u), part + first_send * L.row_stride,
+                        static_cast<uint32_t>(n_send * L.row_stride * 4), cluster_map(&recv_full[kBig ? i & 1 : 0], rank ^ 1u));
+  };
+  const int dn = kThreads / nq, dq = kThreads - dn * nq, qsh = p.c.D == 128 ? 4 : 3;
+  if (warp >= 2) {
+    stage(0);
+    if (kBig && nbatch > 1) stage(1);
+  }
+#pragma unroll 1
+  for (int i = 0; i < nbatch; ++i) {
+    const int b0 = i * p.batch, nb = kBig ? min(p.batch, p.c.R - b0) : p.c.R, n_own = own_rows(nb);
+    const int first = rank ? nb - n_own : 0;  // within the batch
+    const float *part = part_of(i), *recv = recv_of(i);
     __syncwarp();
-    __syncthreads();
-    if (!mbar_wait_unabortable(recv_full, phase)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+    __syncthreads();  // staged
+    if (!mbar_wait_unabortable(&recv_full[kBig ? i & 1 : 0], kBig ? (i >> 1) & 1 : 0)) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
     // Items (verify row, quad), kThreads apart.
     for (int n = tid / nq, q = tid - n * nq; n < n_own;) {
       const int r = b0 + first + n;
       const uint32_t row = s_row[r];
       if (row != kNoRow) {
-        const float *o = part + (first + n) * L.row_stride, *i = recv + n * L.row_stride;
+        const float *o = part + (first + n) * L.row_stride, *in = recv + n * L.row_stride;
         const int r1 = s_qrow[2 * q], r2 = s_qrow[2 * q + 1];
         const float4 o1 = *reinterpret_cast<const float4 *>(o + r1), o2 = *reinterpret_cast<const float4 *>(o + r2);
-        const float4 i1 = *reinterpret_cast<const float4 *>(i + r1), i2 = *reinterpret_cast<const float4 *>(i + r2);
+        const float4 i1 = *reinterpret_cast<const float4 *>(in + r1), i2 = *reinterpret_cast<const float4 *>(in + r2);
         float y1[4] = {o1.x + i1.x, o1.y + i1.y, o1.z + i1.z, o1.w + i1.w};
         float y2[4] = {o2.x + i2.x, o2.y + i2.y, o2.z + i2.z, o2.w + i2.w};
         const int Q = q0 + q, hg = Q >> qsh;
@@ -316,12 +338,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       q += dq;
       if (q >= nq) { q -= nq; ++n; }
     }
-    if (kBig && b0 + p.batch < p.c.R) {
-      if (tid == 0)
-        mbar_arrive_expect_tx(recv_full, static_cast<uint32_t>(own_rows(min(p.batch, p.c.R - b0 - p.batch)) * L.row_stride * 4));
+    if (kBig && i + 2 < nbatch) {
+      if (tid == 0) arm(i + 2);
       __syncwarp();
       __syncthreads();
-      cluster_sync();  // both CTAs have read their staging, and their copies have left it
+      cluster_sync();  // both CTAs have read this region, and their copies have left it
+      if (warp >= 2) stage(i + 2);
     }
   }
   tc_fence_before();
@@ -376,10 +398,12 @@ static Params plan(const Call &c, int sms) {
   if (p.qmax >= 8 && n >= kMinStagesOver && L.recv + kBatch / 2 * L.row_stride * 4 <= L.ring + n * L.stage_bytes) {
     p.stages = n;
     p.over = 1;
-    // As few batches as fit, of nearly equal sizes (multiples of 16): each costs
-    // its barriers and an exchange (389 rows in two of 208 at most instead of
-    // four of 128: 40.7 -> 34.5 us with the row table's cache rows).
-    const int fit = n * L.stage_bytes / (L.row_stride * 6) / 16 * 16, nb = (c.R + fit - 1) / fit;
+    // Two regions, so that a batch's exchange and staging run under the one before
+    // it; at least two batches, as few as fit, of nearly equal sizes (multiples of 16).
+    // 389 paged rows x 5120 x 7168: 33.7 us; in one region 34.8 (two batches) and
+    // 40.7 (four, with pages looked up and divisions per item).
+    const int fit = n * L.stage_bytes / (L.row_stride * 12) / 16 * 16;
+    const int nb = c.R > 2 * fit ? (c.R + fit - 1) / fit : 2;
     p.batch = ((c.R + nb - 1) / nb + 15) / 16 * 16;
   }
   return p;
