@@ -64,6 +64,18 @@ __host__ __device__ inline PairSmem pair_layout(int Ncols, int stages) {
   return s;
 }
 
+// Vocabulary slice of CTA `rank` of pair j.  Pairs walk the k-chunks from different
+// starts, so that not all of them load the same hidden lines from L2 at once:
+// slice s from chunk 2 (s mod ns), as the one-launch form (stages of two chunks)
+// walks it, so a logit is summed in the same order, to the same bits, in either.  A
+// pair has one order: it takes slices s and s + ns, which share it; the last few
+// slices without such a partner pair up with their neighbours.
+__device__ __forceinline__ int pair_slice(int j, int rank, int nslices, int ns) {
+  const int group = j / ns, i = j - group * ns, base = 2 * ns * group;
+  const int both = max(0, min(nslices - base, 2 * ns) - ns);  // pairs (s, s + ns) of this group
+  return i < both ? base + i + rank * ns : base + both + 2 * (i - both) + rank;
+}
+
 __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
     const __grid_constant__ PairParams p, const __grid_constant__ CUtensorMap tm_w,
     const __grid_constant__ CUtensorMap tm_h0, const __grid_constant__ CUtensorMap tm_h1) {
@@ -80,8 +92,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
   const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, false);
 
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
-  const int c = blockIdx.x;
   const uint32_t rank = cluster_ctarank();
+  const int ns = (p.KC + 1) / 2;
+  const int c = pair_slice(blockIdx.x >> 1, rank, p.c.NC, ns);
   const int v_lo = static_cast<int>(static_cast<int64_t>(c) * p.c.V / p.c.NC);
   const int v_hi = static_cast<int>(static_cast<int64_t>(c + 1) * p.c.V / p.c.NC);
   // Both CTAs of a pair walk p.ntiles tiles (a slice one row shorter may leave
@@ -115,9 +128,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
   const uint32_t tmem = *s_tmem;
   const uint32_t h1_off = static_cast<uint32_t>(kWChunkBytes + p.n0w / 2 * 128);
   int tiles_issued = 0;
-  // Pairs walk the k-chunks from different starts, so that not all of them load
-  // the same hidden lines from L2 at once.
-  const int k_rot = (c >> 1) % p.KC;
+  const int k_rot = 2 * (pair_slice(blockIdx.x >> 1, 0, p.c.NC, ns) % ns);
 
   if (warp == 0) {
     // Both CTAs' copies of a stage complete on the even CTA's full barrier,
