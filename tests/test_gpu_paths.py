@@ -88,6 +88,24 @@ def test_lm_head_row_counts(dev, name, mode):
     assert worst["argmax_mismatch"] == 0 and max(worst["max"], worst["lse"], worst["draft_logit"]) <= 1.0, worst
 
 
+# The pair kernel sums a logit in the one-launch form's order (pairs of slices that share it; only
+# the last 8 of 152 slices have no such partner): the rows' maxima have the same bits.
+def test_pairs_sum_as_one_launch(dev):
+    wl = W.make_workload(_spec("order", 330, B=65, k=(3, 3), H=1280, V=20000), device=dev)
+    n, B = 64, 16
+    part = dict(wl, B=B, R=n, hidden=wl["hidden"][:n].contiguous(), draft_tokens=wl["draft_tokens"][:n - B].contiguous(),
+                uniforms=wl["uniforms"][:n].contiguous(), mode=wl["mode"][:B].contiguous(),
+                cu_q=wl["cu_q"][:B + 1].contiguous(), n_draft=wl["n_draft"][:B].contiguous())
+    maxima = []
+    for w, launches in ((wl, 2), (part, 1)):
+        assert spade.spade_accept_launches(w["B"], w["R"], w["H"], w["V"]) == launches
+        ws = spade.accept_workspace(w["B"], w["R"], w["H"], w["V"], device=dev)
+        parity.gpu_accept(w, workspace=ws)
+        torch.cuda.synchronize()
+        maxima.append(spade.read_accept_stats(ws, w["B"], w["R"], w["H"], w["V"])["max"][:n])
+    assert float((maxima[0] == maxima[1]).float().mean()) > 0.8
+
+
 # The draw.  Shares of one piece and of several (more than 8192 entries: two buffers, and the owner's
 # piece again), groups of one CTA and of more, q rows that bulk copies can and cannot read.
 DRAW = {
