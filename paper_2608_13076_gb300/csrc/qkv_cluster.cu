@@ -339,9 +339,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (q >= nq) { q -= nq; ++n; }
     }
     if (kBig && i + 2 < nbatch) {
-      if (tid == 0) arm(i + 2);
       __syncwarp();
       __syncthreads();
+      // Every thread of this CTA has seen batch i's phase complete, and the peer sends
+      // only after the cluster's barrier.  (A last batch of one row brings CTA 1
+      // nothing: armed with 0 bytes its phase completes at once, and a thread still
+      // waiting for batch i's would miss both.)
+      if (tid == 0) arm(i + 2);
+      __syncwarp();
       cluster_sync();  // both CTAs have read this region, and their copies have left it
       if (warp >= 2) stage(i + 2);
     }

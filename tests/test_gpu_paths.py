@@ -24,7 +24,7 @@ def _spec(name, seed, **over):
 
 # The projection.  At most 128 rows: a cluster of two CTAs per range of rotary pairs, each with half
 # of the k-chunks (H = 64: one of them has none).  More rows over wide layers (at least eight quads
-# of pairs per cluster): a second MMA chunk above 256 rows, the exchange in one to three batches.
+# of pairs per cluster): a second MMA chunk above 256 rows, the exchange in two to four batches.
 # More rows over narrow layers, or more than fit the ring: the form with partial sums in a workspace.
 QKV = {
     "one_row_one_chunk": dict(H=64),
@@ -36,6 +36,9 @@ QKV = {
     "rows272_wide_d64": dict(B=34, k=(7, 7), H=192, D=64, Hq=60, Hkv=10),
     "rows389_wide": dict(B=64, k=(1, 10), H=200, Hq=40, Hkv=8),
     "rows512_wide": dict(B=64, k=(7, 7), H=128, Hq=32, Hkv=4),
+    # four batches, the last of one row: CTA 1 of each cluster receives nothing of it
+    "rows193_four_batches": dict(B=1, k=(192, 192), H=128, Hq=58, Hkv=29),
+    "rows193_four_batches_d64": dict(B=193, H=128, D=64, Hq=216, Hkv=8),
     "rows129_narrow": dict(B=3, k=(42, 42), H=200),
 }
 
