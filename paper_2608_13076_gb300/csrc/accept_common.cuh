@@ -1199,6 +1199,7 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
   const int e0 = lo + s.owner_piece * kPiece, len = min(kPiece, hi - e0);
   const float *terms = piece_buf(s, s.owner_piece % nbuf);
   if (warp != s.owner_warp) return;
+  __syncwarp();  // a piece taken again: its terms were stored lane by lane, the walk below reads another lane's
   // The lane block, then the entry.
   const ff2 left = s.tgt;
   const ff2 prev{__shfl_up_sync(0xffffffffu, incl.hi, 1), __shfl_up_sync(0xffffffffu, incl.lo, 1)};

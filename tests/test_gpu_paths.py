@@ -135,6 +135,24 @@ def test_draw_shares(dev, name):
     assert cmp["mismatch_unflagged"] == 0 and cmp["flagged"] < wl["B"] // 2, cmp
 
 
+# A target before the last piece of a share: its piece is copied and turned into terms once more, and
+# the walk reads the terms that other lanes of the warp have just stored.
+@pytest.mark.parametrize("B,k,V", [(80, 1, 20000), (80, 1, 20001), (130, 1, 20004)])
+def test_draw_piece_again(dev, B, k, V):
+    spec = _spec("again", 355 + V % 7, B=B, k=(k, k), V=V, H=128, mode="stochastic", target_accept=0.7, logit_scale=2.0)
+    wl = W.make_workload(spec, device=dev)
+    wl["uniforms"][wl["cu_q"][1:].long() - 1] = torch.linspace(0.01, 0.75, B, device=dev)
+    ref = parity.oracle_accept(wl)
+    assert int((ref["next_token"] < 2 * 8192).sum()) > B // 2
+    ws = spade.accept_workspace(B, wl["R"], wl["H"], V, device=dev)
+    for _ in range(8):
+        acc, tok, st = parity.gpu_accept(wl, workspace=ws)
+        torch.cuda.synchronize()
+        assert int(st.item()) & ~spade.DEV_FALLBACK == 0
+        cmp = parity.compare_accept(acc, tok, ref)
+        assert cmp["mismatch_unflagged"] == 0 and cmp["flagged"] < B // 2, cmp
+
+
 # Vocabularies of at most eight tiles run as one cluster, larger ones as a cooperative grid: one CTA, a
 # ragged last tile, the largest cluster and the smallest grid beyond it, with every option at once.
 @pytest.mark.parametrize("V", [100, 129, 1024, 1025])
