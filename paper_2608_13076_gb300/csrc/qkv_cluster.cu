@@ -250,7 +250,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (nk > 0 && leader) {
       tc_commit(acc_full);
-      if (!ok) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+      if (!ok) {
+        atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+        // Every MMA issued must be done before its operands and the tensor memory go away.
+        mbar_wait_unabortable(acc_full, 0);
+      }
     }
   } else {
     // ===================== epilogue warps: wait for the accumulators =======

@@ -82,8 +82,8 @@ __host__ __device__ inline Layout layout(int Ncols, int stages, int KG) {
   L.ring = 0;
   L.rseq = stages * L.stage_bytes;   // int32 [kMaxR]: sequence of each row (-1: skip)
   L.rpos = L.rseq + kMaxR * 4;       // int32 [kMaxR]: position of each row
-  L.bars = L.rpos + kMaxR * 4;       // full[stages], empty[stages], acc_full[2], acc_empty[2]
-  L.misc = L.bars + (2 * kMaxStages + 4) * 8;  // tmem base, abort flag, last-arrival flag
+  L.bars = L.rpos + kMaxR * 4;       // full[stages], empty[stages], acc_full[2], acc_empty[2], drain
+  L.misc = (L.bars + (2 * kMaxStages + 5) * 8 + 15) & ~15;  // tmem base, abort flag, last-arrival flag
   L.freq = L.misc + 64;              // float [64]: rotary frequencies (per-thread indices
                                      // into the parameter array would serialise)
   L.total = L.freq + 64 * 4 + 1024;  // + slack for the 1024-byte alignment
@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t *bar_empty = bar_full + kMaxStages;
   uint64_t *acc_full = bar_empty + kMaxStages;  // [2]
   uint64_t *acc_empty = acc_full + 2;           // [2]
+  uint64_t *bar_drain = acc_empty + 2;          // every MMA issued is done, after an expired wait
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.misc);
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.misc + 8);
   float *s_freq = reinterpret_cast<float *>(smem + L.freq);
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&acc_full[b], 1);
         mbar_init(&acc_empty[b], kEpiWarps);
       }
+      mbar_init(bar_drain, 1);
       fence_mbar_init();
     }
     __syncwarp();
@@ -325,7 +327,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       c0 = 0;
       if (++buf == p.nbuf) { buf = 0; ++use; }
     }
-    if (!ok && leader) atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+    if (!ok && leader) {
+      atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
+      // Every MMA issued must be done before its operands and the tensor memory go away.
+      tc_commit(bar_drain);
+      mbar_wait_unabortable(bar_drain, 0);
+    }
   } else {
     // ===================== epilogue warps: drain, publish, reduce ==========
     const int et = tid - 64;         // 0..127

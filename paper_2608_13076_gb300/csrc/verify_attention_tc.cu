@@ -54,10 +54,10 @@ constexpr float kRescaleLog2 = 8.f;
 
 // mbarriers.  ODone completes once per PV (chunk); OFinal once per segment,
 // after its last PV, so the epilogue never waits on a parity that an older,
-// still-running PV could alias.
+// still-running PV could alias.  Drain: every MMA issued is done, after an expired wait.
 constexpr int kBarKFull = 0, kBarVFull = 2, kBarKEmpty = 4, kBarVEmpty = 6, kBarSFull = 8,
               kBarSFree = 10, kBarPFull = 12, kBarPFree = 14, kBarODone = 16, kBarSeg = 17,
-              kBarOFinal = 18, kBarQ = 19, kNumBars = 20;
+              kBarOFinal = 18, kBarQ = 19, kBarDrain = 20, kNumBars = 21;
 
 struct Smem {
   static constexpr int K = 0;                               // [stage][2 slabs][128 keys][128 B]
@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bars[kBarSeg], kSoftWarps);
       mbar_init(&bars[kBarQ], kSoftWarps);
       mbar_init(&bars[kBarOFinal], 1);
+      mbar_init(&bars[kBarDrain], 1);
       fence_mbar_init();
     }
     __syncwarp();
@@ -431,7 +432,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       ++seg;
       x = si.seg_end;
     }
-    if (!ok && leader) atomicOr(p.status, SPADE_DEV_TIMEOUT);
+    if (!ok && leader) {
+      atomicOr(p.status, SPADE_DEV_TIMEOUT);
+      // Every MMA issued must be done before its operands and the tensor memory go away.
+      tc_commit(&bars[kBarDrain]);
+      mbar_wait_unabortable(&bars[kBarDrain], 0);
+    }
   } else {
     // ===================== softmax and epilogue (warps 2-9) =================
     constexpr int NH = NR / 2;             // rows (S^T / O^T columns) per softmax warp
