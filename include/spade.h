@@ -448,7 +448,9 @@ const char *spade_version(void);
  * that nothing completes.  After limit_us microseconds of %globaltimer
  * (1 .. 1000000) the wait gives up, SPADE_DEV_TIMEOUT is OR-ed into *status
  * (device int32) and the kernel returns normally, so the context stays
- * usable.  No other effect; for health checks and tests of status reporting.
+ * usable; the waits that it makes after that one (192 of them) return at once,
+ * as every kernel's do.  No other effect; for health checks and tests of status
+ * reporting.
  * Returns SPADE_ERR_INVALID_ARG for a null status or a limit out of range.
  */
 spade_status spade_selftest_wait_timeout(int32_t *status, int32_t limit_us, spade_stream_t stream);

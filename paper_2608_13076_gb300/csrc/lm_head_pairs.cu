@@ -169,29 +169,32 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
     if (!ok && rank == 0 && leader) {
       const uint32_t n = p.stages;
       for (uint32_t j = (issued > n ? issued - n : 0); j < issued; ++j)
-        mbar_wait_unabortable(&full[j % n], (j / n) & 1);
+        if (!mbar_wait_unabortable(&full[j % n], (j / n) & 1)) break;  // (the odd CTA stopped before this stage)
     }
   } else if (warp == 1) {
     if (rank == 0) {
       // Even CTA: M = 256 MMAs over both CTAs' stages; the stages are freed in
-      // both CTAs by one multicast commit.  (After an expired wait the results
-      // are void and the waits no-ops.)
+      // both CTAs by one multicast commit.  (An expired wait of the CTA ends the
+      // MMAs: the results are void.  Every tile's commit still comes, as both
+      // CTAs' teardown waits for the last ones.)
       const bool leader = elect_one();
       int s = 0;
       uint32_t ph = 0;
+      bool ok = true;
       for (int t = 0; t < p.ntiles; ++t) {
         const int buf = p.nacc == 2 ? t & 1 : 0, use = p.nacc == 2 ? t >> 1 : t;
         const uint32_t d0 = tmem + static_cast<uint32_t>(buf * (kTmemCols / 2));
         const uint32_t d1 = d0 + static_cast<uint32_t>(p.n0w);
-        if (use > 0) {
+        if (ok && use > 0) {
           if (leader) mbar_wait_cluster(&acc_empty[buf], (use - 1) & 1, s_abort);
           __syncwarp();
         }
         tc_fence_after();
-        for (int it = 0; it < p.KC; ++it) {
+        for (int it = 0; ok && it < p.KC; ++it) {
           // (cta-scope wait: the copies' completion on this barrier orders them
           // for the MMAs issued after it, the odd CTA's included)
-          warp_wait(&full[s], ph, s_abort);
+          ok = warp_wait(&full[s], ph, s_abort);
+          if (!ok) break;
           // Arm the stage's next use now: its copies are issued only after this
           // use's commit frees the stage.
           if (leader) mbar_arrive_expect_tx(&full[s], 2 * stage_tx);

@@ -69,10 +69,25 @@ SPADE_DEVICE bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Whether phase `parity` has completed, without suspending the thread.
+SPADE_DEVICE bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait for phase `parity` of `bar`.  `abort` is a CTA-shared flag: once
-// any wait of the CTA has expired every later wait returns at once.  Returns
-// false if this wait expired (the caller records the status).
+// any wait of the CTA has expired every later wait returns at once (the flag is
+// read before a wait may suspend its thread; a completed phase is seen without it).
+// Returns false if this wait expired (the caller records the status).
 SPADE_DEVICE bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  if (mbar_test_wait(bar, parity) || *abort) return true;
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer();
   while (true) {
@@ -120,7 +135,10 @@ SPADE_DEVICE bool elect_one() {
 }
 // Bounded wait of a whole warp (all lanes get the same answer): true once the
 // phase has completed, false if this or an earlier wait of the CTA expired.
+// (An earlier expiry is seen before the wait may suspend the warp.)
 SPADE_DEVICE bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+  if (__any_sync(0xffffffffu, *abort != 0)) return false;
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   const uint64_t t0 = globaltimer();
   bool done = false, give_up = false;
@@ -308,7 +326,19 @@ SPADE_DEVICE bool mbar_try_wait_cluster(uint64_t *bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+SPADE_DEVICE bool mbar_test_wait_cluster(uint64_t *bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 SPADE_DEVICE bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, volatile int *abort) {
+  if (mbar_test_wait_cluster(bar, parity) || *abort) return true;
   if (mbar_try_wait_cluster(bar, parity)) return true;  // no timer read on the fast path
   const uint64_t t0 = globaltimer();
   while (true) {

@@ -228,7 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t ph = 0;
     bool ok = true;
     for (int it = 0; it < nk; ++it) {
-      ok &= warp_wait(&full[s], ph, s_abort);  // (after an expired wait the results are void, the waits no-ops)
+      ok = warp_wait(&full[s], ph, s_abort);
+      if (!ok) break;  // (an expired wait of the CTA: the results are void)
       tc_fence_after();
       const uint32_t base = smem_u32(smem + L.ring + s * L.stage_bytes);
       // Descriptors built once per operand; a K step of 16 adds 32 bytes, 2 in

@@ -289,18 +289,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool leader = elect_one();
     const uint32_t idesc0 = idesc_bf16_f32(kTileM, n0);
     const uint32_t idesc1 = idesc_bf16_f32(kTileM, n1 ? n1 : 16);
-    bool ok = true;  // (after an expired wait the results are void and the waits no-ops)
+    bool ok = true;  // (an expired wait of the CTA ends the loops: the results are void)
     int st = 0, buf = 0, use = 0, c0 = u0 % p.KC;
     uint32_t ph = 0;
-    for (int u = u0; u < u1;) {
+    for (int u = u0; ok && u < u1;) {
       const int len = min(u1 - u, p.KC - c0);  // this segment's chunks
       // The buffer's previous segment has been drained by the epilogue warps.
-      if (use > 0) ok &= warp_wait(&acc_empty[buf], (use - 1) & 1, s_abort);
+      if (use > 0) ok = warp_wait(&acc_empty[buf], (use - 1) & 1, s_abort);
       tc_fence_after();
       const uint32_t acc_addr = tmem + static_cast<uint32_t>(buf) * p.buf_cols;
-      for (int done = 0; done < len;) {
+      for (int done = 0; ok && done < len;) {
         const int nch = min(p.KG, len - done);  // as the producer cut the stage
-        ok &= warp_wait(&bar_full[st], ph, s_abort);
+        ok = warp_wait(&bar_full[st], ph, s_abort);
+        if (!ok) break;
         tc_fence_after();
         const uint32_t a0 = smem_base + L.ring + st * L.stage_bytes;
         for (int j = 0; j < nch; ++j) {
@@ -429,7 +430,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (load_acquire(&published[t]) != nparts) {
         const uint64_t t0 = globaltimer();
         while (load_acquire(&published[t]) != nparts) {
-          if (globaltimer() - t0 > kWaitLimitNs) {
+          if (*s_abort || globaltimer() - t0 > kWaitLimitNs) {  // (later slabs do not wait again)
+            *s_abort = 1;
             atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
             s_fin[3] = 0;
             break;

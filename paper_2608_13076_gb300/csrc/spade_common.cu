@@ -115,16 +115,33 @@ bool encode_tmap_rows_by_slab(CUtensorMap *map, const void *base, uint64_t rows,
 }
 
 // One thread waits on an mbarrier that nothing completes, bounded as every
-// kernel's waits are, and reports the expiry in the status word.
+// kernel's waits are, and reports the expiry in the status word; then, with the
+// block's abort flag set as an expired wait leaves it, waits of every kind that
+// must return at once.
 __global__ void selftest_wait_kernel(int32_t *status, uint64_t limit_ns) {
   __shared__ uint64_t bar;
+  __shared__ int abort;
   if (threadIdx.x == 0) {
+    abort = 0;
     mbar_init(&bar, 1);
     fence_mbar_init();
     const uint64_t t0 = globaltimer();
     bool done = mbar_try_wait(&bar, 0);
     while (!done && globaltimer() - t0 <= limit_ns) done = mbar_try_wait(&bar, 0);
-    if (!done) atomicOr(status, SPADE_DEV_TIMEOUT);
+    if (!done) {
+      atomicOr(status, SPADE_DEV_TIMEOUT);
+      abort = 1;
+    }
+  }
+  __syncwarp();
+  volatile int *flag = &abort;
+  for (int i = 0; i < 64 && *flag; ++i) {
+    if (threadIdx.x == 0) {
+      mbar_wait(&bar, 0, flag);
+      mbar_wait_cluster(&bar, 0, flag);
+    }
+    __syncwarp();
+    warp_wait(&bar, 0, flag);
   }
 }
 

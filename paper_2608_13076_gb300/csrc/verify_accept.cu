@@ -219,22 +219,25 @@ __global__ void __launch_bounds__(kThreads, 1) verify_accept_kernel(
     int ws = 0, hs = 0;
     uint32_t wph = 0, hph = 0;
     int tdone = 0;
-    // (after an expired wait the results are void and the waits no-ops)
-    for (int r = 0; r < p.nrounds && tdone < ntiles; ++r) {
+    // (an expired wait of the CTA ends the loops: the results are void.  The round's
+    // commit still comes: teardown waits for it before the tensor memory goes away.)
+    bool ok = true;
+    for (int r = 0; ok && r < p.nrounds && tdone < ntiles; ++r) {
       const int nt = min(p.round_tiles[r], ntiles - tdone);
       const int buf = r & 1;
       // The half's previous round has been read.
-      if (r > 1) warp_wait(&acc_empty[buf], ((r >> 1) - 1) & 1, s_abort);
+      if (r > 1) ok = warp_wait(&acc_empty[buf], ((r >> 1) - 1) & 1, s_abort);
       tc_fence_after();
       int ks = k_rot;
-      for (int it = 0; it < p.NS; ++it) {
+      for (int it = 0; ok && it < p.NS; ++it) {
         const int nch = min(p.KG, p.KC - ks * p.KG);
         if (++ks == p.NS) ks = 0;
-        warp_wait(&h_full[hs], hph, s_abort);
+        ok = warp_wait(&h_full[hs], hph, s_abort);
         tc_fence_after();
         const uint32_t h_addr = smem_u32(h_ring + hs * L.h_slot);
         for (int j = 0; j < nt; ++j) {
-          warp_wait(&w_full[ws], wph, s_abort);
+          ok = ok && warp_wait(&w_full[ws], wph, s_abort);
+          if (!ok) break;
           tc_fence_after();
           const uint32_t w_addr = smem_u32(w_ring + ws * L.w_slot);
           // k-chunk stride in the slot: a full tile's chunks are 16 KB apart,

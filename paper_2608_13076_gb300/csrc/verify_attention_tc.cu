@@ -375,7 +375,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr uint32_t idesc_s = idesc_bf16_f32(128, NR);                           // K-major A, B
     constexpr uint32_t idesc_pv = idesc_bf16_f32(128, NR) | (1u << 15) | (1u << 16);  // MN-major A, B
     const bool leader = elect_one();
-    bool ok = true;  // (after an expired wait the results are void and the waits no-ops)
+    // An expired wait of the CTA ends the loops: the results are void.  (Looked at
+    // once per chunk: a branch at each wait costs 0.7 us at 8 x 4096 keys.)
+    bool ok = true;
     uint32_t it = 0, seg = 0;
     // O^T += V^T P^T for chunk j (first: overwrite instead of accumulate;
     // last: the segment's final product, signalled on OFinal too).
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (last) tc_commit(&bars[kBarOFinal]);
       }
     };
-    for (int64_t x = x_begin; x < x_end;) {
+    for (int64_t x = x_begin; ok && x < x_end;) {
       const SegInfo si = x == x_begin ? seg0 : next_seg_warp(sc, x, x_end, lane);
       const int nchunk = uniform(si.nchunk);
       if (uniform(si.n_here) == 0) break;
@@ -427,7 +429,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           tc_commit(&bars[kBarKEmpty + st]);
         }
         if (c > 0) issue_pv(it - 1, c == 1, false);
+        if (!ok) break;
       }
+      if (!ok) break;
       issue_pv(it - 1, nchunk == 1, true);
       ++seg;
       x = si.seg_end;

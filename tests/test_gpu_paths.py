@@ -187,6 +187,21 @@ def test_top_p_lists(dev, B, V, scale):
     assert int(tok.min()) >= 0 and int(tok.max()) < V
 
 
+# After an expired wait every later wait of the block returns at once: 192 of them, each of which may
+# suspend its warp for 1 ms if it does not look at the flag first, within 20 ms (64 ms is a third of that).
+def test_waits_after_an_expired_one(dev):
+    st = spade.status_tensor(dev)
+    spade.spade_selftest_wait_timeout(st, 1000)
+    torch.cuda.synchronize()
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    spade.spade_selftest_wait_timeout(st, 1000)
+    t1.record()
+    torch.cuda.synchronize()
+    assert int(st.item()) == spade.DEV_TIMEOUT
+    assert 1.0 <= t0.elapsed_time(t1) < 20.0
+
+
 # Attention units split into many parts: the merge's batches of four parts and its rows' remainders.
 @pytest.mark.parametrize("D,G,k,ctx", [(128, 1, 0, 20000), (64, 1, 0, 700), (128, 5, 6, 9000), (64, 8, 7, 20000),
                                        (128, 8, 7, 600), (128, 3, 8, 330)])
