@@ -292,6 +292,7 @@ struct SeqTable {
   int st[kMaxB];  // sampled sequences, ascending
   int gr[kMaxB];  // greedy and invalid ones
   int n_st, n_gr;
+  int rest;  // whether some row belongs to no valid sequence
   // This CTA among the groups that draw: groups, CTAs in each, its group and rank,
   // and its share [lo, hi) of the vocabulary.
   int ngroups, gs, g, rank, lo, hi;
@@ -339,10 +340,12 @@ __device__ __forceinline__ void share_of(int V, int gs, int rank, int *lo, int *
 // one warp, once the table is full.
 __device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int c, int nctas, int lane) {
   int ns = 0, ng = 0;
+  unsigned invalid = 0u;
   for (int b0 = 0; b0 < p.B; b0 += 32) {
     const int b = b0 + lane;
     const unsigned in = p.B - b0 >= 32 ? 0xffffffffu : (1u << (p.B - b0)) - 1u;
     const unsigned ms = t.stoch[b0 / 32] & in, mg = ~t.stoch[b0 / 32] & in;
+    invalid |= ~t.valid[b0 / 32] & in;
     const unsigned bit = 1u << lane, below = bit - 1u;
     if (ms & bit) t.st[ns + __popc(ms & below)] = b;
     if (mg & bit) t.gr[ng + __popc(mg & below)] = b;
@@ -352,6 +355,8 @@ __device__ __forceinline__ void fill_lists(const Call &p, SeqTable &t, int c, in
   if (lane == 0) {
     t.n_st = ns;
     t.n_gr = ng;
+    // (valid sequences follow one another, so all of them cover the rows from the first's start on)
+    t.rest = invalid != 0u || t.r0[0] != 0 || t.r0[p.B - 1] + t.k[p.B - 1] + 1 != p.R;
     t.ngroups = min(ns, nctas);
     t.gs = ns == 0 ? 1 : max(1, min(min(nctas / t.ngroups, kMaxGroup), (p.V + kMinShare - 1) / kMinShare));
     t.g = c / t.gs;
@@ -623,22 +628,69 @@ __device__ __forceinline__ void post_mass(unsigned long long *a, ff2 z) {
   st_relaxed64(a, static_cast<unsigned long long>(lo) << 32 | __float_as_uint(z.hi));
 }
 
+// A row's merged statistics over the NC slice partials (in `part`, lane by lane):
+// the maximum first, then its lowest index and the rescaled sum.  lane 0's values count.
+constexpr int kPartLoads = kMaxNC / 32;
+__device__ __forceinline__ void load_parts(const Call &p, int n, int lane, float4 (&part)[kPartLoads]) {
+#pragma unroll
+  for (int j = 0; j < kPartLoads; ++j) {
+    const int cc = j * 32 + lane;
+    part[j] = cc < p.NC ? __ldcg(&p.pstat[static_cast<size_t>(n) * p.NC + cc])
+                        : make_float4(-INFINITY, 0.f, __int_as_float(INT_MAX), 0.f);
+  }
+}
+__device__ __forceinline__ void merge_parts(const float4 (&part)[kPartLoads], float &m, float &z, int &idx) {
+  m = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < kPartLoads; ++j) m = fmaxf(m, part[j].x);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  z = 0.f;
+  idx = INT_MAX;
+  if (m != -INFINITY) {
+#pragma unroll
+    for (int j = 0; j < kPartLoads; ++j) {
+      z += part[j].y * ex2((part[j].x - m) * kLog2e);
+      if (part[j].x == m) idx = min(idx, __float_as_int(part[j].z));
+    }
+  }
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    z += __shfl_xor_sync(0xffffffffu, z, o);
+    idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, o));
+  }
+}
+
+// Statistics of the rows that belong to no valid sequence (past cu_q[B], or of a
+// sequence that was reported), with accept bit 0; one warp per row.
+__device__ __forceinline__ void rest_rows(const Call &p, const SeqTable &seqs, int c, int nctas, int warp, int lane) {
+#pragma unroll 1
+  for (int n = c * kWarps + warp; n < p.R; n += nctas * kWarps) {
+    bool taken = false;
+    for (int b = lane; b < p.B; b += 32) {
+      const SeqInfo q = table_info(seqs, b);
+      taken |= q.valid && n >= q.r0 && n <= q.r0 + q.k;
+    }
+    if (__any_sync(0xffffffffu, taken)) continue;
+    float4 part[kPartLoads];
+    load_parts(p, n, lane, part);
+    float m, z;
+    int idx;
+    merge_parts(part, m, z, idx);
+    if (lane == 0) __stcg(&p.gstat[n], make_float4(m, z, __int_as_float(idx), __int_as_float(0)));
+  }
+}
+
 // Merged statistics and accept bits of the rows of sequence b, one warp per
 // row over the NC slice partials.  Greedy: the draft is the argmax (lowest
 // index on ties); stochastic: u < p(d) / q(d) (Sec. III-C).
 __device__ __forceinline__ void decide_rows(const Call &p, RowsSmem &s, const RowTables &rows, int b, const SeqInfo &q,
                                             bool writer, int warp, int lane) {
-  constexpr int kLoads = kMaxNC / 32;
 #pragma unroll 1
   for (int i = warp; i <= q.k; i += kWarps) {
     const int n = q.r0 + i;
-    float4 part[kLoads];
-#pragma unroll
-    for (int j = 0; j < kLoads; ++j) {
-      const int cc = j * 32 + lane;
-      part[j] = cc < p.NC ? __ldcg(&p.pstat[static_cast<size_t>(n) * p.NC + cc])
-                          : make_float4(-INFINITY, 0.f, __int_as_float(INT_MAX), 0.f);
-    }
+    float4 part[kPartLoads];
+    load_parts(p, n, lane, part);
     int d = -1;
     float u = 0.f, qd = 0.f, ld = 0.f;
     if (i < q.k) {
@@ -654,26 +706,9 @@ __device__ __forceinline__ void decide_rows(const Call &p, RowsSmem &s, const Ro
         if (q.stoch && d >= 0 && d < p.V) qd = __ldg(&p.draft_probs[static_cast<size_t>(n - b) * p.V + d]);
       }
     }
-    // The maximum first, then its lowest index and the rescaled sum.
-    float m = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < kLoads; ++j) m = fmaxf(m, part[j].x);
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float z = 0.f;
-    int idx = INT_MAX;
-    if (m != -INFINITY) {
-#pragma unroll
-      for (int j = 0; j < kLoads; ++j) {
-        z += part[j].y * ex2((part[j].x - m) * kLog2e);
-        if (part[j].x == m) idx = min(idx, __float_as_int(part[j].z));
-      }
-    }
-#pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) {
-      z += __shfl_xor_sync(0xffffffffu, z, o);
-      idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, o));
-    }
+    float m, z;
+    int idx;
+    merge_parts(part, m, z, idx);
     if (lane == 0) {  // lane 0's values are everyone's
       int ok = 0;
       if (i < q.k) {
@@ -1283,6 +1318,7 @@ __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const Seq
     if (p.kc != nullptr) commit_seq(p, b, q.k, a, tid);
     block_sync();
   }
+  if (seqs.rest) rest_rows(p, seqs, c, nctas, warp, lane);
 }
 
 }  // namespace accept

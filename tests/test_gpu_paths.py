@@ -153,6 +153,32 @@ def test_draw_piece_again(dev, B, k, V):
         assert cmp["mismatch_unflagged"] == 0 and cmp["flagged"] < B // 2, cmp
 
 
+# Every row of a call leaves its statistics, also rows past the last sequence's (padding of a captured
+# call) and of a sequence that is reported: what an earlier call left there must not stay.
+@pytest.mark.parametrize("B,k,V", [(6, 4, 1000), (6, 4, 5000), (60, 4, 5000)])
+def test_statistics_of_every_row(dev, B, k, V):
+    wl = W.make_workload(_spec("rest", 370 + B, B=B, k=(k, k), V=V, mode="mixed", target_accept=0.7), device=dev)
+    R, H = wl["R"], wl["H"]
+    assert spade.spade_accept_launches(B, R, H, V) == (2 if B == 60 else 1)
+    ws = spade.accept_workspace(B, R, H, V, device=dev)
+    other = dict(wl, hidden=wl["hidden"].flip(0).contiguous())
+    parity.gpu_accept(other, workspace=ws)  # (leaves its own statistics)
+    cut, nd = wl["cu_q"].clone(), wl["n_draft"].clone()
+    cut[-1] -= 2  # the last sequence is two drafts shorter: two rows of padding
+    nd[-1] -= 2
+    nd[1] += 1    # reported: its rows and drafts do not agree
+    call = dict(wl, cu_q=cut, n_draft=nd)
+    acc, tok, st = parity.gpu_accept(call, workspace=ws)
+    torch.cuda.synchronize()
+    assert int(st.item()) & ~spade.DEV_FALLBACK == spade.DEV_BAD_INDEX
+    assert int(acc[1]) == 0 and int(tok[1]) == -1
+    logits = parity.oracle_logits(wl)
+    stats = spade.read_accept_stats(ws, B, R, H, V)
+    worst = parity.compare_row_stats(stats, logits, dict(wl, n_draft=torch.zeros_like(nd)))
+    assert worst["argmax_mismatch"] == 0 and max(worst["max"], worst["lse"]) <= 1.0, worst
+    assert stats["accept_bit"][(k + 1):2 * (k + 1)].tolist() == [0] * (k + 1) and stats["accept_bit"][-2:].tolist() == [0, 0]
+
+
 # Vocabularies of at most eight tiles run as one cluster, larger ones as a cooperative grid: one CTA, a
 # ragged last tile, the largest cluster and the smallest grid beyond it, with every option at once.
 @pytest.mark.parametrize("V", [100, 129, 1024, 1025])
