@@ -4,7 +4,8 @@ Each .cu under csrc/ is compiled to an object in parallel, then linked into
 ``paper_2608_13076_gb300/lib/libspade.so`` with the CUDA runtime linked
 statically; csrc/binding.cpp becomes ``lib/_spade_native.so``, an extension
 module over the installed torch.  A rebuild happens only when a source is newer
-than the outputs.
+than the outputs, or the torch or Python that the module was built for is not the
+one at hand.
 """
 from __future__ import annotations
 
@@ -22,6 +23,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB_DIR = os.path.join(HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "libspade.so")
 NATIVE_PATH = os.path.join(LIB_DIR, "_spade_native.so")
+STAMP_PATH = os.path.join(LIB_DIR, "_spade_native.stamp")  # what the extension module was built for
 BINDING = os.path.join(CSRC, "binding.cpp")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -44,9 +46,17 @@ def _deps():
         + [os.path.join(INCLUDE, "spade.h"), os.path.abspath(__file__)]
 
 
+def _built_for() -> str:
+    import torch
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
 def up_to_date() -> bool:
-    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH):
+    if not os.path.exists(LIB_PATH) or not os.path.exists(NATIVE_PATH) or not os.path.exists(STAMP_PATH):
         return False
+    with open(STAMP_PATH) as f:
+        if f.read() != _built_for():
+            return False
     t = min(os.path.getmtime(LIB_PATH), os.path.getmtime(NATIVE_PATH))
     return all(os.path.getmtime(d) <= t for d in _deps())
 
@@ -78,6 +88,8 @@ def _link_binding(obj):
     _run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, LIB_PATH, "-L", lib, "-lc10", "-lc10_cuda",
           "-ltorch_cpu", "-ltorch_python", f"-Wl,-rpath,$ORIGIN,-rpath,{lib}"], "link of the Python binding")
     os.replace(tmp, NATIVE_PATH)
+    with open(STAMP_PATH, "w") as f:
+        f.write(_built_for())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

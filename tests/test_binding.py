@@ -3,11 +3,18 @@ import pytest
 import torch
 
 import paper_2608_13076_gb300 as spade
+from paper_2608_13076_gb300 import _build
 
 
 @pytest.fixture(scope="module", autouse=True)
 def library():
     spade.build()
+
+
+def test_extension_is_rebuilt_for_another_torch(monkeypatch):
+    assert _build.up_to_date()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert not _build.up_to_date()
 
 
 def _args():
