@@ -23,13 +23,9 @@ __global__ void __launch_bounds__(kThreads, 1) accept_rows_kernel(const __grid_c
 }
 
 spade_status launch_accept_rows(const Call &c, int sms, cudaStream_t stream) {
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(accept_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(kRowsBytesDouble));
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(accept_rows)");
-    configured = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t es = set_max_smem(once, static_cast<int>(kRowsBytesDouble), accept_rows_kernel);
+  if (es != cudaSuccess) return cuda_fail(es, "cudaFuncSetAttribute(accept_rows)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(sms < kMaxNC ? sms : kMaxNC);
   cfg.blockDim = dim3(kThreads);

@@ -6,6 +6,7 @@
 #include <cstdint>
 
 #include "../../include/spade.h"
+#include "per_device.h"
 
 namespace spade {
 
@@ -16,6 +17,21 @@ spade_status cuda_fail(cudaError_t e, const char *what);
 
 // Checks that the current device is sm_103 and returns its SM count.
 spade_status device_info(int *num_sms, int *device);
+
+// Lets `kernels` have `bytes` of dynamic shared memory, once per device (the
+// attribute is the current device's).
+template <class... K>
+cudaError_t set_max_smem(OncePerDevice &once, int bytes, K... kernels) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return once(dev, [&] {
+    cudaError_t r = cudaSuccess;
+    for (cudaError_t x : {cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)...})
+      if (r == cudaSuccess) r = x;
+    return r;
+  });
+}
 
 // Encodes a bf16 tensor map of `rank` (2 .. 5) dimensions, innermost first, with
 // the outer dimensions' strides in bytes, 128-byte swizzle, zero fill out of

@@ -330,12 +330,9 @@ spade_status launch_lm_head_pairs(const Call &c, const void *hidden, const void 
   th1 = th0;
   if (p.n1w && !encode_tmap_bf16_sw128(&th1, hidden, H, c.R, pitch, kKChunk, p.n1w / 2)) return SPADE_ERR_CUDA;
 
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(lm_head_pairs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(lm_head_pairs)");
-    configured = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t es = set_max_smem(once, kSmemMax, lm_head_pairs_kernel);
+  if (es != cudaSuccess) return cuda_fail(es, "cudaFuncSetAttribute(lm_head_pairs)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c.NC);
   cfg.blockDim = dim3(kPairThreads);

@@ -446,14 +446,9 @@ spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int
       q += take;
     }
   }
-  static bool configured = false;
-  if (!configured) {
-    for (auto kern : {qkv_cluster_kernel<false>, qkv_cluster_kernel<true>}) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(qkv_cluster)");
-    }
-    configured = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t es = set_max_smem(once, kSmemBudget, qkv_cluster_kernel<false>, qkv_cluster_kernel<true>);
+  if (es != cudaSuccess) return cuda_fail(es, "cudaFuncSetAttribute(qkv_cluster)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.nclusters);
   cfg.blockDim = dim3(kThreads);

@@ -560,13 +560,10 @@ static spade_status qkv_rope_impl(const void *x, const void *w_qkv, const int32_
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   if (p.stages < 2) return fail(SPADE_ERR_SHAPE, "shared memory too small for R = %d", R);
   const int smem = layout(p.Ncols, p.stages, p.KG).total;
-  static bool configured = false;
-  if (!configured) {
-    // The plan above never exceeds kSmemBudget (alignment slack included).
-    cudaError_t e = cudaFuncSetAttribute(qkv_rope_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(qkv_rope)");
-    configured = true;
-  }
+  // The plan above never exceeds kSmemBudget (alignment slack included).
+  static OncePerDevice once;
+  const cudaError_t es = set_max_smem(once, kSmemBudget, qkv_rope_kernel);
+  if (es != cudaSuccess) return cuda_fail(es, "cudaFuncSetAttribute(qkv_rope)");
   CUtensorMap tw, tx0, tx1, tw3;
   const int n0 = p.Ncols > 256 ? 256 : p.Ncols;
   const int n1 = p.Ncols - n0;

@@ -24,7 +24,6 @@ spade_status cuda_fail(cudaError_t e, const char *what) {
 }
 
 namespace {
-constexpr int kMaxDevices = 64;
 struct DevInfo {
   int checked = 0;
   int ok = 0;

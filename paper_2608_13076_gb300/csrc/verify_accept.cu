@@ -499,12 +499,11 @@ static spade_status prepare(Params &p, const void *hidden, const void *w_lm, int
 constexpr int kMaxCluster = 8;
 
 // Whether the device takes such a cluster (asked once per device and size, with
-// the most shared memory that a call may need).
+// the most shared memory that a call may need; a failed question is asked again).
 static bool cluster_fits(cudaLaunchConfig_t cfg, int n) {
-  constexpr int kDevices = 64;
-  static std::atomic<signed char> known[kDevices][kMaxCluster + 1];  // 0: not asked, 1: yes, -1: no
+  static std::atomic<signed char> known[kMaxDevices][kMaxCluster + 1];  // 0: not asked, 1: yes, -1: no
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kDevices) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return false;
   signed char k = known[dev][n].load(std::memory_order_relaxed);
   if (k == 0) {
     cudaLaunchAttribute attr;
@@ -517,22 +516,20 @@ static bool cluster_fits(cudaLaunchConfig_t cfg, int n) {
     cfg.numAttrs = 1;
     int active = 0;
     const cudaError_t e = cudaOccupancyMaxActiveClusters(&active, verify_accept_kernel<true>, &cfg);
-    if (e != cudaSuccess) cudaGetLastError();
-    k = e == cudaSuccess && active > 0 ? 1 : -1;
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    k = active > 0 ? 1 : -1;
     known[dev][n].store(k, std::memory_order_relaxed);
   }
   return k > 0;
 }
 
 static spade_status launch(const Params &p, const Maps &m, cudaStream_t stream) {
-  static bool configured = false;
-  if (!configured) {
-    for (auto kern : {verify_accept_kernel<false>, verify_accept_kernel<true>}) {
-      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - 1024);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(verify_accept)");
-    }
-    configured = true;
-  }
+  static OncePerDevice once;
+  const cudaError_t es = set_max_smem(once, kSmemMax - 1024, verify_accept_kernel<false>, verify_accept_kernel<true>);
+  if (es != cudaSuccess) return cuda_fail(es, "cudaFuncSetAttribute(verify_accept)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.c.NC);
   cfg.blockDim = dim3(kThreads);

@@ -155,7 +155,6 @@ namespace spade {
 namespace attn_noalloc {
 
 constexpr size_t kScratchBytes = size_t(32) << 20;  // 32 MiB
-constexpr int kMaxDevices = 64;
 
 static __device__ __align__(256) uint8_t g_scratch[kScratchBytes];
 

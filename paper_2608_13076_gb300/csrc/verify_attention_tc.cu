@@ -749,12 +749,9 @@ template <int NR, int D>
 static cudaError_t launch_nr(const Params &p, const CUtensorMap &k2, const CUtensorMap &v2,
                              const CUtensorMap &k1, const CUtensorMap &v1, cudaStream_t stream) {
   auto kern = verify_attention_tc_kernel<NR, D>;
-  static bool configured = false;  // per template instance; the attribute is per function
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem::BYTES);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static OncePerDevice once;  // per template instance; the attribute is per function
+  const cudaError_t e = set_max_smem(once, Smem::BYTES, kern);
+  if (e != cudaSuccess) return e;
   // Programmatic dependent launch: the kernel's input-free set-up may overlap
   // the previous kernel in the stream (the kernel waits for it before reading
   // any input).
