@@ -107,7 +107,7 @@ typedef enum {
  *               share a workspace must be ordered.
  * Every pointer is a 16-byte aligned device pointer.  The contraction is split
  * over every SM and its parts' fp32 sums are added in a fixed order, so results
- * do not depend on timing.  Up to 128 rows, and up to 512 over wide layers, two
+ * do not depend on timing.  Up to 128 rows, and up to 464 over wide layers, two
  * CTAs of a cluster each take half of H and add their sums in shared memory:
  * the workspace is not touched.  Other calls add the parts in the workspace;
  * that kernel keeps every block of the grid resident at once (cooperative
@@ -308,10 +308,13 @@ size_t spade_accept_workspace_size(int32_t B, int32_t R, int32_t H, int32_t V);
 
 /*
  * Kernel launches one spade_verify_accept (or spade_verify_accept_commit) call
- * makes for these sizes on the current device: 1 (up to 256 rows, statistics
- * and decisions in one kernel) or 2 (a statistics pass over all rows on pairs
- * of SMs sharing each MMA, then the decisions and draws, from the logits that
- * the first stored); 0 on invalid sizes.  For launch accounting and graph
+ * makes for these sizes on the current device: 1 (statistics and decisions in
+ * one kernel: up to 256 rows, while the 128-entry tiles of an SM's vocabulary
+ * slice times the rows, rounded up to 8, stay within 512; on 152 SMs that is
+ * 256 rows up to 32000 entries, 128 at 64000, 72 at 128256 and 64 at 152064) or
+ * 2 (a statistics pass over all rows on pairs of SMs sharing each MMA, then the
+ * decisions and draws, from the logits that the first stored); 0 on invalid
+ * sizes.  For launch accounting and graph
  * capture; no device work.
  */
 int32_t spade_accept_launches(int32_t B, int32_t R, int32_t H, int32_t V);
@@ -327,8 +330,10 @@ int32_t spade_accept_launches(int32_t B, int32_t R, int32_t H, int32_t V);
  *     bits; 1 iff the row's draft passed its test);
  *   float at byte draft_logit_offset + 4 * r: logits[r, d] of the row's draft
  *     token d (rows i < k_b only; other entries are not written).
- * One copy is stored; `replica_stride` is its length in float4 (R).  Valid
- * until the next call that uses the workspace.  Returns SPADE_ERR_INVALID_ARG on null outputs or bad sizes.
+ * Rows of no valid sequence (past cu_q[B], or of a sequence that was reported)
+ * have theirs too, with accept bit 0.  One copy is stored; `replica_stride` is
+ * its length in float4 (R).  Valid until the next call that uses the workspace.
+ * Returns SPADE_ERR_INVALID_ARG on null outputs or bad sizes.
  */
 spade_status spade_accept_stats_layout(int32_t B, int32_t R, int32_t H, int32_t V,
                                        size_t *row_stats_offset, size_t *draft_logit_offset,

@@ -207,6 +207,7 @@ def spade_verify_attention_noalloc(q, k_cache, v_cache, ctx_lens, n_draft, cu_q,
 
     Calls that overlap on the GPU share that array and race; the first call on
     a device resolves the array's address and should precede any stream capture.
+    An ``lse`` that is given must be a contiguous float32 CUDA tensor.
     """
     rc = (_native or native()).attention_noalloc(
         q, k_cache, v_cache, ctx_lens, n_draft, cu_q, out, lse, max_k, status, stream)

@@ -1265,7 +1265,7 @@ __device__ __forceinline__ void draw_token(const Call &p, RowsSmem &s, int b, co
 // end): decisions, outputs, commit and the draws.  Sampled sequences are dealt
 // to groups of CTAs from the front of the grid, greedy ones to single CTAs
 // from its end; no group waits for another.  The CTAs of a group wait for one
-// another's words (every CTA is resident: cooperative launches).
+// another's words (every CTA is resident: cooperative launches, or one cluster).
 __device__ __forceinline__ void rows_phase(const Call &p, RowsSmem &s, const SeqTable &seqs, const RowTables &rows, int c,
                                            int nctas) {
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;

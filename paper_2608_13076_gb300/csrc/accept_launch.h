@@ -1,6 +1,5 @@
-// accept_launch.h -- host side of the two-launch LM head (more verify rows than
-// half of the tensor memory keeps in one round, or slices too long for it):
-// lm_head_pairs.cu and accept_rows.cu, called by verify_accept.cu.
+// accept_launch.h -- host side of the two-launch LM head (calls that one_launch() in
+// verify_accept.cu does not take): lm_head_pairs.cu and accept_rows.cu.
 #pragma once
 #include "accept_common.cuh"
 

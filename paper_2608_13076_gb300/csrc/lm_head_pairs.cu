@@ -1,5 +1,5 @@
-// lm_head_pairs.cu -- first launch of the two-launch LM head (calls whose rows
-// exceed the one-launch form's tensor memory): logits o = g(x_L) of every verify
+// lm_head_pairs.cu -- first launch of the two-launch LM head (calls that the
+// one-launch form does not take, see one_launch()): logits o = g(x_L) of every verify
 // row against the vocabulary (Sec. III-A), kept as per-slice softmax statistics,
 // and stored for the rows that a sampled sequence may draw from.
 //
@@ -66,10 +66,12 @@ __host__ __device__ inline PairSmem pair_layout(int Ncols, int stages) {
 
 // Vocabulary slice of CTA `rank` of pair j.  Pairs walk the k-chunks from different
 // starts, so that not all of them load the same hidden lines from L2 at once:
-// slice s from chunk 2 (s mod ns), as the one-launch form (stages of two chunks)
-// walks it, so a logit is summed in the same order, to the same bits, in either.  A
-// pair has one order: it takes slices s and s + ns, which share it; the last few
-// slices without such a partner pair up with their neighbours.
+// slice s from chunk 2 (s mod ns), as the one-launch form walks it with stages of two
+// chunks (up to 80 rows; with one-chunk stages, above, it starts at another chunk).
+// A pair has one order: it takes slices s and s + ns, which share it, so their logits
+// are summed in the one-launch form's order, to the same bits.  Slices without such a
+// partner pair up with their neighbours, and the second of the two takes the first's
+// order (4 of 152 slices at H = 5120, 12 at 4096 and 8192, 20 at 12288, 76 at 20480).
 __device__ __forceinline__ int pair_slice(int j, int rank, int nslices, int ns) {
   const int group = j / ns, i = j - group * ns, base = 2 * ns * group;
   const int both = max(0, min(nslices - base, 2 * ns) - ns);  // pairs (s, s + ns) of this group

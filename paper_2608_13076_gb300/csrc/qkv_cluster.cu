@@ -422,8 +422,9 @@ static Params plan(const Call &c, int sms) {
 }  // namespace pair
 
 // Up to 128 rows the cluster form streams W at the rate its ring allows and is
-// taken when at least four stages fit: 14.0 us at 72 rows against 20.5 us of the
-// stream-K form. Above, see plan().
+// taken when at least four stages fit: 13.3 us at 72 rows against 20.5 us of the
+// stream-K form. Above, see plan() (464 rows are the most whose ring fits, over ranges
+// of eight quads).
 bool cluster_fits(const Call &c, int sms) { return pair::plan(c, sms).stages > 0; }
 
 spade_status launch_cluster(const Call &c, const void *x, const void *w_qkv, int sms, cudaStream_t stream) {

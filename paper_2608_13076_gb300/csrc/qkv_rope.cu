@@ -80,7 +80,7 @@ __host__ __device__ inline Layout layout(int Ncols, int stages, int KG) {
   Layout L;
   L.stage_bytes = KG * (kWBytes + Ncols * 128);  // KG W chunks, then KG x chunks
   L.ring = 0;
-  L.rseq = stages * L.stage_bytes;   // int32 [kMaxR]: sequence of each row (-1: skip)
+  L.rseq = stages * L.stage_bytes;   // uint32 [kMaxR]: cache row of each verify row (kNoRow: skip)
   L.rpos = L.rseq + kMaxR * 4;       // int32 [kMaxR]: position of each row
   L.bars = L.rpos + kMaxR * 4;       // full[stages], empty[stages], acc_full[2], acc_empty[2], drain
   L.misc = (L.bars + (2 * kMaxStages + 5) * 8 + 15) & ~15;  // tmem base, abort flag, last-arrival flag

@@ -2,7 +2,7 @@
 // accept test alpha(x) = min(1, p(x)/q(x)) and the residual sampling from
 // p'(x) = norm(max(0, p(x) - q(x))) (Sec. III-C), i.e. the verify / accept /
 // correct steps of Algorithm 1 for every sequence of the batch.  This file holds
-// the one-launch form (up to 256 verify rows) and the entry points; larger
+// the one-launch form (see one_launch()) and the entry points; larger
 // calls take lm_head_pairs.cu and accept_rows.cu.
 //
 // Design (GB300):
@@ -382,9 +382,15 @@ static void slice_shape(int V, int NC, int *tiles_max, int *brs) {
   *brs = last == 0 ? kTileV : (last + 7) / 8 * 8;
 }
 
-// Whether the one-launch form takes the call (its limits bound top-p too, whose
-// search reads every row's logits): at most 256 rows, at most 32 tiles per SM,
-// and tiles x rows (rounded up to 8) within the 512 accumulator columns.
+// Whether the one-launch form takes the call: at most 256 rows (one MMA's N), at most
+// 32 tiles per SM, and tiles x rows (rounded up to 8) within 512 accumulator columns
+// (on 152 SMs 256 rows up to 32000 entries, 128 at 64000, 72 at 128256, 64 at 152064).
+// The kernel's rounds would run with more, but CTA pairs, which stream the hidden
+// rows half as often, are faster there (us, pairs / one launch, no row sampled and
+// all: 80 rows x 4096 x 128256 161 / 164 and 190 / 193, 128 rows 165 / 179 and 203 / 223,
+// 256 rows 199 / 230 and 254 / 296; 72 rows x 5120 x 152064 236 / 237 and 269 / 275; 136 rows x
+// 4096 x 64000 92 / 121 and 108 / 138).  Top-p needs this form: the search's bins are
+// laid out for it only.
 static bool one_launch(int R, int V, int sms) {
   if (R > kMaxRes) return false;
   const Plan pl = make_plan(R, V, sms);
