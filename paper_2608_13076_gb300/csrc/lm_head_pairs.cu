@@ -53,7 +53,7 @@ __host__ __device__ inline PairSmem pair_layout(int Ncols, int stages) {
   PairSmem s;
   s.stage = kWChunkBytes + Ncols / 2 * 128;  // W rows, then this CTA's half of each N-chunk
   s.off_bar = stages * s.stage;
-  s.off_misc = s.off_bar + (2 * kMaxStages + 6) * 8;
+  s.off_misc = s.off_bar + (2 * kMaxStages + 4) * 8;
   s.off_seq = (s.off_misc + 16 + 15) & ~15;
   s.off_rows = s.off_seq + static_cast<int>(sizeof(SeqTable));
   s.off_stat = s.off_rows + row_table_bytes(Ncols, false);
@@ -88,7 +88,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
   uint64_t *empty = full + kMaxStages;
   uint64_t *acc_full = empty + kMaxStages;  // [2]
   uint64_t *acc_empty = acc_full + 2;       // [2]
-  uint64_t *fin = acc_empty + 2;            // teardown handshake
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L.off_misc);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L.off_misc + 8);
   const RowTables rows = row_tables(smem + L.off_rows, p.Ncols, false);
@@ -109,7 +108,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
     *s_abort = 0;
     for (int s = 0; s < p.stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 2 * kPairWarps); }
-    mbar_init(fin, 1);
     if (rank == 0)  // arm every stage's first use with both CTAs' bytes
       for (int s = 0; s < p.stages; ++s) mbar_arrive_expect_tx(&full[s], 2 * stage_tx);
     fence_mbar_init();
@@ -166,8 +164,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
       }
     }
     // After an expired wait the even CTA drains the copies of both (its full
-    // barriers count them); the odd CTA's shared memory stays alive until the
-    // teardown handshake with the even CTA.
+    // barriers count them); the odd CTA's shared memory stays alive until both
+    // CTAs have reached the teardown.
     if (!ok && rank == 0 && leader) {
       const uint32_t n = p.stages;
       for (uint32_t j = (issued > n ? issued - n : 0); j < issued; ++j)
@@ -282,18 +280,16 @@ __global__ void __launch_bounds__(kPairThreads, 1) lm_head_pairs_kernel(
       // only after an expired wait: the statistics consumed the last tile).
       for (int t = max(0, tiles_issued - p.nacc); t < tiles_issued; ++t)
         mbar_wait_unabortable(&acc_full[p.nacc == 2 ? t & 1 : 0], (p.nacc == 2 ? t >> 1 : t) & 1);
-      // The allocation is released by both CTAs together, once both are done
-      // with it (bounded handshake on each other's `fin`).
-      mbar_arrive_cluster(cluster_map(fin, rank ^ 1u));
-      const uint64_t t0 = globaltimer();
-      while (!mbar_try_wait_cluster(fin, 0)) {
-        if (globaltimer() - t0 > kWaitLimitNs) {
-          atomicOr(p.c.status, SPADE_DEV_TIMEOUT);
-          break;
-        }
-      }
     }
     __syncwarp();
+  }
+  // Both CTAs are done with the allocation, with each other's shared memory and with
+  // each other's barriers.  (The cluster's barrier has no limit, and needs none: each
+  // wait before it has one, so both CTAs come.  After an expired wait one of them may
+  // come seconds after the other, which must not have left: its barriers are still
+  // arrived on.)
+  cluster_sync();
+  if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, kTmemCols);
   }
